@@ -130,7 +130,7 @@ class Clocks:
 # the sources the measured solve kernels (the persistent cycle kernel and the batch kernel)
 # are compiled from: the DRAM counters recorded under profiles/ hold while these are unchanged
 KERNEL_SOURCES = ("amg_internal.cuh", "batch.cu", "batch_graded.cu", "batch_kernel.cuh",
-                  "cycle_ops.cuh", "solve.cu")
+                  "cluster_tail.cuh", "cycle_ops.cuh", "solve.cu")
 
 
 def kernel_source_hash():

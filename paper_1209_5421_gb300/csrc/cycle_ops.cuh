@@ -1,9 +1,9 @@
 // Device building blocks of the AMLI-cycle (paper Alg. 1, Alg. 2, Sec. 4.3, Sec. 4.5): the
 // operation descriptors, level views, deterministic reductions, the bounded grid barrier
 // and every cycle operation as a row-parallel device function ("thread tid of nth").
-// The same functions run in three executors (solve.cu): one multi-CTA kernel per op, a
-// persistent cooperative kernel that runs a whole program of ops with grid barriers, and a
-// single-CTA interpreter over levels staged in shared memory.
+// The same functions run in the executors of solve.cu (one multi-CTA kernel per op, and a
+// persistent cooperative kernel that runs a program of ops with grid barriers) and in the
+// batch kernel (one CTA or a team of CTAs per system).
 #pragma once
 
 #include <stdint.h>
@@ -22,7 +22,7 @@ enum OpKind : int {
     OP_ORTH,          // p_i += sum_j beta_ij p_j, beta_ij = -sc[ZQ_j] / sc[PQ_j]
     OP_SPMV_DOT,      // q_i = A p_i, sc[PQ_i] = (p_i, q_i), sc[RP_i] = (r_i, p_i)
     OP_UPDATE,        // alpha_i; e (+)= alpha_i p_i; r = r_i - alpha_i q_i; sc[RR_i] = (r, r)
-    OP_TAIL,          // persistent program: CTA 0 runs the tail program in shared memory
+    OP_TAIL,          // cycle program: B~ of the levels held by the cluster (k_cluster_tail)
     OP_NOP,           // persistent program: only the prologue (finalise a reduction)
     OP_GS_FIRST,      // point GS from zero, first colour: u_i = f_i / a_ii on [i0, i1), 0 elsewhere
     OP_RESID,         // first pass of a split restriction: q_step = f - A u (row by row)
@@ -58,7 +58,7 @@ struct Op {
 
 enum : int { V_RHS = 0, V_E, V_R, V_P0 };  // V_P0 + i = p_i
 
-// view of one level; I = column index type (int in HBM, uint16 in the shared-memory tail);
+// view of one level; I = column index type;
 // B = 1 compiles the lane-parallel block smoother of finest levels with multi-row blocks
 // (a separate kernel instance, so that the code of the others stays as it is)
 template <class T, class I, int B = 0>
@@ -75,7 +75,6 @@ struct LevelDev {
     const I *col;
     const T *val;
     const T *dinv;                  // 1 / a_ii (smoother)
-    const unsigned short *col16;    // 16-bit copy of col (levels read by the tail from HBM)
     const int *bptr;
     const BigSched *big;            // finest level: the big blocks' sweep schedule, or NULL
     const int *parent;
@@ -84,33 +83,6 @@ struct LevelDev {
     const double *Ainv;             // coarsest: dense inverse, FP64 (FP64 cycle)
     const float *Ainv2;             // coarsest, FP32 cycle: the same inverse as n*n high parts
                                     // followed by n*n low parts (Ainv ~ high + low)
-    T *rhs, *e, *r;
-    T *p[kMaxKcycle], *q[kMaxKcycle];
-    double *sc;
-    int nnext;
-};
-
-// view of a level staged in shared memory with one slice width for the whole level: entry k
-// of row i at (i / 32) 32 w + 32 k + i % 32, w = W (compile-time) or the member w (W = 0).
-// No slice pointers to load, and with W fixed every row loop is unrolled without bounds.
-template <class T, int W>
-struct StagedLevel {
-    using val_t = T;
-    using idx_t = unsigned short;
-    static constexpr int fine = 0;  // point smoother (staged levels are coarse)
-    static constexpr int bg = 0;
-    static constexpr int coop = 0;
-    int n, w;
-    const unsigned short *col;
-    const T *val;
-    const T *dinv;
-    const int *bptr;                // unused (fine = 0)
-    static constexpr const BigSched *big = nullptr;
-    const int *parent;
-    const int4 *children;           // children of the NEXT coarser level's rows
-    const int4 *children2;          // octree: their children 4..7 (NULL on a quadtree)
-    const double *Ainv;
-    const float *Ainv2;
     T *rhs, *e, *r;
     T *p[kMaxKcycle], *q[kMaxKcycle];
     double *sc;
@@ -131,13 +103,6 @@ __device__ __forceinline__ void row_span(const LevelDev<T, I, B> &L, int i, int 
         width = (L.sl[s + 1] - a) >> 5;
     }
 }
-template <class T, int W>
-__device__ __forceinline__ void row_span(const StagedLevel<T, W> &L, int i, int &base,
-                                         int &width) {
-    width = W > 0 ? W : L.w;
-    base = (i >> 5) * 32 * width + (i & 31);
-}
-
 // Index checks of the bounds-checking build (compiled with -DAMG_BOUNDS_CHECK): an index of
 // a gather outside [0, n) sets this translation unit's flag (amg_debug_bounds_flags reads it)
 // and the access is skipped, so a bad index is reported instead of read. The normal build
@@ -165,7 +130,6 @@ static inline int bounds_flag_read_clear() { return -1; }
 #endif
 
 __device__ __forceinline__ bool col_ok(int c) { return c >= 0; }
-__device__ __forceinline__ bool col_ok(unsigned short c) { return c != (unsigned short)0xFFFF; }
 
 // a[i] for a run-time i, as a chain of selects: a view built in registers keeps its pointer
 // arrays in registers (an indexed access would move them to the stack)
@@ -188,13 +152,6 @@ __device__ __forceinline__ typename LV::val_t *vec_of(const LV &L, int sel) {
 struct BlockGroup {  // every thread of the CTA; barrier 0
     __device__ __forceinline__ void sync() const { __syncthreads(); }
     __device__ __forceinline__ int nwarps() const { return (blockDim.x + 31) >> 5; }
-};
-struct WarpGroup {  // warps [0, nthreads / 32) of the CTA; hardware barrier 1
-    int nthreads;   // multiple of 32
-    __device__ __forceinline__ void sync() const {
-        asm volatile("bar.sync 1, %0;" ::"r"(nthreads) : "memory");
-    }
-    __device__ __forceinline__ int nwarps() const { return nthreads >> 5; }
 };
 
 // ---------------------------------------------------------------------------------------
@@ -622,14 +579,12 @@ __device__ __forceinline__ void gs_row_at(const LV &L, int i, int base, int widt
     u[i] = (f[i] - row_dot(L, base, 1, width, u)) * L.dinv[i];
 }
 
-// Shared memory a grid-wide executor lends to the big blocks' sweeps: p (null on CTAs
-// without it) and its size. With skip0, CTA 0 (whose shared memory holds the tail) takes no
-// big block; the warp-sized blocks go to warps [0, wwarps) of the other CTAs, each with a
-// slice of wslice bytes at p + warp * wslice (wwarps = 0: to every warp, from global memory).
+// Shared memory a grid-wide executor lends to the big blocks' sweeps: p (null: none) and its
+// size; the warp-sized blocks go to warps [0, wwarps) of every CTA, each with a slice of
+// wslice bytes at p + warp * wslice (wwarps = 0: to every warp, from global memory).
 struct BigScratch {
     unsigned char *p = nullptr;
     unsigned bytes = 0;
-    bool skip0 = false;
     int wwarps = 0;
     unsigned wslice = 0;
 };
@@ -760,10 +715,7 @@ __device__ void op_gs_big_blocks(const LV &L, const Op &op, const typename LV::v
     const int *lofs = bwd ? S->lofs_b : S->lofs_f;
     const int *lp = bwd ? S->lp_b : S->lp_f;
     const int4 *ent = bwd ? S->ent_b : S->ent_f;
-    if (sc.skip0) {  // CTA 0 lends no shared memory: the other CTAs take every big block
-        if (blockIdx.x == 0) return;
-        crank -= 1;
-        ccount -= 1;
+    if (sc.p) {
         const int w = (int)threadIdx.x >> 5;
         if (sc.wwarps > 0 && w < sc.wwarps) {  // warps with a slice: warp-sized blocks
             unsigned char *slice = sc.p + (size_t)w * sc.wslice;

@@ -6,25 +6,23 @@
 // Execution. One application of the preconditioner B^_fine is a fixed program of ops (see
 // cycle_ops.cuh) over device-resident data; every scalar stays on the device. It runs as ONE
 // persistent cooperative kernel (one CTA per SM): the CTAs execute each op row-parallel and
-// meet at a bounded grid barrier before the next. The coarse levels from the "tail" level
-// down (a few thousand rows or less: pure latency) are staged in shared memory by CTA 0 at
-// kernel start, and CTA 0 alone runs their whole recursive Alg. 1 / Alg. 2 there with
-// __syncthreads() between ops while the other CTAs wait at the barrier. The outer Krylov
-// update is four small kernels per iteration; the host reads one residual per iteration.
+// meet at a bounded grid barrier before the next. The coarse levels (pure latency) run in the
+// shared memory of a thread-block cluster (cluster_tail.cuh), a launch of its own between
+// launches of the persistent kernel. The outer Krylov update is four small kernels per
+// iteration; the host reads one residual per iteration.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
 #include <cstring>
 #include <type_traits>
 
+#include "cluster_tail.cuh"
 #include "cycle_ops.cuh"
 
 namespace amg {
 
 template <class T>
 using GLev = LevelDev<T, int>;                 // level in HBM
-template <class T>
-using SLev = LevelDev<T, unsigned short>;      // level staged in shared memory
 
 // persistent kernel CTA size (one CTA per SM): the FP64 cycle runs with fewer threads and
 // twice the registers each, as its ops at the 64-register cap of 1024 threads spill
@@ -32,33 +30,11 @@ constexpr int kPThreads = 1024;
 constexpr int kPThreads64 = 512;
 template <class T>
 constexpr int cycle_threads() { return sizeof(T) == 8 ? kPThreads64 : kPThreads; }
-constexpr int kTailRowsMax = 4096;  // levels larger than this are never staged
 // coarse levels of at least this many rows restrict in two grid-wide passes (OP_RESID,
 // OP_GATHER): their rows' children lie in different colours, far apart in HBM, and the
 // one-pass form's four-lane gathers read scattered slots
 constexpr int kSplitRestrictRows = 524288;
 
-
-// shared-memory image of the tail levels (byte offsets into the dynamic shared memory)
-struct TailLevelLayout {
-    int n, nslices, padded;
-    int gmem;    // 1: the level stays in HBM/L2 (top tail level only); its scalars are staged
-    int w;       // staged: slice width of the image (every slice padded to it)
-    int colors, ncolors;  // staged int[ncolors + 1]: pi-row range of each colour
-    int col, val, dinv, parent, children, children2, Ainv, rhs, e, r;
-    int p[kMaxKcycle], q[kMaxKcycle];
-};
-struct TailLayout {
-    int tl;      // first tail level (nlev = none)
-    int nlev;
-    int narrow;  // threads (whole warps) that run the ops of the staged levels
-    int kc;      // Alg. 1 steps (kcycle_n)
-    int nu_pre, nu_post;  // smoothing sweeps
-    int W;       // slice width of every staged level when fixed (9), else 0
-    int bytes;
-    int sc;      // the tail levels' Alg. 1 scalars, SC_N doubles per level
-    TailLevelLayout lv[kMaxLevels];
-};
 
 constexpr int kTprofCount = 16 * kMaxLevels;  // tail profile slots: 16 op kinds per level
 
@@ -66,23 +42,20 @@ template <class T>
 struct CycleArgs {
     const GLev<T> *tab;
     const Op *prog;
-    int nops;
-    const int *tail_colors;      // colour ranges of the tail levels, copied to shared memory
-    int tail_color_words;
-    TailLayout lay;
+    int nlev;
+    int k0, k1;                  // this launch's ops
+    unsigned long long bar_base; // arrivals at the barrier counter before this launch
     double *partials;            // [2][4][gridDim]
-    unsigned long long *bar;     // barrier counter (zeroed before every launch)
+    unsigned long long *bar;     // barrier counter (zeroed before every application)
     int *err;
     unsigned long long *ts;      // per-op end timestamps (profiling) or null
-    unsigned long long *tprof;   // tail: [16 level + kind] cycles, [kTprofCount + 16 level +
-                                 // kind] count (profiling) or null
     // host-set barrier fault (amg_debug_barrier_fault): wait limit of every grid barrier, and
     // arrivals the first barrier waits for beyond the grid's (0: none)
     unsigned long long bar_limit_ns;
     int bar_extra;
     // the finest level's input and output vectors when not the table's (FGMRES basis vectors)
     T *rhs0, *e0;
-    // CTAs 1.. lend their dynamic shared memory to the big blocks' sweeps; the warp-sized
+    // the CTAs lend their dynamic shared memory to the big blocks' sweeps; the warp-sized
     // ones go to warps [0, big_wwarps) with big_wslice bytes each (0: to every warp, from
     // global memory)
     int big_smem, big_wwarps;
@@ -99,408 +72,7 @@ __global__ void __launch_bounds__(kRedThreads) k_op(const GLev<T> *__restrict__ 
 }
 
 // ---------------------------------------------------------------------------------------
-// persistent cycle kernel: the shared-memory tail
-//
-// CTA 0 runs B~ of the tail levels (Alg. 1 with Alg. 2 inside, down to the exact coarsest
-// solve) as structured code: one device function per level depth, every op a direct call,
-// no op decoding. Staged levels are addressed from the dynamic shared-memory base through
-// the byte offsets of the layout (kept in shared memory), so every access is a shared-memory
-// load, and their slices have one width W (compile-time 9 for the 3x3-cell stencils of
-// span-1 levels). Their ops run on the first `narrow` threads (whole warps) with hardware
-// barrier 1: the other warps would only add issue slots and barrier arrivals to ops of a
-// few hundred rows. The ops of an HBM-resident top level (thousands of rows, each a chain
-// of L2 round trips) run on the whole CTA with CTA-wide barriers.
-extern __shared__ __align__(16) unsigned char amg_smem[];
-
-struct TailCtl {
-    int tl, nlev, narrow, kc, sc_off;
-    int nu_pre, nu_post;
-    int top_w;  // slice width of the HBM-resident top level when uniform, else 0
-    int *err;
-    unsigned long long *tprof;
-    long long t0;
-};
-__shared__ TailCtl tail_ctl;
-__shared__ TailLevelLayout tail_lay[kMaxLevels];
-__shared__ __align__(16) unsigned char tail_gview[sizeof(SLev<double>)];  // SLev<T> of the top
-// The same top level as a StagedLevel<T, W> whose arrays are in HBM (uniform slice width):
-// its phases then run the code the staged levels run, so the tail executes one copy of the
-// phase code instead of two (the tail's time goes largely to instruction fetch)
-__shared__ __align__(16) unsigned char tail_sview[sizeof(StagedLevel<double, 0>)];
-
-template <class T, int W>
-__device__ __forceinline__ StagedLevel<T, W> staged_level(int l) {
-    const TailLevelLayout &y = tail_lay[l];
-    const int nlev = tail_ctl.nlev;
-    auto at = [](int off) { return amg_smem + (off > 0 ? off : 0); };  // -1: absent, never read
-    StagedLevel<T, W> V;
-    V.n = y.n;
-    V.w = y.w;
-    V.col = (const unsigned short *)at(y.col);
-    V.val = (const T *)at(y.val);
-    V.dinv = (const T *)at(y.dinv);
-    V.bptr = nullptr;
-    V.parent = (const int *)at(y.parent);
-    V.children = (const int4 *)at(l + 1 < nlev ? tail_lay[l + 1].children : -1);
-    V.children2 = (l + 1 < nlev && tail_lay[l + 1].children2 >= 0)
-                      ? (const int4 *)(amg_smem + tail_lay[l + 1].children2) : nullptr;
-    V.Ainv = (const double *)at(y.Ainv);  // FP64 cycle: n*n doubles
-    V.Ainv2 = (const float *)at(y.Ainv);  // FP32 cycle: 2*n*n floats, the same bytes
-    V.rhs = (T *)at(y.rhs);
-    V.e = (T *)at(y.e);
-    V.r = (T *)at(y.r);
-#pragma unroll
-    for (int k = 0; k < kMaxKcycle; k++) {
-        V.p[k] = (T *)at(y.p[k]);
-        V.q[k] = (T *)at(y.q[k]);
-    }
-    V.sc = (double *)(amg_smem + tail_ctl.sc_off) + (size_t)(l - tail_ctl.tl) * SC_N;
-    V.nnext = l + 1 < nlev ? tail_lay[l + 1].n : 0;
-    return V;
-}
-
-// tail profiling: SM cycles of the op just finished, by level and kind (thread 0)
-__device__ __forceinline__ void tail_mark(int l, int kind) {
-    if (tail_ctl.tprof && threadIdx.x == 0) {
-        const long long t1 = clock64();
-        const int slot = 16 * l + kind;
-        atomicAdd(&tail_ctl.tprof[slot], (unsigned long long)(t1 - tail_ctl.t0));
-        atomicAdd(&tail_ctl.tprof[kTprofCount + slot], 1ull);
-        tail_ctl.t0 = t1;
-    }
-}
-
-__device__ __forceinline__ Op tail_op() {
-    Op o;
-    memset(&o, 0, sizeof o);
-    o.red_pb = -1;
-    o.fin_pb = -1;
-    return o;
-}
-
-// The recursion of B~ (Alg. 1) and B^ (Alg. 2) over the tail levels is walked as a state
-// machine with three phases per level: ENTER (B~_l starts: the exact solve on the coarsest
-// level, else step 0), PRE (B^_l for step i up to the restriction, then B~_{l+1}) and POST
-// (the prolongation, post-smoothing and the Alg. 1 updates of step i). Every thread of the
-// CTA walks it with the same state, so all know which phases are the top level's.
-enum : int { PH_ENTER = 0, PH_PRE, PH_POST };
-
-// pre-smoothing from zero (colours ascending; the first non-empty colour is u = D^-1 f) and
-// next.rhs = P^t (f - A u1), for z = p_i = B^_l [f], f = rhs (i = 0) or r
-// first non-empty colour [r0, r1) of tail level l (its point-GS first colour)
-__device__ __forceinline__ void tail_first_colour(int l, int &r0, int &r1) {
-    const int *cr = (const int *)(amg_smem + tail_lay[l].colors);
-    const int nc = tail_lay[l].ncolors;
-    int c = 0;
-    while (c < nc && cr[c + 1] == cr[c]) c++;
-    r0 = c < nc ? cr[c] : 0;
-    r1 = c < nc ? cr[c + 1] : 0;
-}
-
-// The first colour of a pre-smoothing was already done by the op before it, except for step
-// 0 of the top tail level: by the last UPDATE (i > 0) or by the restriction into this level
-// (i = 0), which also starts the next level's first colour unless that level is the coarsest.
-template <class T, int W, class LV, class G>
-__device__ __forceinline__ void phase_pre(const LV &L, const G &g, int nth, int l, int i) {
-    const int tid = threadIdx.x;
-    const T *f = i == 0 ? L.rhs : L.r;
-    T *z = pick(L.p, i);
-    const int *cr = (const int *)(amg_smem + tail_lay[l].colors);
-    const int nc = tail_lay[l].ncolors;
-    int c = 0;
-    while (c < nc && cr[c + 1] == cr[c]) c++;
-    Op op = tail_op();
-    if (i == 0 && l == tail_ctl.tl) {
-        op.i0 = c < nc ? cr[c] : 0;
-        op.i1 = c < nc ? cr[c + 1] : 0;
-        op_gs_first(L, op, f, z, tid, nth);
-        g.sync();
-        tail_mark(l, OP_GS_FIRST);
-    }
-    // the first sweep's remaining colours, then nu_pre - 1 further forward sweeps
-    for (int sw = 0, c1 = c + 1; sw < tail_ctl.nu_pre; sw++, c1 = 0)
-        for (c = c1; c < nc; c++) {
-            if (cr[c + 1] == cr[c]) continue;
-            op.i0 = cr[c];
-            op.i1 = cr[c + 1];
-            op_gs(L, op, f, z, tid, nth);
-            g.sync();
-            tail_mark(l, OP_GS);
-        }
-    // next.rhs = P^t (f - A u1) in two passes: the residual row by row into q_i (free until
-    // step i's SpMV writes it), then the children sums
-    T *t = pick(L.q, i);
-    op_resid(L, f, z, t, tid, nth);
-    g.sync();
-    tail_mark(l, OP_RESID);
-    const StagedLevel<T, W> N = staged_level<T, W>(l + 1);
-    if (tail_lay[l + 1].Ainv < 0) {  // the next level smooths: its first colour too
-        int f0, f1;
-        tail_first_colour(l + 1, f0, f1);
-        op_gather_children(L, t, N.rhs, tid, nth, N.p[0], N.dinv, f0, f1);
-    } else {
-        op_gather_children(L, t, N.rhs, tid, nth);
-    }
-    g.sync();
-    tail_mark(l, OP_RESTRICT);
-}
-
-// u2 = u1 + P next.e, post-smoothing (colours descending), then Alg. 1 step i on level l
-template <class T, int W, class LV, class G>
-__device__ __forceinline__ void phase_post(const LV &L, const G &g, int nth, int l, int i) {
-    const int tid = threadIdx.x;
-    const T *f = i == 0 ? L.rhs : L.r;
-    T *z = pick(L.p, i);
-    op_prolong(L, staged_level<T, W>(l + 1).e, z, tid, nth);
-    g.sync();
-    tail_mark(l, OP_PROLONG);
-    const int *cr = (const int *)(amg_smem + tail_lay[l].colors);
-    Op op = tail_op();
-    op.backward = 1;
-    for (int sw = 0; sw < tail_ctl.nu_post; sw++)
-        for (int c = tail_lay[l].ncolors - 1; c >= 0; c--) {
-            if (cr[c + 1] == cr[c]) continue;
-            op.i0 = cr[c];
-            op.i1 = cr[c + 1];
-            op_gs(L, op, f, z, tid, nth);
-            g.sync();
-            tail_mark(l, OP_GS);
-        }
-    const RedCtx rc{nullptr, nullptr};
-    const int kc = tail_ctl.kc;
-    op = tail_op();
-    op.step = i;
-    op.last = (i == kc - 1);
-    if (!op.last) {  // the UPDATE also starts step i+1's pre-smoothing
-        op.fuse = 1;
-        tail_first_colour(l, op.f0, op.f1);
-    }
-    if (i > 0) {
-        op_multidot<LV, RM_BLOCK>(L, op, rc, tid, nth, g);
-        g.sync();
-        tail_mark(l, OP_MULTIDOT);
-        op_orth(L, op, tid, nth, g);
-        g.sync();
-        tail_mark(l, OP_ORTH);
-    }
-    op_spmv_dot<LV, RM_BLOCK>(L, op, rc, tid, nth, g);
-    g.sync();
-    tail_mark(l, OP_SPMV_DOT);
-    op_update<LV, RM_BLOCK>(L, op, rc, tid, nth, g);
-    g.sync();
-    tail_mark(l, OP_UPDATE);
-}
-
-// ENTER on the coarsest level: e = A^{-1} rhs
-template <class LV, class G>
-__device__ __forceinline__ void phase_coarse(const LV &L, const G &g, int nth, int l) {
-    op_coarse(L, threadIdx.x, nth);
-    g.sync();
-    tail_mark(l, OP_COARSE);
-}
-
-// e_tl = B~_tl [rhs_tl] over the whole tail (every thread of CTA 0 calls it)
-template <class T, int W>
-__device__ void tail_btilde(bool inplace) {
-    const int tl = tail_ctl.tl, nlev = tail_ctl.nlev, kc = tail_ctl.kc, narrow = tail_ctl.narrow;
-    const int tid = threadIdx.x;
-    const SLev<T> &top_gv = *reinterpret_cast<const SLev<T> *>(tail_gview);
-    const StagedLevel<T, W> &topv = *reinterpret_cast<const StagedLevel<T, W> *>(tail_sview);
-    const bool top_staged_code = tail_ctl.top_w > 0 && (W == 0 || tail_ctl.top_w == W);
-    int step[kMaxLevels] = {};
-    int l = tl, ph = PH_ENTER;
-    bool prev_top = true;  // the caller's barrier
-    for (;;) {
-        const bool coarsest = tail_lay[l].Ainv >= 0;
-        const int i = step[l];
-        if (inplace && l == tl) {  // the HBM-resident top level: the whole CTA
-            if (!prev_top) __syncthreads();  // the narrow warps' phases are complete
-            prev_top = true;
-            const int nth = blockDim.x;
-            if (top_staged_code) {  // every thread: barrier 1 over the whole CTA
-                const WarpGroup all{nth};
-                if (ph == PH_PRE) phase_pre<T, W>(topv, all, nth, l, i);
-                else if (ph == PH_POST) phase_post<T, W>(topv, all, nth, l, i);
-            } else {
-                if (ph == PH_PRE) phase_pre<T, W>(top_gv, BlockGroup{}, nth, l, i);
-                else if (ph == PH_POST) phase_post<T, W>(top_gv, BlockGroup{}, nth, l, i);
-            }
-        } else {
-            prev_top = false;
-            if (tid < narrow) {
-                const WarpGroup ng{narrow};
-                const StagedLevel<T, W> L = staged_level<T, W>(l);
-                if (ph == PH_ENTER && coarsest) phase_coarse(L, ng, narrow, l);
-                else if (ph == PH_PRE) phase_pre<T, W>(L, ng, narrow, l, i);
-                else if (ph == PH_POST) phase_post<T, W>(L, ng, narrow, l, i);
-            }
-        }
-        // next state (the same in every thread)
-        if (ph == PH_ENTER && !coarsest) {
-            step[l] = 0;
-            ph = PH_PRE;
-            continue;
-        }
-        if (ph == PH_PRE) {  // descend: B~_{l+1}
-            if (l + 1 >= nlev || l + 1 - tl >= kMaxLevels) break;  // never: the coarsest ends it
-            l++;
-            ph = PH_ENTER;
-            continue;
-        }
-        if (ph == PH_POST && i + 1 < kc) {
-            step[l] = i + 1;
-            ph = PH_PRE;
-            continue;
-        }
-        // B~_l done (coarsest solved, or its last step): back to level l-1's POST
-        if (l == tl) break;
-        l--;
-        ph = PH_POST;
-    }
-    if (inplace && !prev_top) __syncthreads();
-}
-
-// CTA 0, kernel start: copy the staged levels into shared memory (slices padded to width w)
-template <class T>
-__device__ void stage_tail(const CycleArgs<T> &a) {
-    const TailLayout &Y = a.lay;
-    const int tid = threadIdx.x, nth = blockDim.x;
-    {
-        const int words = Y.nlev * (int)(sizeof(TailLevelLayout) / sizeof(int));
-        for (int i = tid; i < words; i += nth) ((int *)tail_lay)[i] = ((const int *)Y.lv)[i];
-    }
-    if (tid == 0) {
-        tail_ctl.tl = Y.tl;
-        tail_ctl.nlev = Y.nlev;
-        tail_ctl.narrow = Y.narrow;
-        tail_ctl.kc = Y.kc;
-        tail_ctl.nu_pre = Y.nu_pre;
-        tail_ctl.nu_post = Y.nu_post;
-        tail_ctl.sc_off = Y.sc;
-        tail_ctl.top_w = 0;
-        tail_ctl.err = a.err;
-        tail_ctl.tprof = a.tprof;
-    }
-    for (int l = Y.tl; l < Y.nlev; l++) {
-        const TailLevelLayout &y = Y.lv[l];
-        const GLev<T> &G = a.tab[l];
-        if (y.gmem) {  // read in place from HBM / L2
-            if (tid == 0) {
-                SLev<T> &S = *reinterpret_cast<SLev<T> *>(tail_gview);
-                S.n = G.n;
-                S.fine = 0;
-                S.bg = 0;
-                S.w = G.w;
-                S.sl = G.sl;
-                S.col = G.col16;
-                S.val = G.val;
-                S.dinv = G.dinv;
-                S.col16 = nullptr;
-                S.bptr = nullptr;
-                S.parent = G.parent;
-                S.children = (l + 1 < Y.nlev && Y.lv[l + 1].children >= 0)
-                                 ? (const int4 *)(amg_smem + Y.lv[l + 1].children) : nullptr;
-                S.children2 = (l + 1 < Y.nlev && Y.lv[l + 1].children2 >= 0)
-                                  ? (const int4 *)(amg_smem + Y.lv[l + 1].children2) : nullptr;
-                S.Ainv = G.Ainv;
-                S.Ainv2 = G.Ainv2;
-                S.rhs = G.rhs;
-                S.e = G.e;
-                S.r = G.r;
-                for (int k = 0; k < kMaxKcycle; k++) {
-                    S.p[k] = G.p[k];
-                    S.q[k] = G.q[k];
-                }
-                S.sc = (double *)(amg_smem + Y.sc) + (size_t)(l - Y.tl) * SC_N;
-                S.nnext = G.nnext;
-                StagedLevel<T, 0> &V = *reinterpret_cast<StagedLevel<T, 0> *>(tail_sview);
-                V.n = G.n;
-                V.w = G.w;
-                V.col = G.col16;
-                V.val = G.val;
-                V.dinv = G.dinv;
-                V.bptr = nullptr;
-                V.parent = G.parent;
-                V.children = S.children;
-                V.children2 = S.children2;
-                V.Ainv = nullptr;
-                V.Ainv2 = nullptr;
-                V.rhs = G.rhs;
-                V.e = G.e;
-                V.r = G.r;
-                for (int k = 0; k < kMaxKcycle; k++) {
-                    V.p[k] = G.p[k];
-                    V.q[k] = G.q[k];
-                }
-                V.sc = S.sc;
-                V.nnext = G.nnext;
-                tail_ctl.top_w = G.w;  // 0 unless every slice has one width
-            }
-            continue;
-        }
-        // slot (s, k, lane) of the image <- slot k of slice s in HBM, or padding
-        unsigned short *col = (unsigned short *)(amg_smem + y.col);
-        T *val = (T *)(amg_smem + y.val);
-        const int img = y.nslices * 32 * y.w;
-        for (int i = tid; i < img; i += nth) {
-            const int sidx = i / (32 * y.w), rem = i - sidx * 32 * y.w;
-            const int k = rem >> 5, lane = rem & 31;
-            const int s0 = G.sl[sidx], width = (G.sl[sidx + 1] - s0) >> 5;
-            int c = -1;
-            T v = 0;
-            if (k < width) {
-                c = G.col[s0 + 32 * k + lane];
-                v = G.val[s0 + 32 * k + lane];
-            }
-            col[i] = c >= 0 ? (unsigned short)c : (unsigned short)0xFFFF;
-            val[i] = c >= 0 ? v : T(0);
-        }
-        if (y.dinv >= 0)
-            for (int i = tid; i < y.n; i += nth) ((T *)(amg_smem + y.dinv))[i] = G.dinv[i];
-        if (y.parent >= 0)
-            for (int i = tid; i < y.n; i += nth) ((int *)(amg_smem + y.parent))[i] = G.parent[i];
-        if (y.children >= 0)  // children of this level's rows (in level l-1)
-            for (int i = tid; i < y.n; i += nth)
-                ((int4 *)(amg_smem + y.children))[i] = a.tab[l - 1].children[i];
-        if (y.children2 >= 0)  // octree: children 4..7
-            for (int i = tid; i < y.n; i += nth)
-                ((int4 *)(amg_smem + y.children2))[i] = a.tab[l - 1].children2[i];
-        if (y.Ainv >= 0) {  // n*n doubles or 2*n*n floats
-            if (sizeof(T) == 8)
-                for (int i = tid; i < y.n * y.n; i += nth)
-                    ((double *)(amg_smem + y.Ainv))[i] = G.Ainv[i];
-            else
-                for (int i = tid; i < 2 * y.n * y.n; i += nth)
-                    ((float *)(amg_smem + y.Ainv))[i] = G.Ainv2[i];
-        }
-    }
-    // colour ranges: every level's int[ncolors + 1] at its offset, in one block of words
-    if (a.tail_color_words > 0) {
-        int *dst = (int *)(amg_smem + Y.lv[Y.tl].colors);
-        for (int i = tid; i < a.tail_color_words; i += nth) dst[i] = a.tail_colors[i];
-    }
-}
-
-template <class T, int W>
-__device__ void run_tail(const CycleArgs<T> &a) {
-    const int tl = a.lay.tl, n = tail_lay[tl].n;
-    const int tid = threadIdx.x, nth = blockDim.x;
-    const bool inplace = tail_lay[tl].gmem != 0;
-    if (!inplace) {
-        const T *grhs = a.tab[tl].rhs;
-        T *srhs = (T *)(amg_smem + tail_lay[tl].rhs);
-        for (int i = tid; i < n; i += nth) srhs[i] = grhs[i];
-    }
-    if (tid == 0) tail_ctl.t0 = clock64();
-    __syncthreads();
-    tail_btilde<T, W>(inplace);
-    if (inplace) return;
-    __syncthreads();
-    T *ge = a.tab[tl].e;
-    const T *se = (const T *)(amg_smem + tail_lay[tl].e);
-    for (int i = tid; i < n; i += nth) ge[i] = se[i];
-}
-
+// persistent cycle kernel
 // sum the per-CTA partials of the previous op (every CTA, identical order) into sc; one
 // warp does it, in FP64 for the FP64 cycle and in FP32 for the FP32 cycle (whose per-CTA
 // partials are FP32 sums)
@@ -529,35 +101,39 @@ __device__ __forceinline__ void finalize(const CycleArgs<T> &a, const TAB *tab, 
     __syncthreads();
 }
 
-// B = 1: finest-level blocks of several rows take the lane-parallel block smoother
-template <class T, int W, int B>
+// ops [k0, k1) of an application's program. B = 1: finest-level blocks of several rows take
+// the lane-parallel block smoother
+extern __shared__ __align__(16) unsigned char amg_smem[];
+
+template <class T, int B>
 __global__ void __launch_bounds__(cycle_threads<T>(), 1) k_cycle(CycleArgs<T> a) {
     using GL = LevelDev<T, int, B>;  // the same layout as GLev<T>
     __shared__ GL gtab[kMaxLevels];
     __shared__ unsigned long long target;
     __shared__ int abort_flag;
     if (threadIdx.x == 0) {
-        target = (unsigned long long)a.bar_extra;  // > 0 only under a host-set barrier fault
-        abort_flag = 0;
+        // bar_extra > 0 only under a host-set barrier fault
+        target = a.bar_base + (unsigned long long)a.bar_extra;
+        abort_flag = ld_volatile_int(a.err) & kErrTimeout;  // of an earlier launch
     }
     {  // the level table, read by every op, lives in shared memory
-        const int words = a.lay.nlev * (int)(sizeof(GL) / sizeof(int));
+        const int words = a.nlev * (int)(sizeof(GL) / sizeof(int));
         for (int i = threadIdx.x; i < words; i += blockDim.x)
             ((int *)gtab)[i] = ((const int *)a.tab)[i];
     }
     __syncthreads();
+    if (abort_flag) return;
     if (threadIdx.x == 0) {
         if (a.rhs0) gtab[0].rhs = a.rhs0;
         if (a.e0) gtab[0].e = a.e0;
     }
-    if (blockIdx.x == 0 && a.lay.tl < a.lay.nlev) stage_tail(a);
-    __syncthreads();
     // the op descriptors pass through shared memory: a few threads fetch the next one while
     // the CTA waits at the barrier, and every thread reads its fields from there (a per-thread
     // copy would cost every thread a 72-byte global load and a local-memory round trip)
     __shared__ Op sop[2];
     constexpr int kOpWords = (int)(sizeof(Op) / sizeof(int));
-    if (threadIdx.x < kOpWords) ((int *)&sop[0])[threadIdx.x] = ((const int *)a.prog)[threadIdx.x];
+    if (threadIdx.x < kOpWords)
+        ((int *)&sop[a.k0 & 1])[threadIdx.x] = ((const int *)(a.prog + a.k0))[threadIdx.x];
     __syncthreads();
     // rows go to warps in 32-row chunks with the CTA index fastest, so an op over a few
     // thousand rows (the coarse grid-wide levels) spreads over every SM instead of filling the
@@ -567,28 +143,25 @@ __global__ void __launch_bounds__(cycle_threads<T>(), 1) k_cycle(CycleArgs<T> a)
     const int gnth = gridDim.x * blockDim.x;
     const RedCtx rc{a.partials, nullptr};
     BigScratch sc;
-    if (a.big_smem && gridDim.x > 1) {
+    if (a.big_smem) {
         unsigned dyn;
         asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
-        sc.p = blockIdx.x ? amg_smem : nullptr;  // CTA 0's holds the tail
+        sc.p = amg_smem;
         sc.bytes = dyn;
-        sc.skip0 = true;
         sc.wwarps = a.big_wwarps;
         sc.wslice = a.big_wslice;
     }
-    for (int k = 0; k < a.nops; k++) {
+    for (int k = a.k0; k < a.k1; k++) {
         const Op &op = sop[k & 1];
         // the next descriptor into the other buffer (last read by op k-1), issued before op k
         // runs: a load still in flight at the barrier would delay its release fence
-        if (threadIdx.x < kOpWords && k + 1 < a.nops)
+        if (threadIdx.x < kOpWords && k + 1 < a.k1)
             ((int *)&sop[(k + 1) & 1])[threadIdx.x] = ((const int *)(a.prog + k + 1))[threadIdx.x];
         if (op.fin_pb >= 0) finalize(a, gtab, op);
-        if (op.kind == OP_TAIL) {
-            if (blockIdx.x == 0) run_tail<T, W>(a);
-        } else if (op.kind != OP_NOP) {
-            run_op<GL, RM_PARTIAL>(gtab, op, rc, gtid, gnth, sc);
-        }
-        if (!grid_barrier(a.bar, a.err, target, abort_flag, a.bar_limit_ns)) break;
+        if (op.kind != OP_NOP) run_op<GL, RM_PARTIAL>(gtab, op, rc, gtid, gnth, sc);
+        // the end of the launch orders its last op before whatever follows on the stream
+        const bool last = k + 1 == a.k1;
+        if (!last && !grid_barrier(a.bar, a.err, target, abort_flag, a.bar_limit_ns)) break;
         if (a.ts && blockIdx.x == 0 && threadIdx.x == 0) a.ts[k] = global_ns();
     }
 }
@@ -1024,15 +597,14 @@ static double op_bytes(const amg_hierarchy *h, const Op &op, int w) {
 struct EngineBase {
     Op *prog = nullptr;
     int nops = 0;
-    int *tail_colors = nullptr;  // colour ranges of the tail levels
-    int tail_color_words = 0;
-    TailLayout lay{};
-    size_t smem = 0;
     int grid = 0;
+    size_t smem = 0;   // of the cycle kernel (big blocks)
     int coop = 0;  // the cycle kernel instance with the lane-parallel block smoother
-    int big_smem = 0;  // CTAs 1.. sweep the big blocks in their shared memory
+    int big_smem = 0;  // the CTAs sweep the big blocks in their shared memory
     int big_wwarps = 0;  // warps of a CTA with a slice for the warp-sized blocks
     unsigned big_wslice = 0;
+    ClLayout cl{};                   // the cluster's levels (cl.tl = nlev: none)
+    unsigned char *cl_image = nullptr;
     std::vector<Op> hprog, htail;
     double tail_bytes = 0, cycle_bytes = 0;
     unsigned long long *ts = nullptr;
@@ -1283,7 +855,6 @@ void table_image(amg_hierarchy *h, std::vector<GLev<T>> &tab) {
         else d.val = (const T *)lv.A.val32;
         if constexpr (sizeof(T) == 8) d.dinv = (const T *)lv.dinv64;
         else d.dinv = (const T *)lv.dinv32;
-        d.col16 = lv.col16;
         d.bptr = lv.bptr;
         d.big = (l == 0) ? lv.big_dev : nullptr;
         d.parent = lv.parent;
@@ -1319,7 +890,6 @@ const GLev<T> *dtab(amg_hierarchy *h) {
     return (const GLev<T> *)((sizeof(T) == 8) ? h->lev_tab64 : h->lev_tab32);
 }
 
-// shared-memory image of levels l0..nlev-1; returns false if a level is too large
 // widest slice (slots per row) of each level, from its slice pointers
 std::vector<int> slice_widths(amg_hierarchy *h) {
     std::vector<int> w(h->nlev, 0);
@@ -1343,169 +913,355 @@ std::vector<int> slice_widths(amg_hierarchy *h) {
     return w;
 }
 
-// shared-memory image of the tail from level l0 down (value size `vb` bytes); the top level
-// may stay in HBM (top_in_gmem). False if a level is too large or the tail too deep.
-bool tail_layout(amg_hierarchy *h, int l0, int vb, bool top_in_gmem,
-                 const std::vector<int> &widths, TailLayout &Y) {
-    std::memset(&Y, 0, sizeof Y);
-    Y.tl = l0;
-    Y.nlev = h->nlev;
-    Y.kc = h->opt.kcycle_n;
-    Y.nu_pre = h->opt.nu_pre;
-    Y.nu_post = h->opt.nu_post;
-    size_t off = 0;
-    auto take = [&](size_t bytes) {
-        int o = (int)off;
-        off += align16(bytes);
-        return o;
-    };
-    // colour ranges of every tail level, one block
-    int words = 0;
-    for (int l = l0; l < h->nlev; l++) words += (int)h->lev[l].color_rows.size();
-    const int cbase = take(sizeof(int) * (size_t)words);
-    int cw = 0;
-    // one slice width for the staged levels: 9 (3x3-cell stencils) if every one fits
-    bool w9 = true;
-    for (int l = l0 + (top_in_gmem ? 1 : 0); l < h->nlev; l++) w9 = w9 && widths[l] <= 9;
-    Y.W = w9 ? 9 : 0;
-    const int kc = h->opt.kcycle_n;
-    for (int l = l0; l < h->nlev; l++) {
-        const Level &lv = h->lev[l];
-        TailLevelLayout &y = Y.lv[l];
-        y.n = lv.n;
-        y.nslices = lv.A.nslices;
-        y.padded = (int)lv.A.padded;
-        y.colors = cbase + (int)sizeof(int) * cw;
-        y.ncolors = (int)lv.color_rows.size() - 1;
-        cw += (int)lv.color_rows.size();
-        if (l == l0 && top_in_gmem) {
-            if (lv.n > 65535 || lv.coarsest) return false;
-            y.gmem = 1;
-            y.w = 0;
-            y.col = y.val = y.dinv = y.parent = y.children = y.children2 = y.Ainv = -1;
-            y.rhs = y.e = y.r = -1;
-            for (int k = 0; k < kMaxKcycle; k++) y.p[k] = y.q[k] = -1;
-            continue;
-        }
-        if (lv.n > kTailRowsMax) return false;
-        y.w = w9 ? 9 : std::max(1, widths[l]);
-        const size_t img = (size_t)lv.A.nslices * kSliceH * y.w;
-        y.col = take(2 * img);
-        y.val = take((size_t)vb * img);
-        y.dinv = lv.coarsest ? -1 : take((size_t)vb * lv.n);
-        y.parent = lv.coarsest ? -1 : take(sizeof(int) * (size_t)lv.n);
-        y.children = (l > l0) ? take(sizeof(int4) * (size_t)lv.n) : -1;
-        y.children2 = (l > l0 && lv.children2) ? take(sizeof(int4) * (size_t)lv.n) : -1;
-        y.Ainv = lv.coarsest ? take(sizeof(double) * lv.n * lv.n) : -1;
-        y.rhs = take((size_t)vb * lv.n);
-        y.e = take((size_t)vb * lv.n);
-        y.r = lv.coarsest ? -1 : take((size_t)vb * lv.n);
-        for (int k = 0; k < kMaxKcycle; k++) {
-            y.p[k] = (!lv.coarsest && k < kc) ? take((size_t)vb * lv.n) : -1;
-            y.q[k] = (!lv.coarsest && k < kc) ? take((size_t)vb * lv.n) : -1;
-        }
-        if (off > (size_t)INT32_MAX) return false;
-    }
-    // narrow group: about one thread per row of a colour of the largest staged level (a
-    // quarter of its rows for the 2x2 colouring), whole warps, 128..1024 threads
-    int nmax = 0;
-    for (int l = l0; l < h->nlev; l++)
-        if (!Y.lv[l].gmem) nmax = std::max(nmax, Y.lv[l].n);
-    Y.narrow = std::min(vb == 8 ? kPThreads64 : kPThreads, std::max(128, (nmax / 4 + 31) / 32 * 32));
-    if (const char *e = getenv("AMG_TAIL_NARROW")) {  // tuning knob: threads of the narrow group
-        const int v = atoi(e);
-        if (v >= 32 && v <= (vb == 8 ? kPThreads64 : kPThreads) && v % 32 == 0) Y.narrow = v;
-    }
-    Y.sc = take(sizeof(double) * SC_N * (size_t)(h->nlev - l0));
-    Y.bytes = (int)off;
-    return true;
-}
-
 template <class T>
 EngineBase *&engine_slot(amg_hierarchy *h) {
     return (sizeof(T) == 8) ? h->eng64 : h->eng32;
 }
 
-int max_tail_bytes() {
-    static int v = [] {
-        const char *e = getenv("AMG_TAIL_SMEM");  // tuning knob: cap on the staged tail
-        return e ? atoi(e) : INT32_MAX;
-    }();
-    return v;
+template <class T>
+void *cycle_kernel(int B) {
+    return B ? (void *)k_cycle<T, 1> : (void *)k_cycle<T, 0>;
+}
+
+// ---------------------------------------------------------------------------------------
+// the cluster's levels (cluster_tail.cuh)
+
+// one candidate: swept levels [tl, tl + nsp), the dense level after them
+struct ClPlan {
+    ClLayout y;
+    std::vector<unsigned char> tables;  // [kClRanks][table_bytes]: the head of every image
+    int table_bytes = 0;
+};
+
+// Layout and tables for swept levels first .. of src (win: their windows), or false if they
+// do not fit `budget` bytes of shared memory. `s0`: src index of the first swept level.
+template <class T>
+bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vector<int> &xchild,
+                  const std::vector<int> &widths, int s0, int level0, bool dense, int nch,
+                  const amg_options &opt, long budget, ClPlan &P) {
+    constexpr int vb = (int)sizeof(T), NR = kClRanks;
+    ClLayout &y = P.y;
+    std::memset(&y, 0, sizeof y);
+    y.nsp = G.nsp - s0;
+    y.tl = level0;
+    y.dense = dense;
+    y.kc = opt.kcycle_n;
+    y.nu_pre = opt.nu_pre;
+    y.nu_post = opt.nu_post;
+    const ClSrc &D = G.lv[G.nsp];
+    y.nd = D.n;
+    y.ch = (((D.n + NR - 1) / NR) + 3) & ~3;
+    y.stride = NR * y.ch;
+    auto win_of = [&](int a, int r, int c) {
+        return win[((size_t)(s0 + a) * NR + r) * kClColors + c];
+    };
+    auto own_of = [](const ClSrc &S, int r, int c) {
+        const int len = S.cr[c + 1] - S.cr[c];
+        return make_int2(S.cr[c] + cl_part(len, r), S.cr[c] + cl_part(len, r + 1));
+    };
+    // tables, one image per CTA
+    struct LevelTab {
+        ClHead head;
+        std::vector<ClColor> col;
+        std::vector<ClPush> push;
+    };
+    std::vector<std::vector<LevelTab>> tab(NR, std::vector<LevelTab>(y.nsp));
+    std::vector<std::vector<int>> down(NR), peers(NR);
+    std::vector<std::vector<char>> is_peer(NR, std::vector<char>(NR, 0));
+    std::vector<size_t> max_push(y.nsp, 1), max_own(y.nsp + 1, 1), max_win(y.nsp, 1);
+    for (int a = 0; a < y.nsp; a++) {
+        const ClSrc &S = G.lv[s0 + a];
+        for (int r = 0; r < NR; r++) {
+            LevelTab &t = tab[r][a];
+            t.col.resize(S.ncol);
+            int m0 = 0, seg0 = 0;
+            for (int c = 0; c < S.ncol; c++) {
+                const int2 o = own_of(S, r, c), w = win_of(a, r, c);
+                ClColor &C = t.col[c];
+                std::memset(&C, 0, sizeof C);
+                C.cnt = o.y - o.x;
+                C.m0 = m0;
+                C.seg0 = seg0;
+                C.seglen = w.y - w.x;
+                C.li0 = seg0 + o.x - w.x;
+                C.g0 = o.x;
+                m0 += C.cnt;
+                seg0 += C.seglen;
+            }
+            if (seg0 > 65534) return false;
+            t.head = ClHead{m0, seg0, 0, 0};
+            max_own[a] = std::max(max_own[a], (size_t)m0);
+            max_win[a] = std::max(max_win[a], (size_t)seg0);
+        }
+        for (int r = 0; r < NR; r++)
+            for (int c = 0; c < S.ncol; c++) {
+                const int2 o = own_of(S, r, c);
+                ClColor &C = tab[r][a].col[c];
+                C.push0 = (int)tab[r][a].push.size();
+                for (int d = 0; d < NR; d++) {
+                    if (d == r) continue;
+                    const int2 w = win_of(a, d, c);
+                    const int lo = std::max(o.x, w.x), hi = std::min(o.y, w.y);
+                    if (lo >= hi) continue;
+                    ClColor &X = tab[d][a].col[c];
+                    tab[r][a].push.push_back(ClPush{d + 256 * c, lo - o.x, hi - lo, X.seg0 + lo - w.x});
+                    X.expect += (hi - lo) * vb;
+                    tab[d][a].head.expect_all += (hi - lo) * vb;
+                    is_peer[r][d] = is_peer[d][r] = 1;
+                }
+                C.npush = (int)tab[r][a].push.size() - C.push0;
+            }
+        for (int r = 0; r < NR; r++) {
+            tab[r][a].head.npush = (int)tab[r][a].push.size();
+            max_push[a] = std::max(max_push[a], tab[r][a].push.size());
+        }
+    }
+    for (int r = 0; r < NR; r++) {
+        for (int c = 0; c < D.ncol; c++) {
+            const int2 o = own_of(D, r, c);
+            for (int i = o.x; i < o.y; i++) down[r].push_back(i);
+        }
+        max_own[y.nsp] = std::max(max_own[y.nsp], down[r].size());
+        for (int d = 0; d < NR; d++)
+            if (is_peer[r][d]) peers[r].push_back(d);
+    }
+    size_t off = 0;
+    auto take = [&](size_t bytes) {
+        const int o = (int)off;
+        off += align16(bytes);
+        return o;
+    };
+    y.dhead = take(sizeof(int));
+    y.down = take(sizeof(short) * max_own[y.nsp]);
+    y.peers = take(sizeof(int) * (NR + 1));
+    for (int a = 0; a < y.nsp; a++) {
+        ClLev &L = y.lv[a];
+        const ClSrc &S = G.lv[s0 + a];
+        L.head = take(sizeof(ClHead));
+        L.tab = take(sizeof(ClColor) * S.ncol);
+        L.push = take(sizeof(ClPush) * max_push[a]);
+    }
+    P.table_bytes = (int)off;
+    for (int a = 0; a < y.nsp; a++) {
+        ClLev &L = y.lv[a];
+        const ClSrc &S = G.lv[s0 + a];
+        L.level = level0 + a;
+        L.n = S.n;
+        L.ncol = S.ncol;
+        L.w = std::max(1, widths[level0 + a]);
+        L.R = (int)((max_own[a] + 23) / 32 * 32 + 8);
+        L.c_first = -1;
+        for (int c = 0; c < S.ncol; c++)
+            if (S.cr[c + 1] > S.cr[c]) {
+                if (L.c_first < 0) L.c_first = c;
+                L.c_last = c;
+                L.cmask |= 1u << c;
+            }
+        L.nch = nch;
+        L.Rn = (int)max_own[a + 1];
+        L.xchild = xchild[s0 + a];
+        L.val = take((size_t)L.w * L.R * vb);
+        L.col = take((size_t)L.w * L.R * 2);
+        L.dinv = take(max_win[a] * vb);
+        L.own = take(2 * max_own[a]);
+        L.parent = take(2 * max_win[a]);
+        L.child = take(2 * (size_t)nch * L.Rn);
+    }
+    y.mat = take((size_t)(dense ? 2 : 1) * y.ch * y.stride * vb);
+    if (!dense && vb == 4) y.mat_lo = take((size_t)y.ch * y.stride * vb);
+    y.image_bytes = (int)off;
+    for (int a = 0; a < y.nsp; a++) {
+        ClLev &L = y.lv[a];
+        const size_t b = max_win[a] * vb;
+        L.rhs = take(b);
+        L.e = take(b);
+        L.r = take(b);
+        for (int k = 0; k < y.kc; k++) {
+            L.p[k] = take(b);
+            L.q[k] = take(b);
+        }
+    }
+    const size_t len = (size_t)y.stride * vb;
+    y.F = take(len);
+    y.E = take(len);
+    y.out = take((size_t)2 * y.ch * vb);
+    y.stage = take(max_own[y.nsp] * vb);
+    if (dense) {
+        y.Rv = take(len);
+        for (int k = 0; k < y.kc; k++) {
+            y.P[k] = take(len);
+            y.Q[k] = take(len);
+        }
+    }
+    y.bytes = (int)off;
+    if ((long)off > budget) return false;
+    P.tables.assign((size_t)NR * P.table_bytes, 0);
+    for (int r = 0; r < NR; r++) {
+        unsigned char *im = P.tables.data() + (size_t)r * P.table_bytes;
+        auto put = [&](int o, const void *p, size_t b) { if (b) std::memcpy(im + o, p, b); };
+        const int nd = (int)down[r].size(), np = (int)peers[r].size();
+        put(y.dhead, &nd, sizeof nd);
+        const std::vector<unsigned short> d16(down[r].begin(), down[r].end());
+        put(y.down, d16.data(), 2 * d16.size());
+        put(y.peers, &np, sizeof np);
+        put(y.peers + (int)sizeof(int), peers[r].data(), sizeof(int) * peers[r].size());
+        for (int a = 0; a < y.nsp; a++) {
+            const LevelTab &t = tab[r][a];
+            put(y.lv[a].head, &t.head, sizeof t.head);
+            put(y.lv[a].tab, t.col.data(), sizeof(ClColor) * t.col.size());
+            put(y.lv[a].push, t.push.data(), sizeof(ClPush) * t.push.size());
+        }
+    }
+    return true;
 }
 
 template <class T>
-void *cycle_kernel(int W, int B) {
-    if (B) return W == 9 ? (void *)k_cycle<T, 9, 1> : (void *)k_cycle<T, 0, 1>;
-    return W == 9 ? (void *)k_cycle<T, 9, 0> : (void *)k_cycle<T, 0, 0>;
+void *cluster_kernel() {
+    return (void *)k_cluster_tail<T>;
+}
+
+// Chooses the cluster's levels (the finest level from which everything fits) and builds their
+// image. E->cl.tl = nlev if there are none: every level runs on the grid.
+template <class T>
+void build_cluster(amg_hierarchy *h, EngineBase *E, int optin) {
+    cudaStream_t s = h->stream;
+    const int nlev = h->nlev;
+    std::memset(&E->cl, 0, sizeof E->cl);
+    E->cl.tl = nlev;
+    cudaFuncAttributes fa;
+    AMG_CUDA(cudaFuncGetAttributes(&fa, cluster_kernel<T>()));
+    const long budget = (long)optin - (long)fa.sharedSizeBytes - 1024;
+    AMG_CUDA(cudaFuncSetAttribute(cluster_kernel<T>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)budget));
+    AMG_CUDA(cudaFuncSetAttribute(cluster_kernel<T>(), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    const std::vector<int> widths = slice_widths(h);
+    auto sweepable = [&](int l) {
+        const Level &lv = h->lev[l];
+        return lv.n <= kClRowsMax && (int)lv.color_rows.size() - 1 <= kClColors && !lv.coarsest;
+    };
+    auto source = [&](int l, bool ranges) {
+        ClSrc S;
+        std::memset(&S, 0, sizeof S);
+        const Level &lv = h->lev[l];
+        S.n = lv.n;
+        S.sl = lv.A.sl_ptr;
+        S.col = lv.A.col;
+        S.parent = lv.parent;
+        S.ch = l + 1 < nlev ? h->lev[l + 1].children : nullptr;
+        S.ch2 = l + 1 < nlev ? h->lev[l + 1].children2 : nullptr;
+        S.val64 = lv.A.val;
+        S.val32 = lv.A.val32;
+        S.ncol = ranges ? (int)lv.color_rows.size() - 1 : 1;
+        if (ranges)
+            for (int c = 0; c <= S.ncol; c++) S.cr[c] = lv.color_rows[c];
+        else
+            S.cr[1] = lv.n;
+        return S;
+    };
+    // the dense level is the one above the coarsest (M, A M) or the coarsest (its inverse);
+    // windows are found for every level that may be swept
+    const int last = nlev - 2;  // the coarsest level that is swept or dense
+    if (last < 1) return;
+    int first = last + 1;
+    while (first - 1 >= 1 && sweepable(first - 1) && last + 1 - (first - 1) <= kClLevels) first--;
+    if (first > last) return;
+    const int nch = h->lev[nlev - 1].children2 ? 8 : 4;
+    ClSrcs G;
+    std::memset(&G, 0, sizeof G);
+    G.nsp = last + 1 - first;
+    for (int a = 0; a < G.nsp; a++) G.lv[a] = source(first + a, true);
+    // the coarsest level is not smoothed; its colours only cut it into strips
+    const bool crr = (int)h->lev[nlev - 1].color_rows.size() - 1 <= kClColors &&
+                     h->lev[nlev - 1].color_rows.size() > 1;
+    G.lv[G.nsp] = source(nlev - 1, crr);
+    const size_t words = (size_t)G.nsp * kClRanks * kClColors;
+    std::vector<int2> win(2 * words);
+    for (int a = 0; a < G.nsp; a++)
+        for (int r = 0; r < kClRanks; r++)
+            for (int c = 0; c < kClColors; c++) {
+                const size_t o = ((size_t)a * kClRanks + r) * kClColors + c;
+                const ClSrc &S = G.lv[a];
+                const int len = c < S.ncol ? S.cr[c + 1] - S.cr[c] : 0;
+                win[o] = c < S.ncol ? make_int2(S.cr[c] + cl_part(len, r), S.cr[c] + cl_part(len, r + 1))
+                                    : make_int2(0, 0);
+                win[words + o] = make_int2(INT32_MAX, 0);
+            }
+    Scratch tmp(s);
+    int2 *dwin = tmp.get<int2>(2 * words);
+    AMG_CUDA(cudaMemcpyAsync(dwin, win.data(), sizeof(int2) * win.size(), cudaMemcpyHostToDevice, s));
+    k_cl_windows<<<dim3(nblocks_for(G.lv[0].n, 256), G.nsp), 256, 0, s>>>(G, dwin, dwin + words);
+    AMG_LAUNCH_CHECK();
+    k_cl_parents<<<1, 1024, 0, s>>>(G, dwin, dwin + words);
+    AMG_LAUNCH_CHECK();
+    AMG_CUDA(cudaMemcpyAsync(win.data(), dwin, sizeof(int2) * win.size(), cudaMemcpyDeviceToHost, s));
+    AMG_CUDA(cudaStreamSynchronize(s));
+    std::vector<int> xchild(G.nsp, 0);
+    for (int a = 0; a < G.nsp; a++)
+        for (size_t k = 0; k < (size_t)kClRanks * kClColors; k++) {
+            const int2 w = win[words + (size_t)a * kClRanks * kClColors + k];
+            if (w.x < w.y) xchild[a] = 1;
+        }
+    // the finest start that fits; with the dense matrices if that start allows them
+    ClSrcs GD = G;  // dense level = the last swept one
+    GD.nsp = G.nsp - 1;
+    const bool can_dense = h->lev[last].n <= kClDenseMax;
+    ClPlan P;
+    bool ok = false;
+    int s0 = 0;
+    for (; s0 < G.nsp && !ok; s0++) {
+        ok = can_dense && cluster_plan<T>(GD, win, xchild, widths, s0, first + s0, true, nch, h->opt, budget, P);
+        if (!ok) ok = cluster_plan<T>(G, win, xchild, widths, s0, first + s0, false, nch, h->opt, budget, P);
+        if (ok) break;
+    }
+    if (!ok) return;
+    ClLayout &y = P.y;
+    ClSrcs &U = y.dense ? GD : G;
+    if (s0 > 0) {
+        for (int a = 0; a + s0 <= U.nsp; a++) U.lv[a] = U.lv[a + s0];
+        U.nsp -= s0;
+    }
+    E->cl_image = halloc<unsigned char>(h, (size_t)kClRanks * y.image_bytes);
+    AMG_CUDA(cudaMemsetAsync(E->cl_image, 0, (size_t)kClRanks * y.image_bytes, s));
+    AMG_CUDA(cudaMemcpy2DAsync(E->cl_image, y.image_bytes, P.tables.data(), P.table_bytes, P.table_bytes,
+                               kClRanks, cudaMemcpyHostToDevice, s));
+    const Level &C = h->lev[nlev - 1];
+    k_cl_image<T><<<dim3(4, kClRanks, y.nsp + 1), 256, 0, s>>>(U, y, E->cl_image, C.Ainv, C.Ainv32);
+    AMG_LAUNCH_CHECK();
+    if (y.dense) {
+        const size_t smem = sizeof(double) * (3 * (size_t)y.nd + 2 * (size_t)C.n);
+        k_dense_cycle<T><<<y.nd, 128, smem, s>>>(U.lv[U.nsp], y, E->cl_image, C.Ainv, C.n);
+        AMG_LAUNCH_CHECK();
+    }
+    AMG_CUDA(cudaStreamSynchronize(s));  // P.tables is a local
+    E->cl = y;
 }
 
 template <class T>
 void build_engine(amg_hierarchy *h) {
-    EngineBase *&E = engine_slot<T>(h);
-    if (!E) E = new EngineBase();
+    EngineBase *&slot = engine_slot<T>(h);
+    if (slot) return;
+    // kept only when complete (an allocation can fail part-way)
+    struct Holder {
+        EngineBase *p = new EngineBase();
+        ~Holder() { delete p; }
+    } hold;
+    EngineBase *E = hold.p;
     cudaStream_t s = h->stream;
     int dev = h->device, optin = 0, nsm = 0;
     AMG_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     AMG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    size_t static_smem = 0;
-    for (int W : {0, 9})
-        for (int B : {0, 1}) {
-            cudaFuncAttributes fa;
-            AMG_CUDA(cudaFuncGetAttributes(&fa, cycle_kernel<T>(W, B)));
-            static_smem = std::max(static_smem, fa.sharedSizeBytes);
-        }
     E->coop = coop_blocks(h->lev[0]) ? 1 : 0;
-    const long budget = std::min<long>((long)optin - (long)static_smem - 1024,
-                                       (long)max_tail_bytes());
-    // the tail: the finest coarse level from which everything fits in shared memory, or
-    // fits once that top level is left in HBM/L2 (read in place by CTA 0)
-    const std::vector<int> widths = slice_widths(h);
-    int tl = h->nlev;
-    for (int l = 1; l < h->nlev && tl == h->nlev; l++) {
-        for (int top_gmem = 0; top_gmem <= 1; top_gmem++) {
-            TailLayout Y;
-            if (tail_layout(h, l, sizeof(T), top_gmem != 0, widths, Y) && Y.bytes <= budget) {
-                tl = l;
-                E->lay = Y;
-                break;
-            }
-        }
-    }
-    if (tl < h->nlev && E->lay.lv[tl].gmem && !h->lev[tl].col16) {
-        Level &lv = h->lev[tl];
-        lv.col16 = halloc<unsigned short>(h, lv.A.padded);
-        k_col16<<<nblocks_for(lv.A.padded, 256), 256, 0, h->stream>>>((int)lv.A.padded, lv.A.col, lv.col16);
-        AMG_LAUNCH_CHECK();
-        fill_tables<T>(h);
-    }
-    if (tl == h->nlev) {
-        std::memset(&E->lay, 0, sizeof E->lay);
-        E->lay.tl = h->nlev;
-        E->lay.nlev = h->nlev;
-    }
+    build_cluster<T>(h, E, optin);
+    const int tl = E->cl.tl;
     h->tail_level = tl;
-    E->hprog.clear();
-    E->htail.clear();
     Builder b{h, &E->hprog, tl};
     b.bhat(0, V_RHS, V_E);
     annotate_reductions(E->hprog);
-    E->tail_color_words = 0;
     if (tl < h->nlev) {
-        Builder bt{h, &E->htail, h->nlev + 1};  // the tail's ops (traffic accounting only)
+        Builder bt{h, &E->htail, h->nlev + 1};  // the cluster's ops (traffic accounting only)
         bt.btilde(tl);
-        std::vector<int> words;
-        for (int l = tl; l < h->nlev; l++)
-            words.insert(words.end(), h->lev[l].color_rows.begin(), h->lev[l].color_rows.end());
-        E->tail_color_words = (int)words.size();
-        E->tail_colors = halloc<int>(h, words.size());
-        AMG_CUDA(cudaMemcpyAsync(E->tail_colors, words.data(), sizeof(int) * words.size(),
-                                 cudaMemcpyHostToDevice, s));
-        AMG_CUDA(cudaStreamSynchronize(s));  // words is a local
     }
-    E->tail_bytes = 0;
     for (const Op &op : E->htail) E->tail_bytes += op_bytes(h, op, sizeof(T));
-    E->cycle_bytes = 0;
     for (const Op &op : E->hprog)
         E->cycle_bytes += (op.kind == OP_TAIL) ? E->tail_bytes
                           : (op.kind == OP_NOP) ? 0.0 : op_bytes(h, op, sizeof(T));
@@ -1513,15 +1269,15 @@ void build_engine(amg_hierarchy *h) {
     E->prog = halloc<Op>(h, E->hprog.size());
     AMG_CUDA(cudaMemcpyAsync(E->prog, E->hprog.data(), sizeof(Op) * E->hprog.size(),
                              cudaMemcpyHostToDevice, s));
-    E->smem = tl < h->nlev ? (size_t)E->lay.bytes : 0;
-    // Big blocks: swept in the shared memory of CTAs 1... A CTA-sized block needs as much as
-    // the largest one that fits on the device; the warp-sized ones get a slice each on as
-    // many warps per CTA as the most of them in one colour need (a block that does not fit
-    // takes the global-memory sweep; the forward and backward schedules each count).
-    E->big_smem = 0;
-    E->big_wwarps = 0;
-    E->big_wslice = 0;
-    if (h->lev[0].nbig > 0 && nsm > 1) {
+    // Big blocks: swept in the CTAs' shared memory. A CTA-sized block needs as much as the
+    // largest one that fits on the device; the warp-sized ones get a slice each on as many
+    // warps per CTA as the most of them in one colour need (a block that does not fit takes
+    // the global-memory sweep; the forward and backward schedules each count).
+    void *kern = cycle_kernel<T>(E->coop);
+    cudaFuncAttributes fa;
+    AMG_CUDA(cudaFuncGetAttributes(&fa, kern));
+    const size_t static_smem = fa.sharedSizeBytes;
+    if (h->lev[0].nbig > 0) {
         const Level &F0 = h->lev[0];
         const int vsel = sizeof(T) == 8;
         const size_t avail = (size_t)std::max<long>(0, (long)optin - (long)static_smem - 1024);
@@ -1533,17 +1289,16 @@ void build_engine(amg_hierarchy *h) {
         for (size_t c = 0; c < F0.color_bigc.size(); c++)
             wtasks = std::max(wtasks, F0.color_bigc[c] - F0.color_big[c]);
         if (wneed > 0 && wneed <= avail && wtasks > 0) {
-            const int per_cta = (wtasks + nsm - 2) / (nsm - 1);
+            const int per_cta = (wtasks + nsm - 1) / nsm;
             E->big_wwarps = std::min({cycle_threads<T>() / 32, per_cta, (int)(avail / wneed)});
             E->big_wslice = (unsigned)wneed;
         }
         const size_t smem = std::max(big, (size_t)E->big_wwarps * E->big_wslice);
         if (smem > 0) {
             E->big_smem = 1;
-            E->smem = std::max(E->smem, smem);
+            E->smem = smem;
         }
     }
-    void *kern = cycle_kernel<T>(E->lay.W, E->coop);
     // the kernel's dynamic shared-memory limit is a property of the function, shared by every
     // hierarchy of the process: set it to the device maximum (never lower it below what
     // another hierarchy's launches use); each launch passes its own size
@@ -1557,7 +1312,10 @@ void build_engine(amg_hierarchy *h) {
     E->ts = halloc<unsigned long long>(h, E->hprog.size() + 1);
     E->tprof = halloc<unsigned long long>(h, 2 * kTprofCount);
     AMG_CUDA(cudaMemsetAsync(E->tprof, 0, 2 * kTprofCount * sizeof(unsigned long long), s));
+    slot = E;
+    hold.p = nullptr;
 }
+
 
 template <class T>
 void alloc_vecs(amg_hierarchy *h) {
@@ -1611,7 +1369,9 @@ void ensure_fp32(amg_hierarchy *h) {
     h->fp32_ready = true;
 }
 
-// one launch of the persistent kernel: z = B^_0 [r] on level 0's table buffers
+// one application: z = B^_0 [r] on level 0's table buffers. The program runs as launches of
+// the persistent kernel over the ops between the cluster's levels, and of the cluster kernel
+// for these
 template <class T>
 void launch_cycle(amg_hierarchy *h, T *rhs0 = nullptr, T *e0 = nullptr) {
     // hierarchies of a batched setup get their single-system engine on first use
@@ -1624,10 +1384,7 @@ void launch_cycle(amg_hierarchy *h, T *rhs0 = nullptr, T *e0 = nullptr) {
     a.rhs0 = rhs0;
     a.e0 = e0;
     a.prog = E->prog;
-    a.nops = E->nops;
-    a.tail_colors = E->tail_colors;
-    a.tail_color_words = E->tail_color_words;
-    a.lay = E->lay;
+    a.nlev = h->nlev;
     a.partials = h->cyc_partials;
     a.bar = h->bar;
     a.err = h->err_flag;
@@ -1639,17 +1396,57 @@ void launch_cycle(amg_hierarchy *h, T *rhs0 = nullptr, T *e0 = nullptr) {
     a.big_wslice = E->big_wslice;
     AMG_CUDA(cudaMemsetAsync(h->bar, 0, sizeof(unsigned long long), s));
     a.ts = prof ? E->ts + 1 : nullptr;
-    a.tprof = (prof && h->prof->tail_ops) ? E->tprof : nullptr;
     Profiler::Rec rec{};
     if (prof) {
         k_timestamp<<<1, 1, 0, s>>>(E->ts);
         AMG_LAUNCH_CHECK();
         rec = h->prof->begin(K_CYCLE, 0, E->cycle_bytes, s);
     }
-    void *args[] = {&a};
-    AMG_CUDA(cudaLaunchCooperativeKernel(cycle_kernel<T>(E->lay.W, E->coop), dim3(E->grid),
-                                         dim3(cycle_threads<T>()), args, E->smem, s));
-    AMG_LAUNCH_CHECK();
+    ClArgs<T> ca;
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute attr;
+    if (E->cl.tl < h->nlev) {
+        const Vecs<T> &v = vecs<T>(h->lev[E->cl.tl]);
+        ca.y = E->cl;
+        ca.image = E->cl_image;
+        ca.rhs = v.rhs;
+        ca.e = v.e;
+        ca.err = h->err_flag;
+        ca.limit_ns = a.bar_limit_ns;
+        ca.extra = h->dbg_bar_extra;
+        ca.tprof = (prof && h->prof->tail_ops) ? E->tprof : nullptr;
+        std::memset(&cfg, 0, sizeof cfg);
+        cfg.gridDim = dim3(kClRanks);
+        cfg.blockDim = dim3(kClThreads);
+        cfg.dynamicSmemBytes = (size_t)E->cl.bytes;
+        cfg.stream = s;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = kClRanks;
+        attr.val.clusterDim.y = 1;
+        attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+    }
+    unsigned long long bars = 0;  // barriers of the launches so far
+    for (int k = 0; k < E->nops;) {
+        if (E->hprog[k].kind == OP_TAIL) {
+            ca.ts = prof ? a.ts + k : nullptr;
+            void *args[] = {&ca};
+            AMG_CUDA(cudaLaunchKernelExC(&cfg, cluster_kernel<T>(), args));
+            AMG_LAUNCH_CHECK();
+            k++;
+            continue;
+        }
+        a.k0 = k;
+        while (k < E->nops && E->hprog[k].kind != OP_TAIL) k++;
+        a.k1 = k;
+        a.bar_base = bars * (unsigned long long)E->grid;
+        bars += (unsigned long long)(a.k1 - a.k0 - 1);
+        void *args[] = {&a};
+        AMG_CUDA(cudaLaunchCooperativeKernel(cycle_kernel<T>(E->coop), dim3(E->grid),
+                                             dim3(cycle_threads<T>()), args, E->smem, s));
+        AMG_LAUNCH_CHECK();
+    }
     if (prof) h->prof->end(rec, s);
 }
 
