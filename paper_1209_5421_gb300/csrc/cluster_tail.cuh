@@ -17,8 +17,8 @@
 // auxiliary grid. CTA r's window of colour c is the smallest row interval that holds its own
 // rows, the columns of its own rows, the rows whose columns its own rows are (both, so that
 // the exchange is symmetric), the children of its own rows of the next level, and the parents
-// of its window on the level above. Every vector of a level is stored in window order, one
-// index for all of them.
+// of its window on the level above. The vectors that others read
+// (z, e, the residual) are stored in window order, the others by own row.
 //
 // What keeps the steps in order without a cluster barrier. Neighbour exchanges are numbered;
 // exchange k counts on mbarrier k mod 2. Each CTA sends every neighbour (the same set for all
@@ -38,6 +38,7 @@
 // and the coarsest solve is the dense product.
 #pragma once
 
+#include <cstddef>
 #include <cstring>
 #include <type_traits>
 
@@ -52,38 +53,40 @@ constexpr int kClLevels = 8;       // swept levels at most
 constexpr int kClColors = 32;      // colours of a swept level at most
 constexpr int kClRowsMax = 20480;  // rows of a swept level at most (16-bit window indices)
 constexpr int kClDenseMax = 512;   // rows of the dense level at most
-constexpr int kClBatch = 9;        // slots read together (one batch for a 9-point row)
+constexpr int kClSlots = 8;        // off-diagonal slots a lane takes at most
+constexpr unsigned kClNone = 0x7FFFFFFFu;  // no destination
 
-// one colour of one CTA's strip
+// one colour of a sweep on one CTA's strip; a level's sweeps are lists of these
+struct __align__(16) ClOp {
+    int m0, cnt;       // own rows, times lanes per row
+    int expect;        // bytes its window receives in the exchange
+    int pad;
+};
+struct __align__(16) ClHead {  // of one level's strip
+    int nown, nwin, expect_all, fexp;  // fexp: bytes of the first non-empty colour,
+    int fc0, fcn, fs0, fs1;    //   its own rows [fc0, fc0 + fcn) and window [fs0, fs1)
+    int ls0, ls1, pad[2];      // last non-empty colour: window
+};
+// one colour of one CTA's strip (setup of the image only)
 struct ClColor {
     int li0, cnt;      // own rows: window index of the first, number
-    int m0;            // its index among the own rows of all colours (matrix rows)
+    int m0;            // its index among the own rows of all colours
     int seg0, seglen;  // the colour's window
-    int push0, npush;  // its rows' destinations
-    int expect;        // bytes its window receives from the neighbours in an exchange
     int g0;            // pi-row of the first own row
-    int pad[3];
-};
-// rows [j0, j0 + cnt) of the colour's own rows go to CTA dst, window index dli there
-struct ClPush {
-    int dst_color;     // dst + 256 colour
-    int j0, cnt, dli;
-};
-struct ClHead {        // of one level's strip
-    int nown, nwin, npush, expect_all;
 };
 
 // a swept level: sizes, and byte offsets into the shared memory (the same in every CTA)
-struct ClLev {
-    int level, n, ncol, w;
-    int R;             // matrix rows (own rows of the largest strip, 8 mod 32)
-    int c_first, c_last;
-    unsigned cmask;    // non-empty colours
-    int nch;           // children per row of the next level's rows: 4 or 8
-    int Rn;            // stride of the children's table (own rows of the next level)
+struct __align__(16) ClLev {
+    int own, col, val, diag;   // constant image: own rows' window indices, matrix,
+    int dinv, dst, over, head; //   1 / a_ii, destinations (and further ones), ClHead
+    int lg, ns;        // log2 of the lanes per row; off-diagonal slots a lane takes (even)
+    int R;             // stride of the matrix tables (largest strip's rows times lanes)
     int xchild;        // 1: a child of an own next-level row may lie in another strip
-    int head, tab, push, val, col, dinv, own, parent, child;  // constant image
-    int rhs, e, r, p[kMaxKcycle], q[kMaxKcycle];              // vectors
+    int pre, post, npre, npost;  // sweeps (ClOp) and their lengths
+    int parent, child, nch, Rn;  // maps; children per row of the next level's rows, stride
+    int rhs, r, e, nact;       // vectors: by own row, by window index; warps with rows in sums
+    int p[kMaxKcycle], q[kMaxKcycle];
+    int level, ncol, w, pad;
 };
 
 struct ClLayout {
@@ -95,6 +98,8 @@ struct ClLayout {
     int mat, mat_lo;     // M then A M (or the inverse; FP32: high parts, low parts)
     int dhead, down;     // gather into the dense level: own rows (count; their pi-rows)
     int peers;           // neighbour CTAs: count, ranks
+    int levels;          // lv[] (a copy in the image)
+    int top;             // pi-rows of the top level's own rows
     int F, Rv, E, out, P[kMaxKcycle], Q[kMaxKcycle];  // dense level's vectors (every CTA: all)
     int stage;           // one value per own row of the dense level
     int image_bytes, bytes;
@@ -119,6 +124,46 @@ struct ClArgs {
 __device__ __forceinline__ uint32_t cl_smem(const void *p) {
     return (uint32_t)__cvta_generic_to_shared(p);
 }
+// shared memory by 32-bit address: a load is one instruction and an address one add (through
+// generic pointers each address is a 64-bit sum)
+__device__ __forceinline__ void cl_lds(uint32_t a, float &v) {
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void cl_lds(uint32_t a, double &v) {
+    asm volatile("ld.shared.f64 %0, [%1];" : "=d"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void cl_lds(uint32_t a, int &v) {
+    asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void cl_lds(uint32_t a, unsigned short &v) {
+    asm volatile("ld.shared.u16 %0, [%1];" : "=h"(v) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void cl_lds(uint32_t a, uint2 &v) {
+    asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void cl_lds(uint32_t a, uint4 &v) {
+    asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void cl_lds(uint32_t a, float4 &v) {
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(a) : "memory");
+}
+__device__ __forceinline__ void cl_lds(uint32_t a, double2 &v) {
+    asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "r"(a) : "memory");
+}
+template <class V>
+__device__ __forceinline__ V cl_ld(uint32_t a) {
+    V v;
+    cl_lds(a, v);
+    return v;
+}
+__device__ __forceinline__ void cl_st(uint32_t a, float v) {
+    asm volatile("st.shared.f32 [%0], %1;" ::"r"(a), "f"(v) : "memory");
+}
+__device__ __forceinline__ void cl_st(uint32_t a, double v) {
+    asm volatile("st.shared.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
 __device__ __forceinline__ uint32_t cl_map(uint32_t addr, int rank) {
     uint32_t o;
     asm("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(o) : "r"(addr), "r"(rank));
@@ -131,6 +176,27 @@ __device__ __forceinline__ void cl_store(uint32_t a, float v, uint32_t mb) {
 __device__ __forceinline__ void cl_store(uint32_t a, double v, uint32_t mb) {
     asm volatile("st.async.shared::cluster.mbarrier::complete_tx::bytes.f64 [%0], %1, [%2];" ::"r"(a),
                  "d"(v), "r"(mb) : "memory");
+}
+// the same where `on` (no branch: a branch costs a warp as much as a few instructions)
+__device__ __forceinline__ void cl_store_if(bool on, uint32_t a, float v, uint32_t mb) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.u32 p, %3, 0;\n"
+        "@p st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [%0], %1, [%2];\n}" ::"r"(a),
+        "f"(v), "r"(mb), "r"((unsigned)on) : "memory");
+}
+__device__ __forceinline__ void cl_store_if(bool on, uint32_t a, double v, uint32_t mb) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.u32 p, %3, 0;\n"
+        "@p st.async.shared::cluster.mbarrier::complete_tx::bytes.f64 [%0], %1, [%2];\n}" ::"r"(a),
+        "d"(v), "r"(mb), "r"((unsigned)on) : "memory");
+}
+__device__ __forceinline__ void cl_st_if(bool on, uint32_t a, float v) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p st.shared.f32 [%0], %1;\n}" ::"r"(a), "f"(v),
+                 "r"((unsigned)on) : "memory");
+}
+__device__ __forceinline__ void cl_st_if(bool on, uint32_t a, double v) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p st.shared.f64 [%0], %1;\n}" ::"r"(a), "d"(v),
+                 "r"((unsigned)on) : "memory");
 }
 __device__ __forceinline__ void cl_store16(uint32_t a, const float *v, uint32_t mb) {
     const float4 x = *reinterpret_cast<const float4 *>(v);
@@ -147,8 +213,14 @@ __device__ __forceinline__ void cl_store16(uint32_t a, const double *v, uint32_t
 __device__ __forceinline__ void cl_mb_init(uint32_t mb, int count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(mb), "r"(count) : "memory");
 }
-__device__ __forceinline__ void cl_mb_arrive(uint32_t mb) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(mb) : "memory");
+__device__ __forceinline__ void cl_mb_arrive_if(bool on, uint32_t mb) {
+    asm volatile("{\n.reg .pred p;\nsetp.ne.u32 p, %1, 0;\n@p mbarrier.arrive.shared::cta.b64 _, [%0];\n}" ::"r"(mb),
+                 "r"((unsigned)on) : "memory");
+}
+__device__ __forceinline__ void cl_mb_expect_if(bool on, uint32_t mb, int bytes) {
+    asm volatile(
+        "{\n.reg .pred p;\nsetp.ne.u32 p, %2, 0;\n@p mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n}" ::"r"(mb),
+        "r"(bytes), "r"((unsigned)on) : "memory");
 }
 __device__ __forceinline__ void cl_mb_expect(uint32_t mb, int bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb), "r"(bytes)
@@ -182,31 +254,17 @@ __device__ __noinline__ bool cl_wait_slow(uint32_t mb, unsigned parity, volatile
     }
 }
 
-// sum over slots k0 <= k < w of row m (matrix rows stored slot by slot, stride R); padding
-// has value 0 and the row's own column
-template <class T>
-__device__ __forceinline__ T cl_row_dot(const T *val, const unsigned short *col, int m, int R,
-                                        int k0, int w, const T *x, int nwin) {
-    T acc = 0;
-    for (int kb = k0; kb < w; kb += kClBatch) {
-        unsigned short c[kClBatch];
-        T v[kClBatch], xv[kClBatch];
-#pragma unroll
-        for (int j = 0; j < kClBatch; j++) {
-            const bool in = kb + j < w;
-            c[j] = in ? col[(kb + j) * R + m] : (unsigned short)0;
-            v[j] = in ? val[(kb + j) * R + m] : T(0);
-        }
-#pragma unroll
-        for (int j = 0; j < kClBatch; j++)
-            xv[j] = (kb + j < w && idx_ok((int)c[j], nwin)) ? x[c[j]] : T(0);
-#pragma unroll
-        for (int j = 0; j < kClBatch; j++) acc += v[j] * xv[j];
-    }
-    return acc;
-}
-
-// ---------------------------------------------------------------------------------------
+// At these sizes a step is a few dozen instructions per thread, each about 4-5 cycles after the
+// one before, so what counts is the number of instructions between the end of one wait and
+// the stores that end the next. A row's constants (its columns' addresses, values, 1 / a_ii,
+// its destinations' addresses) are therefore read into registers before the wait of the step
+// before it, so that only the gathers of z, f and the sum follow the wait; level constants
+// stay in registers, stores are predicated rather than branched around. One Gauss-Seidel
+// colour, exchange included: 0.59-0.80 us with each step's code in line and no read ahead,
+// 1.1-1.5 us as an interpreter of ops with all bodies in one loop, 0.40 us in this form
+// (FP64: 0.91-0.98 -> 0.63-0.75 us). All levels from 16,384 rows down, 2 Alg. 1 steps each,
+// 1.05M unknowns, FP32: 118 us per visit (8 per application); on one CTA the levels from
+// 4,096 rows down took 139-150 us (16 per application) and the level above 3.0 us per step.
 extern __shared__ __align__(16) unsigned char cl_dyn[];
 
 template <class T>
@@ -214,644 +272,734 @@ __global__ void __launch_bounds__(kClThreads, 1)
 k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
     constexpr bool F64 = sizeof(T) == 8;
     constexpr int NR = kClRanks;
-    __shared__ __align__(8) unsigned long long mbs[5];  // neighbours x 2, all CTAs x 2, image
-    __shared__ __align__(16) T red[2][NR][4];           // sums over the cluster: partials
-    __shared__ T sred[F64 ? 3 * kClThreads : 4 * kClWarps];
-    __shared__ T coef[4], lsum[4];
-    __shared__ T pqs[kClLevels + 1][kMaxKcycle];        // (p_i, A p_i) of every level
-    __shared__ int stops[kClLevels + 1][kMaxKcycle];    // Alg. 1 stopped at or before step i
-    __shared__ int gave_up_s, token, img_ok;
+    __shared__ __align__(8) unsigned long long mbs[5];   // neighbours x 2, all CTAs x 2, image
+    __shared__ __align__(16) T red[2][NR * kClWarps][2]; // sums over the cluster: the warps'
+    __shared__ T coef_s[4];
+    __shared__ T pqs[kClLevels + 1][kMaxKcycle];         // (p_i, A p_i) of every level; FP64:
+                                                         //   its reciprocal (0: not positive)
+    __shared__ int stops[kClLevels + 1][kMaxKcycle];     // Alg. 1 stopped at or before step i
+    __shared__ int gave_up_s, token;
     volatile int *gave_up = &gave_up_s;
     const ClLayout &y = a.y;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int rank;
     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
-    const uint32_t mb0 = cl_smem(mbs);
+    const uint32_t mb0 = cl_smem(mbs), dyn = cl_smem(cl_dyn);
     if (tid == 0) {
-        cl_mb_init(mb0, kClWarps);
-        cl_mb_init(mb0 + 8, kClWarps);
-        cl_mb_init(mb0 + 16, 1);
-        cl_mb_init(mb0 + 24, 1);
+        for (int k = 0; k < 4; k++) cl_mb_init(mb0 + 8 * k, kClWarps);
         cl_mb_init(mb0 + 32, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         gave_up_s = 0;
-        img_ok = 1;
         token = 0;
     }
     __syncthreads();
     if (tid == 0) {  // this CTA's constant image, one bulk copy
         cl_mb_expect(mb0 + 32, y.image_bytes);
         asm volatile(
-            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                cl_smem(cl_dyn)),
+            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dyn),
             "l"(a.image + (size_t)rank * y.image_bytes), "r"(y.image_bytes), "r"(mb0 + 32)
             : "memory");
     }
     cl_sync_all();  // every CTA's mbarriers are ready
-    if (tid == 0 && !cl_mb_try(mb0 + 32, 0) &&
-        !cl_wait_slow(mb0 + 32, 0, gave_up, a.err, kBarrierLimitNs))
-        img_ok = 0;
-    __syncthreads();
-    if (img_ok) (void)cl_mb_try(mb0 + 32, 0);  // complete: every thread acquires the copy
-    // an error of an earlier launch of this application, or no image: nothing to run (the
-    // copy in flight is waited for above; the CTAs leave together)
-    bool alive = img_ok && !(ld_volatile_int(a.err) & kErrTimeout);
-    if (!img_ok) {
+    bool alive = cl_mb_try(mb0 + 32, 0) || cl_wait_slow(mb0 + 32, 0, gave_up, a.err, kBarrierLimitNs);
+    if (!__syncthreads_and(alive)) {  // no image: the others give up at their first exchange
         cl_sync_all();
         return;
     }
+    // after an error of an earlier launch of this application the steps run without exchanges
+    alive = !(ld_volatile_int(a.err) & kErrTimeout);
     unsigned kn = 0, ka = 0;  // exchanges so far: neighbours, all CTAs
     int extra = a.extra;
     auto at = [&](int off) { return cl_dyn + off; };
+    const ClLev *lvs = (const ClLev *)at(y.levels);
+    auto vec = [&](int off) { return (T *)(cl_dyn + off); };
     const int npeer = ((const int *)at(y.peers))[0];
+    // a token for every neighbour: lane p of the last warp
+    const bool has_peer = warp == kClWarps - 1 && lane < npeer;
+    const int peer = has_peer ? ((const int *)at(y.peers))[1 + lane] : 0;
+    const uint32_t peer_tok = cl_map(cl_smem(&token), peer), peer_mb = cl_map(mb0, peer);
     long long tp0 = 0;
     const bool mark_on = a.tprof && rank == 0 && tid == 0;
     // profiling: cycles and count per (level, kind), summed here and added up at the end
     __shared__ unsigned prof_s[2][16 * (kClLevels + 2)];
-    if (mark_on)
+    if (mark_on) {
         for (int k = 0; k < 2 * 16 * (kClLevels + 2); k++) (&prof_s[0][0])[k] = 0;
-    auto mark = [&](int level, int kind) {
+        tp0 = clock64();
+    }
+    auto mark = [&](int slot_level, int kind) {
         if (!mark_on) return;
         const long long t1 = clock64();
-        const int slot = 16 * (level - y.tl) + kind;
+        const int slot = 16 * slot_level + kind;
         prof_s[0][slot] += (unsigned)(t1 - tp0);
         prof_s[1][slot] += 1;
         tp0 = t1;
     };
-    if (mark_on) tp0 = clock64();
-
-    // this CTA's arrivals of neighbour exchange kn (which receives `bytes` of rows) and the
-    // wait for everybody's
-    auto exchange = [&](int bytes) {
-        const uint32_t mb = mb0 + 8 * (kn & 1);
+    // this CTA's arrivals at mbarrier mb, which counts its warps and `bytes` of stores (the last
+    // warp, which seldom has rows, announces them)
+    auto arrive = [&](uint32_t mb, int bytes) {
         __syncwarp();
-        if (alive) {
-            if (lane == 0) {
-                if (warp == 0) {
-                    cl_mb_expect(mb, bytes + 4 * npeer + extra);
-                    extra = 0;
-                } else {
-                    cl_mb_arrive(mb);
-                }
-            }
-            if (warp == kClWarps - 1)
-                for (int p = lane; p < npeer; p += 32) {
-                    const int dst = ((const int *)at(y.peers))[1 + p];
-                    cl_store(cl_map(cl_smem(&token), dst), 0.f, cl_map(mb, dst));
-                }
-            if (!cl_mb_try(mb, (kn >> 1) & 1))
-                alive = cl_wait_slow(mb, (kn >> 1) & 1, gave_up, a.err, a.limit_ns);
-        }
+        const bool one = alive && lane == 0;
+        cl_mb_expect_if(one && warp == kClWarps - 1, mb, bytes + extra);
+        cl_mb_arrive_if(one && warp != kClWarps - 1, mb);
+        extra = 0;
+    };
+    auto wait = [&](uint32_t mb, unsigned k) {
+        if (alive && !cl_mb_try(mb, (k >> 1) & 1))
+            alive = cl_wait_slow(mb, (k >> 1) & 1, gave_up, a.err, a.limit_ns);
+    };
+    // neighbour exchange kn: this CTA's end of its stores; `bytes` of rows come in
+    auto arrive_n = [&](int bytes) {
+        const uint32_t par = 8 * (kn & 1);
+        cl_store_if(has_peer && alive, peer_tok, 0.f, peer_mb + par);
+        arrive(mb0 + par, bytes + 4 * npeer);
+    };
+    auto wait_n = [&]() {
+        wait(mb0 + 8 * (kn & 1), kn);
         kn++;
     };
-    // the wait of an exchange between all CTAs; thread 0 announces the bytes it receives
-    auto mb_all = [&]() { return mb0 + 16 + 8 * (ka & 1); };
-    auto wait_all = [&](int bytes) {
-        const uint32_t mb = mb_all();
-        if (alive) {
-            if (tid == 0) {
-                cl_mb_expect(mb, bytes + extra);
-                extra = 0;
-            }
-            if (!cl_mb_try(mb, (ka >> 1) & 1))
-                alive = cl_wait_slow(mb, (ka >> 1) & 1, gave_up, a.err, a.limit_ns);
-        }
+    auto mb_a = [&]() { return mb0 + 16 + 8 * (ka & 1); };
+    auto wait_a = [&]() {
+        wait(mb_a(), ka);
         ka++;
     };
-    // row j of a colour's own rows to the neighbours that hold it
-    auto push_row = [&](const ClLev &L, const ClColor &C, int j, uint32_t vec, T v) {
-        const ClPush *P = (const ClPush *)at(L.push) + C.push0;
-        const uint32_t mb = mb0 + 8 * (kn & 1);
-        for (int e = 0; e < C.npush; e++) {
-            const ClPush q = P[e];
-            if ((unsigned)(j - q.j0) < (unsigned)q.cnt && alive) {
-                const int dst = q.dst_color & 255;
-                cl_store(cl_map(vec + (uint32_t)sizeof(T) * (q.dli + j - q.j0), dst), v,
-                         cl_map(mb, dst));
-            }
-        }
-    };
-    // every own row of vector `off` (complete in this CTA) to the neighbours
-    auto push_all = [&](const ClLev &L, int off) {
-        const ClHead &H = *(const ClHead *)at(L.head);
-        const ClPush *P = (const ClPush *)at(L.push);
-        const T *v = (const T *)at(off);
-        const uint32_t vec = cl_smem(v), mb = mb0 + 8 * (kn & 1);
-        if (alive)
-            for (int e = warp; e < H.npush; e += kClWarps) {
-                const ClPush q = P[e];
-                const int dst = q.dst_color & 255;
-                const ClColor &C = ((const ClColor *)at(L.tab))[q.dst_color >> 8];
-                const T *src = v + C.li0 + q.j0;
-                const uint32_t to = cl_map(vec + (uint32_t)sizeof(T) * q.dli, dst),
-                               mbd = cl_map(mb, dst);
-                for (int j = lane; j < q.cnt; j += 32)
-                    cl_store(to + (uint32_t)sizeof(T) * j, src[j], mbd);
-            }
-    };
-    // Sums of v[0..nv) over the own rows' threads (warps [0, nact)) of this CTA (ALL = false)
-    // or of the cluster; coefs(s, c) turns the sums into coefficients, the same in every CTA.
-    // FP32: sums and coefficients in every thread; FP64 (scarce): one warp per sum, the
-    // coefficients by one thread.
-    auto reduce = [&](auto all_tag, T (&v)[3], int nv, int nact, auto coefs, T (&c)[2]) {
-        constexpr bool ALL = decltype(all_tag)::value;
-        nact = min(nact, kClWarps);
-        T s[3] = {T(0), T(0), T(0)};
-        if constexpr (!F64) {
-            if (warp < nact) {
-#pragma unroll
-                for (int k = 0; k < 3; k++)
-                    if (k < nv) {
-                        T x = v[k];
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-                        if (lane == 0) sred[4 * warp + k] = x;
-                    }
-            }
-            __syncthreads();
-            if constexpr (ALL) {
-                if (warp == 0 && lane < NR && alive) {
-                    float p[4] = {0.f, 0.f, 0.f, 0.f};
-                    for (int w2 = 0; w2 < nact; w2++)
-#pragma unroll
-                        for (int k = 0; k < 3; k++)
-                            if (k < nv) p[k] += sred[4 * w2 + k];
-                    const uint32_t mb = mb_all();
-                    asm volatile(
-                        "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.f32 [%0], {%1, %2, %3, %4}, [%5];" ::"r"(
-                            cl_map(cl_smem(&red[ka & 1][rank][0]), lane)),
-                        "f"(p[0]), "f"(p[1]), "f"(p[2]), "f"(p[3]), "r"(cl_map(mb, lane))
-                        : "memory");
-                }
-                const T(*part)[4] = red[ka & 1];
-                wait_all(NR * 16);
-#pragma unroll
-                for (int k = 0; k < 3; k++)
-                    if (k < nv) {
-                        T x = part[lane & (NR - 1)][k];
-#pragma unroll
-                        for (int o = NR / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-                        s[k] = x;
-                    }
-            } else {
-                for (int w2 = 0; w2 < nact; w2++)
-#pragma unroll
-                    for (int k = 0; k < 3; k++)
-                        if (k < nv) s[k] += sred[4 * w2 + k];
-                __syncthreads();  // sred is reused by the next reduction
-            }
-            coefs(s, c);
-        } else {
-            if (warp < nact)
-#pragma unroll
-                for (int k = 0; k < 3; k++)
-                    if (k < nv) sred[k * kClThreads + tid] = v[k];
-            __syncthreads();
-            if (warp < nv) {
-                T x = 0;
-                for (int j = lane; j < 32 * nact; j += 32) x += sred[warp * kClThreads + j];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-                if constexpr (ALL) {
-                    if (lane < NR && alive)
-                        cl_store(cl_map(cl_smem(&red[ka & 1][rank][warp]), lane), x,
-                                 cl_map(mb_all(), lane));
-                } else if (lane == 0) {
-                    lsum[warp] = x;
-                }
-            }
-            if constexpr (ALL) {
-                const T(*part)[4] = red[ka & 1];
-                wait_all(NR * 8 * nv);
-                if (warp == 0) {
-#pragma unroll
-                    for (int k = 0; k < 3; k++)
-                        if (k < nv) {
-                            T x = part[lane & (NR - 1)][k];
-#pragma unroll
-                            for (int o = NR / 2; o > 0; o >>= 1)
-                                x += __shfl_xor_sync(0xffffffffu, x, o);
-                            s[k] = x;
-                        }
-                }
-            } else {
-                __syncthreads();
-                if (warp == 0)
-                    for (int k = 0; k < nv; k++) s[k] = lsum[k];
-            }
-            if (tid == 0) {
-                T cc[2] = {T(0), T(0)};
-                coefs(s, cc);
-                coef[0] = cc[0];
-                coef[1] = cc[1];
-            }
-            __syncthreads();
-            c[0] = coef[0];
-            c[1] = coef[1];
-        }
-    };
-    
-    // alpha_i of Alg. 1 from the sums (p, q), (r, p), (r, r); c[1] = 1 if Alg. 1 has stopped
-    auto alpha_of = [&](int lv, int i) {
-        return [=](const T *s, T *c) {
-            const bool prev = i > 0 && (stops[lv][i - 1] || s[2] == T(0));
-            const bool stopped = prev || !(s[0] > T(0)) || !isfinite(s[0]);
-            c[0] = stopped ? T(0) : (T)ratio<T>((double)s[1], (double)s[0]);
-            c[1] = stopped ? T(1) : T(0);
-        };
-    };
 
-    // one colour of a Gauss-Seidel sweep
-    auto gs_colour = [&](const ClLev &L, int c, const T *f, T *z) {
-        const ClColor C = ((const ClColor *)at(L.tab))[c];
-        const int nwin = ((const ClHead *)at(L.head))->nwin;
-        const T *val = (const T *)at(L.val), *dinv = (const T *)at(L.dinv);
-        const unsigned short *col = (const unsigned short *)at(L.col);
-        const uint32_t vec = cl_smem(z);
-        for (int j = tid; j < C.cnt; j += kClThreads) {
-            const int li = C.li0 + j;
-            const T u = (f[li] - cl_row_dot(val, col, C.m0 + j, L.R, 1, L.w, z, nwin)) * dinv[li];
-            z[li] = u;
-            push_row(L, C, j, vec, u);
+    int lv = 0;                    // current swept level
+    unsigned long long steps = 0;  // Alg. 1 step of every swept level, 4 bits each
+    // the destinations as addresses: (place, mbarrier) of two, mapped once
+    for (int l = 0; l < y.nsp; l++) {
+        uint4 *d = (uint4 *)at(lvs[l].dst);
+        const int nown = ((const ClHead *)at(lvs[l].head))->nown;
+#pragma unroll 1
+        for (int m = tid; m < nown; m += kClThreads) {
+            uint4 q = d[m];
+            auto place = [&](unsigned &p, unsigned &b) {
+                if (p >> 31 || p == kClNone) return;  // further ones: stays as it is
+                b = cl_map(mb0, (int)(p >> 16));
+                p = cl_map(dyn, (int)(p >> 16)) + (p & 0xFFFFu);
+            };
+            place(q.x, q.y);
+            place(q.z, q.w);
+            d[m] = q;
         }
-        exchange(C.expect);
-        mark(L.level, OP_GS);
+    }
+    __syncthreads();
+    // ---- the level's constants ----------------------------------------------------------
+    // (in registers: every wait and store makes the compiler read shared memory again)
+    uint4 lt0{}, lt1{}, lt2{};  // ClLev: own, col, val, diag | dinv, dst, over, head | lg, ns, R, xchild
+    uint4 h0{}, h1{};           // ClHead: nown, nwin, expect_all, fexp | fc0, fcn, fs0, fs1
+    uint32_t lvb = cl_smem(lvs);  // its ClLev
+    auto bind = [&](int l) {
+        lvb = cl_smem(&lvs[l]);
+        lt0 = cl_ld<uint4>(lvb);
+        lt1 = cl_ld<uint4>(lvb + 16);
+        lt2 = cl_ld<uint4>(lvb + 32);
+        h0 = cl_ld<uint4>(dyn + lt1.w);
+        h1 = cl_ld<uint4>(dyn + lt1.w + 16);
+    };
+    auto field = [&](size_t off) { return cl_ld<int>(lvb + (uint32_t)off); };
+#define CL_F(name) field(offsetof(ClLev, name))
+    auto p_off = [&](int i) { return field(offsetof(ClLev, p) + 4 * i); };
+    auto q_off = [&](int i) { return field(offsetof(ClLev, q) + 4 * i); };
+    // ---- a row's constants ------------------------------------------------------------
+    int mi = 0;                        // own row
+    uint32_t lb = 0;                   // its byte offset in a window vector
+    uint32_t d0 = 0, d1 = 0;           // its place in two strips' windows,
+    uint32_t m0 = 0, m1 = 0;           //   their mbarriers of the exchange it is sent in
+    bool to0 = false, to1 = false;     //   if any
+    unsigned more = 0;                 // further ones: bit 31 and their list
+    bool has = false, own = false;     // this lane has a row; is the one that stores it
+    T dinv = 0, dg = 0, v[kClSlots];
+    uint32_t za[kClSlots];             // addresses of its columns in z
+#pragma unroll
+    for (int k = 0; k < kClSlots; k++) {
+        v[k] = T(0);
+        za[k] = dyn;
+    }
+    // destinations of own row m (if on) for the vector at `off`, in neighbour exchange kx
+    auto load_dst = [&](bool on, int m, int off, unsigned kx) {
+        const uint4 q = cl_ld<uint4>(dyn + lt1.y + 16 * m);
+        const uint32_t par = 8 * (kx & 1);
+        on = on && alive;
+        to0 = on && q.x != kClNone;
+        to1 = on && (int)q.z >= 0 && q.z != kClNone;
+        more = on && q.z >> 31 ? q.z : 0;
+        d0 = q.x + (uint32_t)off;
+        m0 = q.y + par;
+        d1 = q.z + (uint32_t)off;
+        m1 = q.w + par;
+    };
+    // row vr of rows [vr0, vr0 + cnt) (times lanes per row): this thread's; its products are
+    // with the vector at zoff, its new value goes to the one at doff in exchange kx. A lane
+    // without a row takes row 0 and stores nothing: no branches
+    auto load_row = [&](int vr0, int vr, int cnt, int zoff, int doff, unsigned kx) {
+        has = vr < cnt;
+        const int o = has ? vr0 + vr : 0, m = o >> lt2.x;
+        mi = m;
+        own = has && (o & ((1 << lt2.x) - 1)) == 0;
+        lb = cl_ld<unsigned short>(dyn + lt0.x + 2 * m);
+        const uint4 c = cl_ld<uint4>(dyn + lt0.y + 16 * o);
+        dg = cl_ld<T>(dyn + lt0.w + (int)sizeof(T) * m);
+        if constexpr (!F64) {
+            const float4 x0 = cl_ld<float4>(dyn + lt0.z + 16 * o),
+                         x1 = cl_ld<float4>(dyn + lt0.z + 16 * ((int)lt2.z + o));
+            v[0] = x0.x; v[1] = x0.y; v[2] = x0.z; v[3] = x0.w;
+            v[4] = x1.x; v[5] = x1.y; v[6] = x1.z; v[7] = x1.w;
+        } else {
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (2 * k < (int)lt2.y) {
+                    const double2 x = cl_ld<double2>(dyn + lt0.z + 16 * (k * (int)lt2.z + o));
+                    v[2 * k] = x.x;
+                    v[2 * k + 1] = x.y;
+                }
+        }
+        const unsigned cw[4] = {c.x, c.y, c.z, c.w};
+        const uint32_t zb = dyn + zoff;
+#pragma unroll
+        for (int k = 0; k < kClSlots; k++) za[k] = zb + ((k & 1) ? cw[k / 2] >> 16 : cw[k / 2] & 0xFFFFu);
+        dinv = cl_ld<T>(dyn + lt1.x + (int)sizeof(T) * m);
+        load_dst(own, m, doff, kx);
+    };
+    // off-diagonal part of the row's product with z, over its lanes
+    auto gather = [&](int k) {
+#ifdef AMG_BOUNDS_CHECK
+        if (!idx_ok((int)(za[k] - dyn), y.bytes)) return T(0);
+#endif
+        return cl_ld<T>(za[k]);
+    };
+    auto row_dot = [&]() {
+        T acc;
+        if constexpr (!F64) {
+            T x[kClSlots];
+#pragma unroll
+            for (int k = 0; k < kClSlots; k++) x[k] = gather(k);
+            T s0 = v[0] * x[0], s1 = v[1] * x[1];
+#pragma unroll
+            for (int k = 2; k < kClSlots; k += 2) {
+                s0 += v[k] * x[k];
+                s1 += v[k + 1] * x[k + 1];
+            }
+            acc = s0 + s1;
+        } else {
+            // one FP64 instruction of a warp takes 64 cycles whatever its lanes do: no more of
+            // them than the level's slots need
+            acc = T(0);
+            auto part = [&](auto k0, auto k1) {
+                T x[kClSlots];
+#pragma unroll
+                for (int k = decltype(k0)::value; k < decltype(k1)::value; k++) x[k] = gather(k);
+#pragma unroll
+                for (int k = decltype(k0)::value; k < decltype(k1)::value; k++)
+                    acc = k == 0 ? v[0] * x[0] : acc + v[k] * x[k];
+            };
+            using std::integral_constant;
+            if (lt2.y > 4) part(integral_constant<int, 0>{}, integral_constant<int, 8>{});
+            else if (lt2.y > 2) part(integral_constant<int, 0>{}, integral_constant<int, 4>{});
+            else part(integral_constant<int, 0>{}, integral_constant<int, 2>{});
+        }
+        if (lt2.x > 0) {
+            acc += __shfl_xor_sync(0xffffffffu, acc, 1);
+            if (lt2.x > 1) acc += __shfl_xor_sync(0xffffffffu, acc, 2);
+        }
+        return acc;
+    };
+    // the row's new value to the strips that hold the row
+    auto push = [&](int off, T u) {
+        cl_store_if(to0, d0, u, m0);
+        cl_store_if(to1, d1, u, m1);
+        if (more) {
+            const uint32_t par = 8 * (kn & 1);
+            const unsigned *list = (const unsigned *)at(lt1.z) + (more & 0x7FFFFFFFu);
+#pragma unroll 1
+            for (unsigned d = *list; d != kClNone; d = *++list)
+                cl_store(cl_map(dyn + off + (d & 0xFFFFu), (int)(d >> 16)), u,
+                         cl_map(mb0 + par, (int)(d >> 16)));
+        }
     };
     // z = 0 on the window, except the colour whose values come next
-    auto zero_window = [&](const ClLev &L, T *z) {
-        const ClColor &C = ((const ClColor *)at(L.tab))[L.c_first];
-        const int nwin = ((const ClHead *)at(L.head))->nwin;
-        const int s0 = C.seg0, s1 = C.seg0 + C.seglen;
-        for (int i = tid; i < nwin; i += kClThreads)
-            if (i < s0 || i >= s1) z[i] = T(0);
+    auto zero_window = [&](uint32_t z) {  // of the level bound
+#pragma unroll 1
+        for (unsigned k = tid; k < h0.y; k += kClThreads)
+            if (k < h1.z || k >= h1.w) cl_st(z + (uint32_t)sizeof(T) * k, T(0));
     };
-
-    // ---- entry: this strip's rows of the right-hand side -------------------------------
-    if (y.nsp > 0) {
-        const ClLev &L = y.lv[0];
-        const ClColor *tab = (const ClColor *)at(L.tab);
-        T *rhs = (T *)at(L.rhs), *z = (T *)at(L.p[0]);
-        for (int c = 0; c < L.ncol; c++)
-            for (int j = tid; j < tab[c].cnt; j += kClThreads)
-                rhs[tab[c].li0 + j] = __ldcg(&a.rhs[tab[c].g0 + j]);
-        zero_window(L, z);
-        __syncthreads();
-        const ClColor C = tab[L.c_first];
-        const T *dinv = (const T *)at(L.dinv);
-        const uint32_t vec = cl_smem(z);
-        for (int j = tid; j < C.cnt; j += kClThreads) {
-            const T u = rhs[C.li0 + j] * dinv[C.li0 + j];
-            z[C.li0 + j] = u;
-            push_row(L, C, j, vec, u);
+    // Gauss-Seidel sweeps over n colours; the first one's rows are loaded already. The rows of
+    // the step after the sweep (all own rows of the level; sent, if at all, to the vector at
+    // next_off in the next exchange) are loaded before its last wait.
+    auto sweep = [&](int ops, int n, int foff, int zoff, int next_cnt, int next_off) {
+        const uint32_t z = dyn + zoff, f = dyn + foff;
+        uint4 op = cl_ld<uint4>(dyn + ops);  // a ClOp
+#pragma unroll 1
+        for (int k = 0; k < n; k++) {
+            auto relax = [&] {
+                const T fi = cl_ld<T>(f + (uint32_t)sizeof(T) * mi);
+                const T u = (fi - row_dot()) * dinv;
+                push(zoff, u);
+                cl_st_if(own, z + lb, u);
+            };
+            // (a warp without rows goes on at once)
+            if (32 * warp < (int)op.y) relax();
+#pragma unroll 1
+            for (int c = kClThreads; c < (int)op.y; c += kClThreads) {  // strips of large levels
+                load_row(op.x, c + tid, op.y, zoff, zoff, kn);
+                if (c + 32 * warp < (int)op.y) relax();
+            }
+            arrive_n(op.z);
+            if (k + 1 < n) {
+                op = cl_ld<uint4>(dyn + ops + 16 * (k + 1));
+                load_row(op.x, tid, op.y, zoff, zoff, kn + 1);
+            } else {
+                load_row(0, tid, next_cnt, zoff, next_off, kn + 1);
+            }
+            wait_n();
+            mark(lv, OP_GS);
         }
-        exchange(C.expect);
-        mark(L.level, OP_GS_FIRST);
+    };
+    // Sums of s0 and s1 over the cluster, then the coefficient f(sums) in every thread. Lanes 0-15
+    // end with the first sum, 16-31 with the second (one add per step for both); every warp
+    // sends its sums to every CTA. FP32: every warp adds them up; FP64 (scarce): warp 0, and
+    // warp 1 beside it for what only later steps read (g).
+    auto half_sum = [&](T x, T y) {
+        const bool hi = lane >= 16;
+        T k = hi ? y : x;
+        const T other = hi ? x : y;
+        k += __shfl_xor_sync(0xffffffffu, other, 16);
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+        return k;
+    };
+    auto cluster_sum = [&](T s0, T s1, int nact, auto before_wait, auto f, auto g) {
+        const uint32_t mb = mb_a(), part = cl_smem(&red[ka & 1][0][0]);
+        if (warp < nact) {
+            const T k = half_sum(s0, s1);
+            if (alive)
+                cl_store(cl_map(part + (uint32_t)sizeof(T) * (2 * (rank * nact + warp) + (lane >> 4)), lane & (NR - 1)),
+                         k, cl_map(mb, lane & (NR - 1)));
+        }
+        arrive(mb, NR * nact * 2 * (int)sizeof(T));
+        before_wait();
+        wait_a();
+        T c = 0;
+        if (!F64 || warp < 2) {
+            const uint32_t mine = part + (uint32_t)sizeof(T) * (2 * (lane & (NR - 1)) * nact + (lane >> 4));
+            T k = cl_ld<T>(mine);
+#pragma unroll 1
+            for (int w2 = 1; w2 < nact; w2++) k += cl_ld<T>(mine + 2 * (uint32_t)sizeof(T) * w2);
+#pragma unroll
+            for (int o = 8; o > 0; o >>= 1) k += __shfl_xor_sync(0xffffffffu, k, o);
+            const T other = __shfl_xor_sync(0xffffffffu, k, 16);
+            s0 = lane < 16 ? k : other;
+            s1 = lane < 16 ? other : k;
+            if constexpr (!F64) {
+                c = f(s0, s1);
+                g(s0);
+            } else if (warp == 0) {
+                c = f(s0, s1);
+                if (lane == 0) coef_s[0] = c;
+            } else {
+                g(s0);
+            }
+        }
+        if constexpr (F64) {
+            __syncthreads();
+            c = coef_s[0];
+        }
+        return c;
+    };
+    // positive and finite (FP64 without FP64 comparisons)
+    auto positive = [](T x) {
+        if constexpr (F64) return (unsigned long long)__double_as_longlong(x) - 1 < 0x7FEFFFFFFFFFFFFFull;
+        else return x > T(0) && isfinite(x);
+    };
+    // Alg. 1 on level slot lv: alpha_i from (p_i, q_i) and (r_i, p_i), 0 once it has stopped (a
+    // zero residual stops it here too: its p_i and q_i are zero); what step i leaves to later
+    // ones; beta_ij from (z, q_j)
+    auto alpha = [&](int lv, int i, T pq, T rp) {
+        const bool stopped = (i > 0 && stops[lv][i - 1]) || !positive(pq);
+        if (tid == 0) stops[lv][i] = stopped;
+        return stopped ? T(0) : (T)ratio<T>((double)rp, (double)pq);
+    };
+    auto keep_pq = [&](int lv, int i, T pq) {
+        T k = pq;
+        if constexpr (F64) k = positive(pq) ? T(1) / pq : T(0);  // off the path to the next step
+        if (tid == (F64 ? 32 : 0)) pqs[lv][i] = k;
+    };
+    auto beta = [&](int lv, int j, T zq) {
+        const T k = pqs[lv][j];
+        if constexpr (F64) return -(zq * k);
+        else return k > T(0) ? -(T)ratio<T>((double)zq, (double)k) : T(0);
+    };
+    auto nothing = [] {};
+    auto no_pq = [](T) {};
+
+    // ---- entry ---------------------------------------------------------------------------
+    {  // dense level's right-hand side: zero beyond its rows
+        T *F = vec(y.F);
+#pragma unroll 1
+        for (int k = tid; k < NR * y.ch; k += kClThreads)
+            F[k] = (y.nsp == 0 && k < y.nd) ? __ldcg(&a.rhs[k]) : T(0);
     }
-    {  // dense level's vectors: zero beyond its rows
-        T *F = (T *)at(y.F);
-        for (int i = tid; i < NR * y.ch; i += kClThreads)
-            F[i] = (y.nsp == 0 && i < y.nd) ? __ldcg(&a.rhs[i]) : T(0);
+    // the first colour of a sweep from zero: own row m, right-hand side x (z zeroed before)
+    auto first_colour = [&](int m, int zoff, T x) {
+        if ((unsigned)(m - (int)h1.x) < h1.y) {
+            const T u = x * cl_ld<T>(dyn + lt1.x + (uint32_t)sizeof(T) * m);
+            lb = cl_ld<unsigned short>(dyn + lt0.x + 2 * m);
+            load_dst(true, m, zoff, kn);
+            push(zoff, u);
+            cl_st(dyn + zoff + lb, u);
+        }
+    };
+    // its exchange; the sweep's next colour (or all rows) is loaded before the wait
+    auto first_exchange = [&](int zoff, int qoff) {
+        arrive_n((int)h0.w);
+        const int npre = CL_F(npre);
+        const uint4 op = cl_ld<uint4>(dyn + CL_F(pre));
+        load_row(npre ? op.x : 0, tid, npre ? op.y : h0.x << lt2.x, zoff, npre ? zoff : qoff, kn + 1);
+        wait_n();
+    };
+    if (y.nsp > 0) {  // this strip's rows of the right-hand side, and their first colour
+        bind(0);
+        const int zoff = p_off(0), roff = CL_F(rhs);
+        zero_window(dyn + zoff);
+#pragma unroll 1
+        for (int m = tid; m < (int)h0.x; m += kClThreads) {
+            const T x = __ldcg(&a.rhs[((const int *)at(y.top))[m]]);
+            vec(roff)[m] = x;
+            first_colour(m, zoff, x);
+        }
+        first_exchange(zoff, q_off(0));
+        mark(0, OP_GS_FIRST);
     }
     __syncthreads();
 
     // ---- Alg. 2 / Alg. 1 over the levels ------------------------------------------------
-    int lv = 0;            // current swept level
-    unsigned long long steps = 0;  // Alg. 1 step of every swept level, 4 bits each
     for (;;) {
         if (y.nsp > 0) {  // B^ of level lv for step i: pre-smoothing, then the restriction
-            const ClLev &L = y.lv[lv];
             const int i = (int)(steps >> (4 * lv)) & 15;
-            const T *f = (const T *)at(i == 0 ? L.rhs : L.r);
-            T *z = (T *)at(L.p[i]);
-            for (int sw = 0; sw < y.nu_pre; sw++)
-                for (int c = sw == 0 ? L.c_first + 1 : 0; c < L.ncol; c++)
-                    if (L.cmask >> c & 1) gs_colour(L, c, f, z);
-            const ClHead H = *(const ClHead *)at(L.head);
+            const int foff = i == 0 ? CL_F(rhs) : CL_F(r), zoff = p_off(i), toff = q_off(i);
+            const int rows = (int)(h0.x << lt2.x), npre = CL_F(npre);
+            if (npre > 0) sweep(CL_F(pre), npre, foff, zoff, rows, toff);
             const bool to_swept = lv + 1 < y.nsp;
-            T *t = (T *)at(L.q[i]);  // free until step i's product writes it
-            {
-                const unsigned short *own = (const unsigned short *)at(L.own);
-                const T *val = (const T *)at(L.val);
-                const unsigned short *col = (const unsigned short *)at(L.col);
-                for (int m = tid; m < H.nown; m += kClThreads) {
-                    const int li = own[m];
-                    t[li] = f[li] - cl_row_dot(val, col, m, L.R, 0, L.w, z, H.nwin);
+            const int child = CL_F(child), nch = CL_F(nch), Rn = CL_F(Rn);
+            const bool xchild = lt2.w != 0;
+            // t = f - A z into q_i (free until step i's product)
+#pragma unroll 1
+            for (int c = 0;;) {
+                if (c + 32 * warp < rows) {
+                    const T fi = cl_ld<T>(dyn + foff + (uint32_t)sizeof(T) * mi), zi = cl_ld<T>(dyn + zoff + lb);
+                    const T u = fi - (row_dot() + dg * zi);
+                    if (xchild) push(toff, u);
+                    cl_st_if(own, dyn + toff + lb, u);
                 }
-                if (to_swept) zero_window(y.lv[lv + 1], (T *)at(y.lv[lv + 1].p[0]));
+                c += kClThreads;
+                if (c >= rows) break;
+                load_row(0, c + tid, rows, zoff, toff, kn);
             }
-            __syncthreads();
-            if (L.xchild) {
-                push_all(L, L.q[i]);
-                exchange(H.expect_all);
-            }
-            mark(L.level, OP_RESID);
-            const unsigned short *child = (const unsigned short *)at(L.child);
-            auto child_sum = [&](int m) {
-                T v[8];
-#pragma unroll
-                for (int q = 0; q < 8; q++) {
-                    const int ci = q < L.nch ? child[q * L.Rn + m] : 0xFFFF;
-                    v[q] = (ci != 0xFFFF && idx_ok(ci, H.nwin)) ? t[ci] : T(0);
-                }
-                const T lo = (v[0] + v[1]) + (v[2] + v[3]);
-                return L.nch == 8 ? lo + ((v[4] + v[5]) + (v[6] + v[7])) : lo;
-            };
+            const int nwin = (int)h0.y;
+            if (xchild) arrive_n((int)h0.z);
+            int zn = 0;
             if (to_swept) {
-                const ClLev &N = y.lv[lv + 1];
-                const int nown = ((const ClHead *)at(N.head))->nown;
-                const unsigned short *own = (const unsigned short *)at(N.own);
-                const ClColor C = ((const ClColor *)at(N.tab))[N.c_first];
-                const T *dinv = (const T *)at(N.dinv);
-                T *rhs = (T *)at(N.rhs), *zn = (T *)at(N.p[0]);
-                const uint32_t vec = cl_smem(zn);
-                for (int m = tid; m < nown; m += kClThreads) {
-                    const int li = own[m];
-                    const T v = child_sum(m);
-                    rhs[li] = v;
-                    const int j = m - C.m0;
-                    if ((unsigned)j < (unsigned)C.cnt) {
-                        const T u = v * dinv[li];
-                        zn[li] = u;
-                        push_row(N, C, j, vec, u);
-                    }
+                bind(lv + 1);
+                zn = p_off(0);
+                zero_window(dyn + zn);
+            }
+            // (the zeros too are complete before the next level's rows come in: the stores
+            // of its first colour leave them out, those of later colours wait for this CTA's)
+            if (xchild) wait_n();
+            __syncthreads();
+            mark(lv, OP_RESID);
+            const uint32_t t = dyn + toff;
+            auto child_sum = [&](int m) {
+                T w[2] = {T(0), T(0)};
+#pragma unroll
+                for (int h = 0; h < 2; h++) {
+                    if (h == 1 && nch == 4) break;
+                    const uint2 c = cl_ld<uint2>(dyn + child + 8 * (h * Rn + m));
+                    const unsigned ci[4] = {c.x & 0xFFFFu, c.x >> 16, c.y & 0xFFFFu, c.y >> 16};
+                    T x[4];
+#pragma unroll
+                    for (int q = 0; q < 4; q++)
+                        x[q] = (ci[q] != 0xFFFFu && idx_ok((int)ci[q], nwin))
+                                   ? cl_ld<T>(t + (uint32_t)sizeof(T) * ci[q]) : T(0);
+                    w[h] = (x[0] + x[1]) + (x[2] + x[3]);
                 }
-                exchange(C.expect);
-                mark(L.level, OP_RESTRICT);
+                return w[0] + w[1];
+            };
+            if (to_swept) {  // its right-hand side and first colour
+                const uint32_t rn = dyn + CL_F(rhs);
+#pragma unroll 1
+                for (int m = tid; m < (int)h0.x; m += kClThreads) {
+                    const T x = child_sum(m);
+                    cl_st(rn + (uint32_t)sizeof(T) * m, x);
+                    first_colour(m, zn, x);
+                }
+                first_exchange(zn, q_off(0));
+                mark(lv, OP_RESTRICT);
                 lv++;
                 steps &= ~(15ull << (4 * lv));
                 continue;
             }
             // into the dense level: every CTA gets every row
             const int nown = *(const int *)at(y.dhead);
-            T *stage = (T *)at(y.stage);
+            T *stage = vec(y.stage);
+#pragma unroll 1
             for (int m = tid; m < nown; m += kClThreads) stage[m] = child_sum(m);
             __syncthreads();
-            if (alive) {
-                const unsigned short *pi = (const unsigned short *)at(y.down);
-                const uint32_t vec = cl_smem(at(y.F)), mb = mb_all();
+            const unsigned short *pi = (const unsigned short *)at(y.down);
+            const uint32_t to = dyn + y.F, mb = mb_a();
+            if (alive)
+#pragma unroll 1
                 for (int k = tid; k < NR * nown; k += kClThreads)
-                    cl_store(cl_map(vec + (uint32_t)sizeof(T) * pi[k >> 4], k & (NR - 1)), stage[k >> 4],
+                    cl_store(cl_map(to + (uint32_t)sizeof(T) * pi[k >> 4], k & (NR - 1)), stage[k >> 4],
                              cl_map(mb, k & (NR - 1)));
-            }
-            wait_all((int)sizeof(T) * y.nd);
-            mark(L.level, OP_RESTRICT);
+            arrive(mb, (int)sizeof(T) * y.nd);
+            wait_a();
+            mark(lv, OP_RESTRICT);
         }
-        // ---- the dense level: e = B~ [F] ------------------------------------------------
+        // ---- the dense level: E = B~ [F] ------------------------------------------------
         {
             const int ch = y.ch, len = NR * ch;
-            const int dl = y.tl + y.nsp;  // its level number
-            T *E = (T *)at(y.E), *out = (T *)at(y.out);
-            auto gather_out = [&](int dst0, int dst1, int parts) {  // `out` to every CTA
-                constexpr int V = 16 / (int)sizeof(T);
-                const int per = ch / V;  // 16-byte pieces per part
-                if (alive)
-                    for (int k = tid; k < NR * parts * per; k += kClThreads) {
-                        const int dst = k & (NR - 1), piece = k >> 4;
-                        const int part = piece >= per, o = (piece - part * per) * V;
-                        const uint32_t to = cl_smem(at(part ? dst1 : dst0)) +
-                                            (uint32_t)sizeof(T) * (rank * ch + o);
-                        cl_store16(cl_map(to, dst), out + part * ch + o, cl_map(mb_all(), dst));
-                    }
-                wait_all((int)sizeof(T) * parts * len);
-            };
+            T *E = vec(y.E), *out = vec(y.out), *Rv = vec(y.Rv);
+            const int nsteps = y.dense ? y.kc : 1, parts = y.dense ? 2 : 1;
             constexpr int LPR = 8;  // lanes per row
-            const int q = tid & (LPR - 1);
-            if (!y.dense) {  // coarsest level: e = A^{-1} F (FP32: op_coarse's compensated sum)
-                const T *F = (const T *)at(y.F);
-                for (int row = tid / LPR; row < ch; row += kClThreads / LPR) {
-                    const T *m = (const T *)at(y.mat) + (size_t)row * y.stride;
-                    if constexpr (!F64) {
-                        const T *ml = (const T *)at(y.mat_lo) + (size_t)row * y.stride;
-                        float s = 0.f, cs = 0.f;
+            constexpr int V = 16 / (int)sizeof(T);
+#pragma unroll 1
+            for (int st = 0; st < nsteps; st++) {
+                const T *r = st == 0 ? vec(y.F) : Rv;
+                const int q = tid & (LPR - 1);
+#pragma unroll 1
+                for (int row = tid / LPR; row < parts * ch; row += kClThreads / LPR) {
+                    const T *m = vec(y.mat) + (size_t)row * y.stride;
+                    T sum = 0, err = 0;
+                    if (F64 || y.dense) {  // [z; w] = [M; A M] r (or A^{-1} r): 16-byte reads
+#pragma unroll 8
+                        for (int j = q * V; j < len; j += LPR * V) {
+                            if constexpr (!F64) {
+                                const float4 mv = *(const float4 *)(m + j), xv = *(const float4 *)(r + j);
+                                sum += mv.x * xv.x;
+                                err += mv.y * xv.y;
+                                sum += mv.z * xv.z;
+                                err += mv.w * xv.w;
+                            } else {
+                                const double2 mv = *(const double2 *)(m + j), xv = *(const double2 *)(r + j);
+                                sum += mv.x * xv.x;
+                                err += mv.y * xv.y;
+                            }
+                        }
+                        sum += err;
+#pragma unroll
+                        for (int o = LPR / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+                    } else if constexpr (!F64) {  // A^{-1} r in FP32: op_coarse's compensated sum
+                        const T *ml = vec(y.mat_lo) + (size_t)row * y.stride;
+#pragma unroll 1
                         for (int j = q; j < y.nd; j += LPR) {
-                            const float x = F[j];
+                            const float x = r[j];
                             const float ph = __fmul_rn(m[j], x);
                             const float pe = fmaf(ml[j], x, fmaf(m[j], x, -ph));
                             float t2, e2;
-                            two_sum(s, ph, t2, e2);
-                            s = t2;
-                            cs = __fadd_rn(cs, __fadd_rn(e2, pe));
+                            two_sum(sum, ph, t2, e2);
+                            sum = t2;
+                            err = __fadd_rn(err, __fadd_rn(e2, pe));
                         }
 #pragma unroll
                         for (int o = LPR / 2; o > 0; o >>= 1) {
-                            const float so = __shfl_down_sync(0xffffffffu, s, o, LPR);
-                            const float co = __shfl_down_sync(0xffffffffu, cs, o, LPR);
+                            const float so = __shfl_xor_sync(0xffffffffu, sum, o);
+                            const float co = __shfl_xor_sync(0xffffffffu, err, o);
                             float t2, e2;
-                            two_sum(s, so, t2, e2);
-                            s = t2;
-                            cs = __fadd_rn(cs, __fadd_rn(co, e2));
+                            two_sum(sum, so, t2, e2);
+                            sum = t2;
+                            err = __fadd_rn(err, __fadd_rn(co, e2));
                         }
-                        if (q == 0) out[row] = __fadd_rn(s, cs);
-                    } else {
-                        double s = 0.0;
-                        for (int j = q; j < y.nd; j += LPR) s += m[j] * F[j];
-#pragma unroll
-                        for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, LPR);
-                        if (q == 0) out[row] = s;
+                        sum = __fadd_rn(sum, err);
                     }
+                    if (q == 0) out[row] = sum;
                 }
                 __syncthreads();
-                gather_out(y.E, y.E, 1);
-                mark(dl, OP_COARSE);
-            } else {
-                T *Rv = (T *)at(y.Rv);
-                const int nact = (y.nd + 31) / 32;
-                for (int i = 0; i < y.kc; i++) {
-                    // [z; w] = [M; A M] r: this CTA's rows, 16-byte reads
-                    const T *x = (const T *)at(i == 0 ? y.F : y.Rv);
-                    constexpr int V = 16 / (int)sizeof(T);
-                    for (int row = tid / LPR; row < 2 * ch; row += kClThreads / LPR) {
-                        const T *m = (const T *)at(y.mat) + (size_t)row * y.stride;
-                        T s = 0;
-                        for (int j = q * V; j < len; j += LPR * V) {
-                            if constexpr (!F64) {
-                                const float4 mv = *(const float4 *)(m + j), xv = *(const float4 *)(x + j);
-                                s += mv.x * xv.x;
-                                s += mv.y * xv.y;
-                                s += mv.z * xv.z;
-                                s += mv.w * xv.w;
-                            } else {
-                                const double2 mv = *(const double2 *)(m + j), xv = *(const double2 *)(x + j);
-                                s += mv.x * xv.x;
-                                s += mv.y * xv.y;
-                            }
+                {  // this CTA's part of the product to every CTA
+                    const uint32_t mb = mb_a();
+                    const int per = ch / V, o0 = y.dense ? y.P[st] : y.E, o1 = y.Q[st];
+                    if (alive)
+#pragma unroll 1
+                        for (int k = tid; k < NR * parts * per; k += kClThreads) {
+                            const int piece = k >> 4, part = piece >= per, o = (piece - part * per) * V;
+                            const uint32_t to = dyn + (part ? o1 : o0) + (uint32_t)sizeof(T) * (rank * ch + o);
+                            cl_store16(cl_map(to, k & (NR - 1)), out + part * ch + o, cl_map(mb, k & (NR - 1)));
                         }
+                    arrive(mb, (int)sizeof(T) * parts * len);
+                    wait_a();
+                }
+                if (!y.dense) break;
+                // Alg. 1 step st, the same in every CTA: beta_j for j < st, then alpha
+                T *p = vec(y.P[st]), *w = vec(y.Q[st]);
+                const bool last = st == y.kc - 1;
+#pragma unroll 1
+                for (int j = 0; j <= st; j++) {
+                    const T *qj = vec(y.Q[j]), *pj = vec(y.P[j]);
+                    T c = 0;
+                    if constexpr (!F64) {  // every warp sums all rows: no barrier
+                        T s0 = 0, s1 = 0;
+#pragma unroll 2
+                        for (int k = 4 * lane; k < len; k += 128) {
+                            const float4 pv = *(const float4 *)(p + k), qv = *(const float4 *)(qj + k),
+                                         rv = *(const float4 *)(r + k);
+                            s0 += pv.x * qv.x; s1 += pv.x * rv.x;
+                            s0 += pv.y * qv.y; s1 += pv.y * rv.y;
+                            s0 += pv.z * qv.z; s1 += pv.z * rv.z;
+                            s0 += pv.w * qv.w; s1 += pv.w * rv.w;
+                        }
+                        const T k = half_sum(s0, s1), other = __shfl_xor_sync(0xffffffffu, k, 16);
+                        s0 = lane < 16 ? k : other;
+                        s1 = lane < 16 ? other : k;
+                        if (j < st) {
+                            c = beta(kClLevels, j, s0);
+                        } else {
+                            c = alpha(kClLevels, st, s0, s1);
+                            keep_pq(kClLevels, st, s0);
+                        }
+                        __syncthreads();  // every warp has read what changes now
+                    } else {  // warp k sums value k; one thread each for the coefficients
+                        if (warp < 2) {
+                            const T *u1 = warp == 0 ? qj : r;
+                            T x = 0;
+#pragma unroll 4
+                            for (int k = lane; k < len; k += 32) x += p[k] * u1[k];
 #pragma unroll
-                        for (int o = LPR / 2; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o, LPR);
-                        if (q == 0) out[row] = s;
+                            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                            if (lane == 0) coef_s[1 + warp] = x;
+                        }
+                        __syncthreads();
+                        if (tid == 0)
+                            coef_s[0] = j < st ? beta(kClLevels, j, coef_s[1])
+                                               : alpha(kClLevels, st, coef_s[1], coef_s[2]);
+                        else if (tid == 32 && j == st)
+                            keep_pq(kClLevels, st, coef_s[1]);
+                        __syncthreads();
+                        c = coef_s[0];
                     }
-                    __syncthreads();
-                    gather_out(y.P[i], y.Q[i], 2);
-                    // Alg. 1 step i, the same in every CTA
-                    T *p = (T *)at(y.P[i]), *qv = (T *)at(y.Q[i]);
-                    const T *r = x;
-                    T c[2];
-                    if (i > 0) {
-                        T v[3] = {T(0), T(0), T(0)};
-                        for (int k = tid; k < y.nd; k += kClThreads)
-#pragma unroll
-                            for (int j = 0; j < 3; j++)
-                                if (j < i) v[j] += p[k] * ((const T *)at(y.Q[j]))[k];
-                        for (int j = 0; j < i; j++) {  // one coefficient per sum
-                            T vj[3] = {j == 0 ? v[0] : j == 1 ? v[1] : v[2], T(0), T(0)};
-                            reduce(std::false_type{}, vj, 1, nact,
-                                   [&](const T *s, T *cc) {
-                                       const T pq = pqs[kClLevels][j];
-                                       cc[0] = pq > T(0) ? -(T)ratio<T>((double)s[0], (double)pq) : T(0);
-                                   },
-                                   c);
-                            const T *pj = (const T *)at(y.P[j]), *qj = (const T *)at(y.Q[j]);
-                            for (int k = tid; k < y.nd; k += kClThreads) {
-                                p[k] += c[0] * pj[k];
-                                qv[k] += c[0] * qj[k];
-                            }
+#pragma unroll 1
+                    for (int k = tid; k < len; k += kClThreads) {
+                        if (j < st) {
+                            p[k] += c * pj[k];
+                            w[k] += c * qj[k];
+                        } else {
+                            E[k] = st > 0 ? E[k] + c * p[k] : c * p[k];
+                            if (!last) Rv[k] = r[k] - c * w[k];
                         }
                     }
-                    T v[3] = {T(0), T(0), T(0)};
-                    for (int k = tid; k < y.nd; k += kClThreads) {
-                        v[0] += p[k] * qv[k];
-                        v[1] += r[k] * p[k];
-                        v[2] += r[k] * r[k];
-                    }
-                    auto f = alpha_of(kClLevels, i);
-                    reduce(std::false_type{}, v, 3, nact,
-                           [&](const T *s, T *cc) {
-                               f(s, cc);
-                               if (tid == 0) {
-                                   pqs[kClLevels][i] = s[0];
-                                   stops[kClLevels][i] = cc[1] != T(0);
-                               }
-                           },
-                           c);
-                    const T al = c[0];
-                    const bool last = i == y.kc - 1;
-                    for (int k = tid; k < y.nd; k += kClThreads) {
-                        E[k] = i == 0 ? al * p[k] : E[k] + al * p[k];
-                        if (!last) Rv[k] = r[k] - al * qv[k];
-                    }
-                    if (i == 0 && !last)
-                        for (int k = y.nd + tid; k < len; k += kClThreads) Rv[k] = T(0);
                     __syncthreads();
                 }
-                mark(dl, OP_COARSE);
             }
+            mark(y.nsp, OP_COARSE);
         }
         if (y.nsp == 0) break;
         // ---- back up: B^ of level lv after the correction, Alg. 1 step i ------------------
         bool done = false;
         for (;;) {
-            const ClLev &L = y.lv[lv];
             const int i = (int)(steps >> (4 * lv)) & 15;
-            const ClHead H = *(const ClHead *)at(L.head);
-            const ClColor *tab = (const ClColor *)at(L.tab);
-            const T *f = (const T *)at(i == 0 ? L.rhs : L.r);
-            T *z = (T *)at(L.p[i]);
-            {  // z += P e on the window; the colour swept next is overwritten unread
-                const bool from_swept = lv + 1 < y.nsp;
-                const T *en = (const T *)at(from_swept ? y.lv[lv + 1].e : y.E);
-                const unsigned short *par = (const unsigned short *)at(L.parent);
-                const int s0 = tab[L.c_last].seg0, s1 = s0 + tab[L.c_last].seglen;
-                for (int k = tid; k < H.nwin; k += kClThreads)
-                    if (k < s0 || k >= s1) z[k] += en[par[k]];
-                __syncthreads();
-                mark(L.level, OP_PROLONG);
-            }
-            for (int sw = 0; sw < y.nu_post; sw++)
-                for (int c = L.c_last; c >= 0; c--)
-                    if (L.cmask >> c & 1) gs_colour(L, c, f, z);
-            const unsigned short *own = (const unsigned short *)at(L.own);
-            const int nact = (H.nown + 31) / 32;
+            const int foff = i == 0 ? CL_F(rhs) : CL_F(r), zoff = p_off(i), qoff = q_off(i);
+            const int post = CL_F(post), npost = CL_F(npost), nact = CL_F(nact), eoff = CL_F(e);
+            const int rows = (int)(h0.x << lt2.x), nwin = (int)h0.y;
             const bool last = i == y.kc - 1;
-            T c[2];
-            if (i > 0) {  // p_i = z + sum_j beta_j p_j, on the window
-                T v[3] = {T(0), T(0), T(0)};
-                for (int m = tid; m < H.nown; m += kClThreads) {
-                    const int li = own[m];
-                    const T zl = z[li];
-#pragma unroll
-                    for (int j = 0; j < 3; j++)
-                        if (j < i) v[j] += zl * ((const T *)at(L.q[j]))[li];
+            const uint32_t z = dyn + zoff;
+            {  // z += P e on the window; the colour swept next is overwritten unread
+                const uint4 op = cl_ld<uint4>(dyn + post);
+                load_row(op.x, tid, op.y, zoff, zoff, kn);
+                const uint32_t en = dyn + (lv + 1 < y.nsp ? cl_ld<int>(lvb + (uint32_t)(sizeof(ClLev) + offsetof(ClLev, e)))
+                                                          : y.E);
+                const uint32_t par = dyn + CL_F(parent);
+                const uint2 ls = cl_ld<uint2>(dyn + lt1.w + 32);
+#pragma unroll 1
+                for (unsigned k = tid; k < (unsigned)nwin; k += kClThreads)
+                    if (k < ls.x || k >= ls.y) {
+                        const uint32_t zk = z + (uint32_t)sizeof(T) * k;
+                        cl_st(zk, cl_ld<T>(zk) + cl_ld<T>(en + (uint32_t)sizeof(T) * cl_ld<unsigned short>(par + 2 * k)));
+                    }
+                __syncthreads();
+                mark(lv, OP_PROLONG);
+            }
+            sweep(post, npost, foff, zoff, rows, zoff);
+#pragma unroll 1
+            for (int j = 0; j < i; j++) {  // p_i = z + sum_j beta_j p_j, on the window
+                T zq = 0;
+                const uint32_t qj = dyn + q_off(j), pj = dyn + p_off(j);
+#pragma unroll 1
+                for (int m = tid; m < (int)h0.x; m += kClThreads) {
+                    const uint32_t l2 = cl_ld<unsigned short>(dyn + lt0.x + 2 * m);
+                    zq += cl_ld<T>(z + l2) * cl_ld<T>(qj + l2);
                 }
-                for (int j = 0; j < i; j++) {
-                    T vj[3] = {j == 0 ? v[0] : j == 1 ? v[1] : v[2], T(0), T(0)};
-                    reduce(std::true_type{}, vj, 1, nact,
-                           [&](const T *s, T *cc) {
-                               const T pq = pqs[lv][j];
-                               cc[0] = pq > T(0) ? -(T)ratio<T>((double)s[0], (double)pq) : T(0);
-                           },
-                           c);
-                    mark(L.level, OP_MULTIDOT);
-                    const T *pj = (const T *)at(L.p[j]);
-                    for (int k = tid; k < H.nwin; k += kClThreads) z[k] += c[0] * pj[k];
+                const T c = cluster_sum(zq, T(0), nact, nothing, [&](T x, T) { return beta(lv, j, x); }, no_pq);
+                mark(lv, OP_MULTIDOT);
+#pragma unroll 1
+                for (int k = tid; k < nwin; k += kClThreads) {
+                    const uint32_t o = (uint32_t)sizeof(T) * k;
+                    cl_st(z + o, cl_ld<T>(z + o) + c * cl_ld<T>(pj + o));
                 }
                 __syncthreads();
-                mark(L.level, OP_ORTH);
+                mark(lv, OP_ORTH);
             }
-            T *qv = (T *)at(L.q[i]);
-            {  // q = A p; (p, q), (r, p), (r, r)
-                const T *val = (const T *)at(L.val);
-                const unsigned short *col = (const unsigned short *)at(L.col);
-                T v[3] = {T(0), T(0), T(0)};
-                for (int m = tid; m < H.nown; m += kClThreads) {
-                    const int li = own[m];
-                    const T acc = cl_row_dot(val, col, m, L.R, 0, L.w, z, H.nwin);
-                    qv[li] = acc;
-                    const T pl = z[li], rl = f[li];
-                    v[0] += pl * acc;
-                    v[1] += rl * pl;
-                    v[2] += rl * rl;
+            // q = A p; (p, q), (r, p); the next step's z = 0
+            T pq = 0, rp = 0;
+#pragma unroll 1
+            for (int c = 0;;) {
+                if (c + 32 * warp < rows) {
+                    const T fi = cl_ld<T>(dyn + foff + (uint32_t)sizeof(T) * mi), zi = cl_ld<T>(z + lb);
+                    const T qi = row_dot() + dg * zi;
+                    cl_st_if(own, dyn + qoff + lb, qi);
+                    const T zo = own ? zi : T(0);
+                    pq += zo * qi;
+                    rp += fi * zo;
                 }
-                if (!last) zero_window(L, (T *)at(L.p[i + 1]));
-                auto fa = alpha_of(lv, i);
-                reduce(std::true_type{}, v, 3, nact,
-                       [&](const T *s, T *cc) {
-                           fa(s, cc);
-                           if (tid == 0) {
-                               pqs[lv][i] = s[0];
-                               stops[lv][i] = cc[1] != T(0);
-                           }
-                       },
-                       c);
-                mark(L.level, OP_SPMV_DOT);
+                c += kClThreads;
+                if (c >= rows) break;
+                load_row(0, c + tid, rows, zoff, zoff, kn);
             }
-            {  // e (+)= alpha p, r = r - alpha q; the next step's first colour
-                const T al = c[0];
-                T *e = (T *)at(L.e), *r = (T *)at(L.r);
-                const ClColor C = tab[L.c_first];
-                const T *dinv = (const T *)at(L.dinv);
-                T *zn = last ? nullptr : (T *)at(L.p[i + 1]);
-                const uint32_t vec = last ? 0 : cl_smem(zn);
-                for (int m = tid; m < H.nown; m += kClThreads) {
-                    const int li = own[m];
-                    e[li] = i == 0 ? al * z[li] : e[li] + al * z[li];
-                    if (!last) {
-                        const T rn = f[li] - al * qv[li];
-                        r[li] = rn;
-                        const int j = m - C.m0;
-                        if ((unsigned)j < (unsigned)C.cnt) {
-                            const T u = rn * dinv[li];
-                            zn[li] = u;
-                            push_row(L, C, j, vec, u);
-                        }
+            const int poff = last ? eoff : p_off(i + 1), roff = CL_F(r);
+            if (!last) zero_window(dyn + poff);
+            auto load_own = [&](int m) {  // offset, 1 / a_ii and destinations of own row m
+                if (m >= (int)h0.x) return;
+                lb = cl_ld<unsigned short>(dyn + lt0.x + 2 * m);
+                dinv = cl_ld<T>(dyn + lt1.x + (uint32_t)sizeof(T) * m);
+                load_dst(true, m, poff, kn);
+            };
+            const T al = cluster_sum(pq, rp, nact, [&] { load_own(tid); },
+                                     [&](T x, T y2) { return alpha(lv, i, x, y2); },
+                                     [&](T x) { keep_pq(lv, i, x); });
+            mark(lv, OP_SPMV_DOT);
+            // e (+)= alpha p, r = r - alpha q; the next step's first colour
+#pragma unroll 1
+            for (int m = tid; m < (int)h0.x;) {
+                const T zi = cl_ld<T>(z + lb);
+                T u = i > 0 ? cl_ld<T>(dyn + eoff + lb) + al * zi : al * zi;
+                cl_st(dyn + eoff + lb, u);
+                bool to = last && lv > 0;
+                if (!last) {
+                    const uint32_t mo = (uint32_t)sizeof(T) * m;
+                    const T rn = cl_ld<T>(dyn + foff + mo) - al * cl_ld<T>(dyn + qoff + lb);
+                    cl_st(dyn + roff + mo, rn);
+                    to = (unsigned)(m - (int)h1.x) < h1.y;
+                    if (to) {
+                        u = rn * dinv;
+                        cl_st(dyn + poff + lb, u);
                     }
                 }
-                if (!last) {
-                    exchange(C.expect);
-                } else if (lv > 0) {  // e, to the windows the prolongation reads
-                    __syncthreads();
-                    push_all(L, L.e);
-                    exchange(H.expect_all);
-                }
-                mark(L.level, OP_UPDATE);
+                if (to) push(poff, u);
+                m += kClThreads;
+                load_own(m);
             }
             if (!last) {
+                first_exchange(poff, q_off(i + 1));
+                mark(lv, OP_UPDATE);
                 steps += 1ull << (4 * lv);
                 break;  // B^ for the next step
             }
             if (lv == 0) {
+                mark(lv, OP_UPDATE);
                 done = true;
                 break;
             }
+            arrive_n((int)h0.z);  // e, to the windows the prolongation reads
+            bind(lv - 1);
+            wait_n();
+            mark(lv, OP_UPDATE);
             lv--;
         }
         if (done) break;
@@ -859,16 +1007,15 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
     __syncthreads();
     if (alive) {
         if (y.nsp > 0) {
-            const ClLev &L = y.lv[0];
-            const ClColor *tab = (const ClColor *)at(L.tab);
-            const T *e = (const T *)at(L.e);
-            for (int c = 0; c < L.ncol; c++)
-                for (int j = tid; j < tab[c].cnt; j += kClThreads)
-                    a.e[tab[c].g0 + j] = e[tab[c].li0 + j];
+            const int nown = (int)h0.x;  // (level 0 is bound)
+            const unsigned short *own = (const unsigned short *)at(lvs[0].own);
+            const T *e = vec(lvs[0].e);
+#pragma unroll 1
+            for (int m = tid; m < nown; m += kClThreads) a.e[((const int *)at(y.top))[m]] = *(const T *)((const unsigned char *)e + own[m]);
         } else {
-            const T *E = (const T *)at(y.E);
-            for (int i = rank * y.ch + tid; i < min(y.nd, (rank + 1) * y.ch); i += kClThreads)
-                a.e[i] = E[i];
+            const T *E = vec(y.E);
+#pragma unroll 1
+            for (int k = rank * y.ch + tid; k < min(y.nd, (rank + 1) * y.ch); k += kClThreads) a.e[k] = E[k];
         }
     }
     if (mark_on)
@@ -880,7 +1027,6 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
     cl_sync_all();  // no CTA leaves while a neighbour may still write into it
     if (a.ts && rank == 0 && tid == 0) *a.ts = global_ns();
 }
-
 
 // ---------------------------------------------------------------------------------------
 // setup of the cluster's image (device)
@@ -911,18 +1057,28 @@ __device__ __forceinline__ int cl_owner(const ClSrc &S, int c, int i) {
     const int len = S.cr[c + 1] - S.cr[c];
     return (kClRanks * (i - S.cr[c] + 1) - 1) / len;
 }
-// window tables: [level][rank][colour] (first, last + 1); cwin: the children's part alone
+// Window tables: [level][rank][colour] (first, last + 1). The children of the next level's rows
+// that lie in another strip than the row's owner have tables of their own: cwin[0] with the
+// next level's strips as owners (a swept level), cwin[1] with the owner of a row's first child
+// (the dense level, whose rows have no strips: fo[R]).
 __device__ __forceinline__ void cl_extend(int2 *w, int i) {
     volatile int *v = (volatile int *)w;
     if (i < v[0]) atomicMin(&w->x, i);
     if (i + 1 > v[1]) atomicMax(&w->y, i + 1);
 }
-__device__ __forceinline__ int2 *cl_win(int2 *win, int a, int r, int c) {
-    return win + ((size_t)a * kClRanks + r) * kClColors + c;
+__host__ __device__ inline size_t cl_win(int a, int r, int c) {
+    return ((size_t)a * kClRanks + r) * kClColors + c;
+}
+__device__ __forceinline__ int cl_child(const ClSrc &S, int R, int q) {
+    const int4 ch = (q < 4 ? S.ch : S.ch2)[R];
+    return (q & 3) == 0 ? ch.x : (q & 3) == 1 ? ch.y : (q & 3) == 2 ? ch.z : ch.w;
 }
 
-// columns of own rows, both ways, and children of own next-level rows in other strips
-__global__ void k_cl_windows(const __grid_constant__ ClSrcs G, int2 *win, int2 *cwin) {
+// columns of own rows, both ways, and children of own next-level rows in other strips. Rows
+// of a strip's inside touch nothing; the few at its edges hit a table entry that mostly holds
+// them already (read before the atomic).
+__global__ void k_cl_windows(const __grid_constant__ ClSrcs G, int2 *win, int2 *cwin, size_t words,
+                             int *fo) {
     const int a = blockIdx.y;
     const ClSrc &S = G.lv[a], &N = G.lv[a + 1];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -934,46 +1090,54 @@ __global__ void k_cl_windows(const __grid_constant__ ClSrcs G, int2 *win, int2 *
             if (j < 0) continue;
             const int cj = cl_colour(S, j), rj = cl_owner(S, cj, j);
             if (rj == r) continue;
-            cl_extend(cl_win(win, a, r, cj), j);
-            cl_extend(cl_win(win, a, rj, c), i);
+            cl_extend(win + cl_win(a, r, cj), j);
+            cl_extend(win + cl_win(a, rj, c), i);
         }
     }
     if (i < N.n) {
-        const int rn = cl_owner(N, cl_colour(N, i), i);
+        const int ra = cl_owner(N, cl_colour(N, i), i);
+        int rb = -1;
         for (int q = 0; q < (S.ch2 ? 8 : 4); q++) {
-            const int4 ch = (q < 4 ? S.ch : S.ch2)[i];
-            const int j = (q & 3) == 0 ? ch.x : (q & 3) == 1 ? ch.y : (q & 3) == 2 ? ch.z : ch.w;
+            const int j = cl_child(S, i, q);
             if (j < 0) continue;
-            const int cj = cl_colour(S, j);
-            if (cl_owner(S, cj, j) != rn) cl_extend(cl_win(cwin, a, rn, cj), j);
+            const int cj = cl_colour(S, j), rj = cl_owner(S, cj, j);
+            if (rb < 0) rb = rj;
+            if (rj != ra) cl_extend(cwin + cl_win(a, ra, cj), j);
+            if (rj != rb) cl_extend(cwin + words + cl_win(a, rb, cj), j);
         }
+        if (a == G.nsp - 1) fo[i] = max(rb, 0);
+        if (a == G.nsp - 2) fo[G.lv[G.nsp].n + i] = max(rb, 0);
     }
 }
 
-// one CTA, level by level: the children's part joins the window; then the parents of the
-// window's rows join the next level's window
+// one CTA, level by level: the children's part joins the window (the last level's next one
+// is dense, the one before may have either kind); then the parents of the window's rows join
+// the next level's window
 __global__ void __launch_bounds__(1024) k_cl_parents(const __grid_constant__ ClSrcs G, int2 *win,
-                                                     const int2 *cwin) {
+                                                     const int2 *cwin, size_t words) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     for (int a = 0; a < G.nsp; a++) {
         const ClSrc &S = G.lv[a];
         for (int k = threadIdx.x; k < kClRanks * S.ncol; k += blockDim.x) {
-            const int r = k / S.ncol, c = k - r * S.ncol;
-            const size_t o = ((size_t)a * kClRanks + r) * kClColors + c;
-            if (cwin[o].x < cwin[o].y) {
-                win[o].x = min(win[o].x, cwin[o].x);
-                win[o].y = max(win[o].y, cwin[o].y);
+            const size_t o = cl_win(a, k / S.ncol, k % S.ncol);
+            for (int kind = 0; kind < 2; kind++) {
+                if (kind == 0 ? a == G.nsp - 1 : a < G.nsp - 2) continue;
+                const int2 w = cwin[kind * words + o];
+                if (w.x < w.y) {
+                    win[o].x = min(win[o].x, w.x);
+                    win[o].y = max(win[o].y, w.y);
+                }
             }
         }
         __syncthreads();
         if (a + 1 < G.nsp) {
             const ClSrc &N = G.lv[a + 1];
             for (int k = warp; k < kClRanks * S.ncol; k += (int)(blockDim.x >> 5)) {
-                const int r = k / S.ncol, c = k - r * S.ncol;
-                const int2 w = *cl_win(win, a, r, c);
+                const int r = k / S.ncol;
+                const int2 w = win[cl_win(a, r, k % S.ncol)];
                 for (int i = w.x + lane; i < w.y; i += 32) {
                     const int p = S.parent[i];
-                    cl_extend(cl_win(win, a + 1, r, cl_colour(N, p)), p);
+                    cl_extend(win + cl_win(a + 1, r, cl_colour(N, p)), p);
                 }
             }
             __syncthreads();
@@ -982,10 +1146,12 @@ __global__ void __launch_bounds__(1024) k_cl_parents(const __grid_constant__ ClS
 }
 
 // the constant image of strip blockIdx.y, level blockIdx.z (nsp: the coarsest inverse); the
-// tables at its start are there already
+// tables at its start (op lists, heads) are there already. geo: [level][rank][colour]; over_n:
+// entries used in each strip's list of further destinations
 template <class T>
 __global__ void k_cl_image(const __grid_constant__ ClSrcs G, const __grid_constant__ ClLayout y,
-                           unsigned char *image, const double *Ainv, const float *Ainv2) {
+                           unsigned char *image, const ClColor *geo, int *over_n,
+                           const double *Ainv, const float *Ainv2) {
     const int a = blockIdx.z, r = blockIdx.y;
     unsigned char *im = image + (size_t)r * y.image_bytes;
     const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
@@ -1007,36 +1173,63 @@ __global__ void k_cl_image(const __grid_constant__ ClSrcs G, const __grid_consta
     const ClLev &L = y.lv[a];
     const ClSrc &S = G.lv[a];
     const ClHead H = *(const ClHead *)(im + L.head);
-    const ClColor *tab = (const ClColor *)(im + L.tab);
-    T *val = (T *)(im + L.val), *dinv = (T *)(im + L.dinv);
+    const ClColor *tab = geo + cl_win(a, r, 0);
+    T *val = (T *)(im + L.val), *diag = (T *)(im + L.diag), *dinv = (T *)(im + L.dinv);
     unsigned short *col = (unsigned short *)(im + L.col), *own = (unsigned short *)(im + L.own);
     unsigned short *par = (unsigned short *)(im + L.parent), *child = (unsigned short *)(im + L.child);
+    uint4 *dst = (uint4 *)(im + L.dst);  // (d0, 0, d1 or bit 31 and a list, 0)
+    unsigned *over = (unsigned *)(im + L.over);
     auto local = [&](const ClColor *tb, const ClSrc &s, int i) {  // window index of pi-row i
         const ClColor &C = tb[cl_colour(s, i)];
         return (unsigned short)(C.li0 + i - C.g0);
     };
+    constexpr int B = (int)sizeof(T);  // own rows, columns and destinations are byte offsets
+    const int G1 = 1 << L.lg;
+    constexpr int V = 16 / (int)sizeof(T);  // values per 16-byte piece
     for (int m = t0; m < H.nown; m += nt) {
         int c = 0;
         while (c + 1 < L.ncol && m >= tab[c + 1].m0) c++;
         const int i = tab[c].g0 + m - tab[c].m0;
         const int li = tab[c].li0 + m - tab[c].m0;
-        own[m] = (unsigned short)li;
+        own[m] = (unsigned short)(B * li);
         const int s0 = S.sl[i >> 5], width = (S.sl[(i >> 5) + 1] - s0) >> 5;
-        for (int k = 0; k < L.w; k++) {
+        // lane q of the row takes slots 1 + ns q ..; padding: value 0, the row's own column
+        for (int k = 1; k < 1 + L.ns * G1; k++) {
             const int o = s0 + 32 * k + (i & 31);
             const int j = k < width ? S.col[o] : -1;
-            col[k * L.R + m] = j >= 0 ? local(tab, S, j) : (unsigned short)li;
             T v = T(0);
             if (j >= 0) {
                 if constexpr (sizeof(T) == 8) v = S.val64[o];
                 else v = S.val32[o];
             }
-            val[k * L.R + m] = v;
+            const int vr = m * G1 + (k - 1) / L.ns, e = (k - 1) % L.ns;
+            col[(size_t)vr * kClSlots + e] = (unsigned short)(B * (j >= 0 ? local(tab, S, j) : li));
+            val[((size_t)(e / V) * L.R + vr) * V + e % V] = v;
         }
-        dinv[li] = (T)(1.0 / S.val64[s0 + (i & 31)]);
+        const double d = S.val64[s0 + (i & 31)];
+        if constexpr (sizeof(T) == 8) diag[m] = d;
+        else diag[m] = S.val32[s0 + (i & 31)];
+        dinv[m] = (T)(1.0 / d);
+        // the strips whose window holds the row
+        unsigned to[kClRanks];
+        int nd = 0;
+        for (int q = 0; q < kClRanks; q++) {
+            const ClColor &C = geo[cl_win(a, q, c)];
+            const int k = C.li0 + i - C.g0 - C.seg0;  // position in its window
+            if (q != r && k >= 0 && k < C.seglen) to[nd++] = (unsigned)q << 16 | (unsigned)(B * (C.seg0 + k));
+        }
+        uint4 d2 = make_uint4(nd > 0 ? to[0] : kClNone, 0, nd > 1 ? to[1] : kClNone, 0);
+        if (nd > 2) {
+            const int o = atomicAdd(&over_n[a * kClRanks + r], nd);
+            for (int k = 1; k < nd; k++) over[o + k - 1] = to[k];
+            over[o + nd - 1] = kClNone;
+            d2.z = 0x80000000u | (unsigned)o;
+        }
+        dst[m] = d2;
+        if (a == 0) ((int *)(im + y.top))[m] = i;
     }
     const bool swept = a + 1 < y.nsp;
-    const ClColor *ntab = swept ? (const ClColor *)(im + y.lv[a + 1].tab) : nullptr;
+    const ClColor *ntab = swept ? geo + cl_win(a + 1, r, 0) : nullptr;
     for (int k = t0; k < H.nwin; k += nt) {
         int c = 0;
         while (c + 1 < L.ncol && k >= tab[c + 1].seg0) c++;
@@ -1054,9 +1247,9 @@ __global__ void k_cl_image(const __grid_constant__ ClSrcs G, const __grid_consta
             R = ((const unsigned short *)(im + y.down))[m];
         }
         for (int q = 0; q < L.nch; q++) {
-            const int4 ch = (q < 4 ? S.ch : S.ch2)[R];
-            const int j = (q & 3) == 0 ? ch.x : (q & 3) == 1 ? ch.y : (q & 3) == 2 ? ch.z : ch.w;
-            child[q * L.Rn + m] = j >= 0 ? local(tab, S, j) : (unsigned short)0xFFFF;
+            const int j = cl_child(S, R, q);
+            // four per 8-byte entry
+            child[((size_t)(q >> 2) * L.Rn + m) * 4 + (q & 3)] = j >= 0 ? local(tab, S, j) : (unsigned short)0xFFFF;
         }
     }
 }
@@ -1096,8 +1289,7 @@ k_dense_cycle(const __grid_constant__ ClSrc S, const __grid_constant__ ClLayout 
     for (int R = tid; R < nc; R += nt) {
         double v = 0.0;
         for (int q = 0; q < (S.ch2 ? 8 : 4); q++) {
-            const int4 ch = (q < 4 ? S.ch : S.ch2)[R];
-            const int j = (q & 3) == 0 ? ch.x : (q & 3) == 1 ? ch.y : (q & 3) == 2 ? ch.z : ch.w;
+            const int j = cl_child(S, R, q);
             if (j >= 0) v += t[j];
         }
         fc[R] = v;
@@ -1119,5 +1311,7 @@ k_dense_cycle(const __grid_constant__ ClSrc S, const __grid_constant__ ClLayout 
         row[(size_t)y.ch * y.stride + unit] = (T)dot(i, 0);
     }
 }
+
+#undef CL_F
 
 }  // namespace amg

@@ -929,15 +929,18 @@ void *cycle_kernel(int B) {
 // one candidate: swept levels [tl, tl + nsp), the dense level after them
 struct ClPlan {
     ClLayout y;
+    std::vector<ClColor> geo;           // the strips of every swept level
     std::vector<unsigned char> tables;  // [kClRanks][table_bytes]: the head of every image
     int table_bytes = 0;
 };
 
-// Layout and tables for swept levels first .. of src (win: their windows), or false if they
-// do not fit `budget` bytes of shared memory. `s0`: src index of the first swept level.
+// Layout and tables for the swept levels G.lv[s0 ..] (hierarchy levels level0 ..) and the dense
+// level after them, or false if they do not fit `budget` bytes of shared memory. win: their
+// windows; xchild: [2][nlv], by the next level's kind (swept, dense); fo: owner of each row of
+// the dense level.
 template <class T>
-bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vector<int> &xchild,
-                  const std::vector<int> &widths, int s0, int level0, bool dense, int nch,
+bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vector<int> &xchild, int nlv,
+                  const int *fo, const std::vector<int> &widths, int s0, int level0, bool dense, int nch,
                   const amg_options &opt, long budget, ClPlan &P) {
     constexpr int vb = (int)sizeof(T), NR = kClRanks;
     ClLayout &y = P.y;
@@ -953,78 +956,139 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
     y.ch = (((D.n + NR - 1) / NR) + 3) & ~3;
     y.stride = NR * y.ch;
     auto win_of = [&](int a, int r, int c) {
-        return win[((size_t)(s0 + a) * NR + r) * kClColors + c];
+        return win[cl_win(s0 + a, r, c)];
     };
     auto own_of = [](const ClSrc &S, int r, int c) {
         const int len = S.cr[c + 1] - S.cr[c];
         return make_int2(S.cr[c] + cl_part(len, r), S.cr[c] + cl_part(len, r + 1));
     };
-    // tables, one image per CTA
-    struct LevelTab {
-        ClHead head;
-        std::vector<ClColor> col;
-        std::vector<ClPush> push;
-    };
-    std::vector<std::vector<LevelTab>> tab(NR, std::vector<LevelTab>(y.nsp));
-    std::vector<std::vector<int>> down(NR), peers(NR);
+    // the strips: windows, bytes exchanged, neighbours
+    P.geo.assign((size_t)std::max(1, y.nsp) * NR * kClColors, ClColor{});
+    auto geo = [&](int a, int r, int c) -> ClColor & { return P.geo[cl_win(a, r, c)]; };
+    std::vector<std::vector<ClHead>> head(y.nsp, std::vector<ClHead>(NR));
+    std::vector<std::vector<std::vector<int>>> expect(y.nsp);
+    std::vector<int> c_first(y.nsp, 0);
+    std::vector<std::vector<int>> peers(NR);
     std::vector<std::vector<char>> is_peer(NR, std::vector<char>(NR, 0));
-    std::vector<size_t> max_push(y.nsp, 1), max_own(y.nsp + 1, 1), max_win(y.nsp, 1);
+    std::vector<size_t> max_own(y.nsp + 1, 1), max_win(y.nsp, 1), over(y.nsp, 0);
     for (int a = 0; a < y.nsp; a++) {
         const ClSrc &S = G.lv[s0 + a];
+        ClLev &L = y.lv[a];
+        L.level = level0 + a;
+        L.ncol = S.ncol;
+        L.w = std::max(1, widths[level0 + a]);
+        // Lanes per row: as few as take its slots, eight each. FP64: one instruction of a warp
+        // takes 64 cycles, of each of nw warps at once 19 nw (measured, whatever the lanes do),
+        // so rows are split further where their warps still run side by side: the sum over a
+        // step's colours (the largest one's rows) and its two products with all own rows
+        L.lg = -1;
+        double best = 0;
+        int rows = 1, all = 0, colours = 0;
+        for (int c = 0; c < S.ncol; c++) {
+            const int len = (S.cr[c + 1] - S.cr[c] + NR - 1) / NR;
+            rows = std::max(rows, len);
+            all += len;
+            colours += S.cr[c + 1] > S.cr[c] ? 2 : 0;
+        }
+        for (int lg = 0; lg <= 2; lg++) {
+            int ns = 2;  // 2, 4 or 8
+            while (ns << lg < L.w - 1 && ns <= kClSlots) ns *= 2;
+            if (ns > kClSlots) continue;
+            auto fp64 = [&](int r, int instr) {
+                const int t = r << lg, full = t / kClThreads, rest = (t % kClThreads + 31) / 32;
+                return (full * 19.0 * kClWarps + (rest ? std::max(64, 19 * rest) : 0)) * instr + 70.0 * lg;
+            };
+            const double cost = vb == 8 ? colours * fp64(rows, ns + lg + 2) + 2 * fp64(all, ns + lg + 3) : lg;
+            if (L.lg >= 0 && cost >= best) continue;
+            L.lg = lg;
+            L.ns = vb == 8 ? ns : kClSlots;
+            best = cost;
+        }
+        if (L.lg < 0) return false;
+        L.nch = nch;
+        int cf = -1, cl = 0;
+        for (int c = 0; c < S.ncol; c++)
+            if (S.cr[c + 1] > S.cr[c]) {
+                if (cf < 0) cf = c;
+                cl = c;
+            }
+        cf = std::max(cf, 0);
         for (int r = 0; r < NR; r++) {
-            LevelTab &t = tab[r][a];
-            t.col.resize(S.ncol);
-            int m0 = 0, seg0 = 0;
+            ClHead &h = head[a][r];
+            std::memset(&h, 0, sizeof h);
             for (int c = 0; c < S.ncol; c++) {
                 const int2 o = own_of(S, r, c), w = win_of(a, r, c);
-                ClColor &C = t.col[c];
-                std::memset(&C, 0, sizeof C);
+                ClColor &C = geo(a, r, c);
                 C.cnt = o.y - o.x;
-                C.m0 = m0;
-                C.seg0 = seg0;
+                C.m0 = h.nown;
+                C.seg0 = h.nwin;
                 C.seglen = w.y - w.x;
-                C.li0 = seg0 + o.x - w.x;
+                C.li0 = h.nwin + o.x - w.x;
                 C.g0 = o.x;
-                m0 += C.cnt;
-                seg0 += C.seglen;
+                h.nown += C.cnt;
+                h.nwin += C.seglen;
             }
-            if (seg0 > 65534) return false;
-            t.head = ClHead{m0, seg0, 0, 0};
-            max_own[a] = std::max(max_own[a], (size_t)m0);
-            max_win[a] = std::max(max_win[a], (size_t)seg0);
+            if (h.nwin * vb > 65535) return false;  // 16-bit byte offsets
+            h.fc0 = geo(a, r, cf).m0;
+            h.fcn = geo(a, r, cf).cnt;
+            c_first[a] = cf;
+            h.fs0 = geo(a, r, cf).seg0;
+            h.fs1 = h.fs0 + geo(a, r, cf).seglen;
+            h.ls0 = geo(a, r, cl).seg0;
+            h.ls1 = h.ls0 + geo(a, r, cl).seglen;
+            max_own[a] = std::max(max_own[a], (size_t)h.nown);
+            max_win[a] = std::max(max_win[a], (size_t)h.nwin);
         }
-        for (int r = 0; r < NR; r++)
+        expect[a].assign(NR, std::vector<int>(S.ncol, 0));
+        for (int r = 0; r < NR; r++) {
+            size_t all = 0;
             for (int c = 0; c < S.ncol; c++) {
                 const int2 o = own_of(S, r, c);
-                ClColor &C = tab[r][a].col[c];
-                C.push0 = (int)tab[r][a].push.size();
+                int holders = 0;  // strips that hold some of these rows
+                size_t rows = 0;
                 for (int d = 0; d < NR; d++) {
                     if (d == r) continue;
                     const int2 w = win_of(a, d, c);
                     const int lo = std::max(o.x, w.x), hi = std::min(o.y, w.y);
                     if (lo >= hi) continue;
-                    ClColor &X = tab[d][a].col[c];
-                    tab[r][a].push.push_back(ClPush{d + 256 * c, lo - o.x, hi - lo, X.seg0 + lo - w.x});
-                    X.expect += (hi - lo) * vb;
-                    tab[d][a].head.expect_all += (hi - lo) * vb;
+                    expect[a][d][c] += (hi - lo) * vb;
+                    head[a][d].expect_all += (hi - lo) * vb;
                     is_peer[r][d] = is_peer[d][r] = 1;
+                    holders++;
+                    rows += hi - lo;
                 }
-                C.npush = (int)tab[r][a].push.size() - C.push0;
+                if (holders > 2) all += rows;  // may need the list of further destinations
             }
-        for (int r = 0; r < NR; r++) {
-            tab[r][a].head.npush = (int)tab[r][a].push.size();
-            max_push[a] = std::max(max_push[a], tab[r][a].push.size());
+            over[a] = std::max(over[a], all);
         }
     }
-    for (int r = 0; r < NR; r++) {
-        for (int c = 0; c < D.ncol; c++) {
-            const int2 o = own_of(D, r, c);
-            for (int i = o.x; i < o.y; i++) down[r].push_back(i);
-        }
-        max_own[y.nsp] = std::max(max_own[y.nsp], down[r].size());
+    for (int r = 0; r < NR; r++)
         for (int d = 0; d < NR; d++)
             if (is_peer[r][d]) peers[r].push_back(d);
-    }
+    // the dense level's rows, each with its first child
+    std::vector<std::vector<unsigned short>> down(NR);
+    for (int i = 0; i < D.n && y.nsp > 0; i++) down[fo[i]].push_back((unsigned short)i);
+    for (int r = 0; r < NR; r++) max_own[y.nsp] = std::max(max_own[y.nsp], down[r].size());
+    for (int a = 0; a < y.nsp; a++)
+        for (int r = 0; r < NR; r++) head[a][r].fexp = expect[a][r][c_first[a]];
+    // the sweeps of every strip: before the restriction (the first colour is done by the step
+    // before) and after the correction
+    auto lists = [&](int a, int r, std::vector<ClOp> &pre, std::vector<ClOp> &post) {
+        const ClLev &L = y.lv[a];
+        const ClSrc &S = G.lv[s0 + a];
+        pre.clear();
+        post.clear();
+        auto colour = [&](int c) {
+            const ClColor &C = geo(a, r, c);
+            return ClOp{C.m0 << L.lg, C.cnt << L.lg, expect[a][r][c], 0};
+        };
+        for (int sw = 0; sw < y.nu_pre; sw++)
+            for (int c = 0; c < S.ncol; c++)
+                if (S.cr[c + 1] > S.cr[c] && (sw > 0 || c > c_first[a])) pre.push_back(colour(c));
+        for (int sw = 0; sw < y.nu_post; sw++)
+            for (int c = S.ncol - 1; c >= 0; c--)
+                if (S.cr[c + 1] > S.cr[c]) post.push_back(colour(c));
+    };
     size_t off = 0;
     auto take = [&](size_t bytes) {
         const int o = (int)off;
@@ -1034,48 +1098,44 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
     y.dhead = take(sizeof(int));
     y.down = take(sizeof(short) * max_own[y.nsp]);
     y.peers = take(sizeof(int) * (NR + 1));
+    y.levels = take(sizeof(ClLev) * y.nsp);
+    std::vector<ClOp> pre, post;
     for (int a = 0; a < y.nsp; a++) {
         ClLev &L = y.lv[a];
-        const ClSrc &S = G.lv[s0 + a];
+        lists(a, 0, pre, post);  // the same length in every strip
+        L.npre = (int)pre.size();
+        L.npost = (int)post.size();
         L.head = take(sizeof(ClHead));
-        L.tab = take(sizeof(ClColor) * S.ncol);
-        L.push = take(sizeof(ClPush) * max_push[a]);
+        L.pre = take(sizeof(ClOp) * std::max<size_t>(1, pre.size()));
+        L.post = take(sizeof(ClOp) * post.size());
     }
     P.table_bytes = (int)off;
     for (int a = 0; a < y.nsp; a++) {
         ClLev &L = y.lv[a];
-        const ClSrc &S = G.lv[s0 + a];
-        L.level = level0 + a;
-        L.n = S.n;
-        L.ncol = S.ncol;
-        L.w = std::max(1, widths[level0 + a]);
-        L.R = (int)((max_own[a] + 23) / 32 * 32 + 8);
-        L.c_first = -1;
-        for (int c = 0; c < S.ncol; c++)
-            if (S.cr[c + 1] > S.cr[c]) {
-                if (L.c_first < 0) L.c_first = c;
-                L.c_last = c;
-                L.cmask |= 1u << c;
-            }
-        L.nch = nch;
+        L.R = (int)max_own[a] << L.lg;
+        L.nact = std::min(kClWarps, (L.R + 31) / 32);
         L.Rn = (int)max_own[a + 1];
-        L.xchild = xchild[s0 + a];
-        L.val = take((size_t)L.w * L.R * vb);
-        L.col = take((size_t)L.w * L.R * 2);
-        L.dinv = take(max_win[a] * vb);
+        L.xchild = xchild[(a + 1 < y.nsp ? 0 : 1) * nlv + s0 + a];
+        L.over = take(sizeof(unsigned) * over[a]);
+        L.val = take((size_t)L.ns * L.R * vb);
+        L.col = take((size_t)kClSlots * L.R * 2);
+        L.diag = take(max_own[a] * vb);
+        L.dinv = take(max_own[a] * vb);
         L.own = take(2 * max_own[a]);
+        L.dst = take(sizeof(uint4) * max_own[a]);
         L.parent = take(2 * max_win[a]);
         L.child = take(2 * (size_t)nch * L.Rn);
     }
+    y.top = take(sizeof(int) * max_own[0]);
     y.mat = take((size_t)(dense ? 2 : 1) * y.ch * y.stride * vb);
     if (!dense && vb == 4) y.mat_lo = take((size_t)y.ch * y.stride * vb);
     y.image_bytes = (int)off;
     for (int a = 0; a < y.nsp; a++) {
         ClLev &L = y.lv[a];
         const size_t b = max_win[a] * vb;
-        L.rhs = take(b);
+        L.rhs = take(max_own[a] * vb);
+        L.r = take(max_own[a] * vb);
         L.e = take(b);
-        L.r = take(b);
         for (int k = 0; k < y.kc; k++) {
             L.p[k] = take(b);
             L.q[k] = take(b);
@@ -1087,7 +1147,7 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
     y.out = take((size_t)2 * y.ch * vb);
     y.stage = take(max_own[y.nsp] * vb);
     if (dense) {
-        y.Rv = take(len);
+        y.Rv = y.F;  // r_{i+1} over r_i
         for (int k = 0; k < y.kc; k++) {
             y.P[k] = take(len);
             y.Q[k] = take(len);
@@ -1101,15 +1161,15 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
         auto put = [&](int o, const void *p, size_t b) { if (b) std::memcpy(im + o, p, b); };
         const int nd = (int)down[r].size(), np = (int)peers[r].size();
         put(y.dhead, &nd, sizeof nd);
-        const std::vector<unsigned short> d16(down[r].begin(), down[r].end());
-        put(y.down, d16.data(), 2 * d16.size());
+        put(y.down, down[r].data(), 2 * down[r].size());
         put(y.peers, &np, sizeof np);
+        put(y.levels, y.lv, sizeof(ClLev) * y.nsp);
         put(y.peers + (int)sizeof(int), peers[r].data(), sizeof(int) * peers[r].size());
         for (int a = 0; a < y.nsp; a++) {
-            const LevelTab &t = tab[r][a];
-            put(y.lv[a].head, &t.head, sizeof t.head);
-            put(y.lv[a].tab, t.col.data(), sizeof(ClColor) * t.col.size());
-            put(y.lv[a].push, t.push.data(), sizeof(ClPush) * t.push.size());
+            lists(a, r, pre, post);
+            put(y.lv[a].head, &head[a][r], sizeof(ClHead));
+            put(y.lv[a].pre, pre.data(), sizeof(ClOp) * pre.size());
+            put(y.lv[a].post, post.data(), sizeof(ClOp) * post.size());
         }
     }
     return true;
@@ -1130,7 +1190,7 @@ void build_cluster(amg_hierarchy *h, EngineBase *E, int optin) {
     E->cl.tl = nlev;
     cudaFuncAttributes fa;
     AMG_CUDA(cudaFuncGetAttributes(&fa, cluster_kernel<T>()));
-    const long budget = (long)optin - (long)fa.sharedSizeBytes - 1024;
+    const long budget = (long)optin - (long)fa.sharedSizeBytes;
     AMG_CUDA(cudaFuncSetAttribute(cluster_kernel<T>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   (int)budget));
     AMG_CUDA(cudaFuncSetAttribute(cluster_kernel<T>(), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
@@ -1175,32 +1235,37 @@ void build_cluster(amg_hierarchy *h, EngineBase *E, int optin) {
                      h->lev[nlev - 1].color_rows.size() > 1;
     G.lv[G.nsp] = source(nlev - 1, crr);
     const size_t words = (size_t)G.nsp * kClRanks * kClColors;
-    std::vector<int2> win(2 * words);
+    std::vector<int2> win(3 * words);
     for (int a = 0; a < G.nsp; a++)
         for (int r = 0; r < kClRanks; r++)
             for (int c = 0; c < kClColors; c++) {
-                const size_t o = ((size_t)a * kClRanks + r) * kClColors + c;
+                const size_t o = cl_win(a, r, c);
                 const ClSrc &S = G.lv[a];
                 const int len = c < S.ncol ? S.cr[c + 1] - S.cr[c] : 0;
                 win[o] = c < S.ncol ? make_int2(S.cr[c] + cl_part(len, r), S.cr[c] + cl_part(len, r + 1))
                                     : make_int2(0, 0);
-                win[words + o] = make_int2(INT32_MAX, 0);
+                win[words + o] = win[2 * words + o] = make_int2(INT32_MAX, 0);
             }
+    const int nc = h->lev[nlev - 1].n, nfo = nc + (G.nsp > 1 ? h->lev[last].n : 0);
     Scratch tmp(s);
-    int2 *dwin = tmp.get<int2>(2 * words);
+    int2 *dwin = tmp.get<int2>(3 * words);
+    int *dfo = tmp.get<int>(nfo);
     AMG_CUDA(cudaMemcpyAsync(dwin, win.data(), sizeof(int2) * win.size(), cudaMemcpyHostToDevice, s));
-    k_cl_windows<<<dim3(nblocks_for(G.lv[0].n, 256), G.nsp), 256, 0, s>>>(G, dwin, dwin + words);
+    k_cl_windows<<<dim3(nblocks_for(G.lv[0].n, 256), G.nsp), 256, 0, s>>>(G, dwin, dwin + words, words, dfo);
     AMG_LAUNCH_CHECK();
-    k_cl_parents<<<1, 1024, 0, s>>>(G, dwin, dwin + words);
+    k_cl_parents<<<1, 1024, 0, s>>>(G, dwin, dwin + words, words);
     AMG_LAUNCH_CHECK();
+    std::vector<int> fo(nfo);
     AMG_CUDA(cudaMemcpyAsync(win.data(), dwin, sizeof(int2) * win.size(), cudaMemcpyDeviceToHost, s));
+    AMG_CUDA(cudaMemcpyAsync(fo.data(), dfo, sizeof(int) * nfo, cudaMemcpyDeviceToHost, s));
     AMG_CUDA(cudaStreamSynchronize(s));
-    std::vector<int> xchild(G.nsp, 0);
-    for (int a = 0; a < G.nsp; a++)
-        for (size_t k = 0; k < (size_t)kClRanks * kClColors; k++) {
-            const int2 w = win[words + (size_t)a * kClRanks * kClColors + k];
-            if (w.x < w.y) xchild[a] = 1;
-        }
+    std::vector<int> xchild(2 * G.nsp, 0);
+    for (int kind = 0; kind < 2; kind++)
+        for (int a = 0; a < G.nsp; a++)
+            for (size_t k = 0; k < (size_t)kClRanks * kClColors; k++) {
+                const int2 w = win[(1 + kind) * words + cl_win(a, 0, 0) + k];
+                if (w.x < w.y) xchild[kind * G.nsp + a] = 1;
+            }
     // the finest start that fits; with the dense matrices if that start allows them
     ClSrcs GD = G;  // dense level = the last swept one
     GD.nsp = G.nsp - 1;
@@ -1208,9 +1273,12 @@ void build_cluster(amg_hierarchy *h, EngineBase *E, int optin) {
     ClPlan P;
     bool ok = false;
     int s0 = 0;
-    for (; s0 < G.nsp && !ok; s0++) {
-        ok = can_dense && cluster_plan<T>(GD, win, xchild, widths, s0, first + s0, true, nch, h->opt, budget, P);
-        if (!ok) ok = cluster_plan<T>(G, win, xchild, widths, s0, first + s0, false, nch, h->opt, budget, P);
+    for (; s0 < G.nsp; s0++) {
+        ok = can_dense && cluster_plan<T>(GD, win, xchild, G.nsp, fo.data() + nc, widths, s0, first + s0, true,
+                                          nch, h->opt, budget, P);
+        if (!ok)
+            ok = cluster_plan<T>(G, win, xchild, G.nsp, fo.data(), widths, s0, first + s0, false, nch, h->opt,
+                                 budget, P);
         if (ok) break;
     }
     if (!ok) return;
@@ -1225,14 +1293,18 @@ void build_cluster(amg_hierarchy *h, EngineBase *E, int optin) {
     AMG_CUDA(cudaMemcpy2DAsync(E->cl_image, y.image_bytes, P.tables.data(), P.table_bytes, P.table_bytes,
                                kClRanks, cudaMemcpyHostToDevice, s));
     const Level &C = h->lev[nlev - 1];
-    k_cl_image<T><<<dim3(4, kClRanks, y.nsp + 1), 256, 0, s>>>(U, y, E->cl_image, C.Ainv, C.Ainv32);
+    ClColor *geo = tmp.get<ClColor>(P.geo.size());
+    int *over_n = tmp.get<int>(kClLevels * kClRanks);
+    AMG_CUDA(cudaMemcpyAsync(geo, P.geo.data(), sizeof(ClColor) * P.geo.size(), cudaMemcpyHostToDevice, s));
+    AMG_CUDA(cudaMemsetAsync(over_n, 0, sizeof(int) * kClLevels * kClRanks, s));
+    k_cl_image<T><<<dim3(4, kClRanks, y.nsp + 1), 256, 0, s>>>(U, y, E->cl_image, geo, over_n, C.Ainv, C.Ainv32);
     AMG_LAUNCH_CHECK();
     if (y.dense) {
         const size_t smem = sizeof(double) * (3 * (size_t)y.nd + 2 * (size_t)C.n);
         k_dense_cycle<T><<<y.nd, 128, smem, s>>>(U.lv[U.nsp], y, E->cl_image, C.Ainv, C.n);
         AMG_LAUNCH_CHECK();
     }
-    AMG_CUDA(cudaStreamSynchronize(s));  // P.tables is a local
+    AMG_CUDA(cudaStreamSynchronize(s));  // P's tables are locals
     E->cl = y;
 }
 
