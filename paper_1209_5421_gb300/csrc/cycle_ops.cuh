@@ -328,13 +328,18 @@ __device__ __forceinline__ void red_release_add_u64(unsigned long long *p, unsig
     asm volatile("red.release.gpu.global.add.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
+// ahead() runs between the arrival and the wait: loads that do not depend on other CTAs
+template <class Ahead>
 __device__ __forceinline__ bool grid_barrier(unsigned long long *count, int *err,
                                              unsigned long long &target, int &abort_flag,
-                                             unsigned long long limit_ns = kBarrierLimitNs) {
+                                             unsigned long long limit_ns, const Ahead &ahead) {
     __syncthreads();
     if (threadIdx.x == 0) {
         target += gridDim.x;
         red_release_add_u64(count, 1ull);
+    }
+    ahead();
+    if (threadIdx.x == 0) {
         unsigned long long t0 = 0;
         int spins = 0;
         while (ld_acquire_u64(count) < target) {
@@ -363,10 +368,10 @@ constexpr int kRowBatch = 9;  // one batch for a 9-point row
 // sum over slots k0 <= k < width of a_ik x[c_ik] (padding contributes nothing)
 template <class LV>
 __device__ __forceinline__ typename LV::val_t row_dot(const LV &L, int base, int k0, int width,
-                                                      const typename LV::val_t *x) {
+                                                      const typename LV::val_t *x,
+                                                      typename LV::val_t acc = 0) {
     using T = typename LV::val_t;
     using I = typename LV::idx_t;
-    T acc = 0;
     for (int kb = k0; kb < width; kb += kRowBatch) {
         I c[kRowBatch];
         T a[kRowBatch];
@@ -383,6 +388,46 @@ __device__ __forceinline__ typename LV::val_t row_dot(const LV &L, int base, int
 #pragma unroll
         for (int j = 0; j < kRowBatch; j++) acc += a[j] * xv[j];
     }
+    return acc;
+}
+
+// The first batch of a row's slots in registers, read ahead of its op. A row costs two dependent
+// round trips to memory: its columns and values, then the gathered x. The first depends on
+// nothing an op computes, so the grid-wide executor issues it before the barrier in front of
+// the op (op_ahead), for ops of at most one row per thread.
+template <class LV>
+struct RowAhead {
+    int row = -1;                  // the row held, -1: none
+    int base = 0, width = 0;
+    typename LV::idx_t c[kRowBatch];
+    typename LV::val_t a[kRowBatch];
+};
+template <class LV>
+__device__ __forceinline__ void row_load(const LV &L, int i, int k0, RowAhead<LV> &p) {
+    using T = typename LV::val_t;
+    using I = typename LV::idx_t;
+    p.row = i;
+    row_span(L, i, p.base, p.width);
+#pragma unroll
+    for (int j = 0; j < kRowBatch; j++) {
+        const int k = k0 + j;
+        p.c[j] = k < p.width ? L.col[p.base + 32 * k] : (I)-1;
+        p.a[j] = k < p.width ? L.val[p.base + 32 * k] : T(0);
+    }
+}
+// sum over slots k >= k0 of the row held (row_dot's operations in its order)
+template <class LV>
+__device__ __forceinline__ typename LV::val_t row_dot_held(const LV &L, const RowAhead<LV> &p, int k0,
+                                                           const typename LV::val_t *x) {
+    using T = typename LV::val_t;
+    T xv[kRowBatch];
+#pragma unroll
+    for (int j = 0; j < kRowBatch; j++)
+        xv[j] = (col_ok(p.c[j]) && idx_ok((int)p.c[j], L.n)) ? x[p.c[j]] : T(0);
+    T acc = 0;
+#pragma unroll
+    for (int j = 0; j < kRowBatch; j++) acc += p.a[j] * xv[j];
+    if (p.width > k0 + kRowBatch) acc = row_dot(L, p.base, k0 + kRowBatch, p.width, x, acc);
     return acc;
 }
 
@@ -1149,6 +1194,75 @@ __device__ void op_update(const LV &L, const Op &op, const RedCtx &rc, int tid, 
 
 // run one op (everything except OP_TAIL / OP_NOP) on level view L by threads tid < nth of
 // group g; next() gives the view of the next coarser level (only its rhs and e are used)
+// Does op_ahead read the op's rows? At most one per thread (more rows are better left to loads
+// that overlap each other: a loop reading one row ahead took 36 us instead of 17 for the
+// residual of 965k rows), on a quadtree's levels (an octree's rows are wider than the batch
+// held, and their first batch ahead of the rest gained nothing: 4.7 -> 5.4 us per colour of
+// 32,768 rows). Every thread answers the same. Per Gauss-Seidel colour, barrier included, FP32
+// (FP64): 1,046,529 rows 6.5 -> 5.6 us, 965,510 rows 5.9 -> 4.7, 262,144 rows 3.8 -> 3.2 (4.5 ->
+// 3.7), 65,536 rows 3.5 -> 3.0 (3.5 -> 2.8).
+template <class LV>
+__device__ __forceinline__ bool op_has_ahead(const LV &L, const Op &op, int nth) {
+    if (LV::coop || L.children2) return false;
+    if (op.kind == OP_GS) return op.i1 - op.i0 <= nth;
+    return (op.kind == OP_SPMV_DOT || op.kind == OP_RESID) && L.n <= nth;
+}
+// this thread's row of the op, read before the barrier in front of it (the matrix and the
+// block bounds only, which no op changes)
+template <class LV>
+__device__ __forceinline__ void op_ahead(const LV &L, const Op &op, int tid, int nth,
+                                         RowAhead<LV> &held) {
+    held.row = -1;
+    if (!op_has_ahead(L, op, nth)) return;
+    if (op.kind == OP_GS) {
+        const int b = op.i0 + tid;
+        if (b < op.i1) row_load(L, !L.fine ? b : op.backward ? L.bptr[b + 1] - 1 : L.bptr[b], 1, held);
+    } else if (tid < L.n) {
+        row_load(L, tid, 0, held);
+    }
+}
+// the op on the rows held (op_gs, op_resid, op_spmv_dot with their first rows read ahead)
+template <class LV, int RM, class G>
+__device__ __forceinline__ void run_op_held(const LV &L, const Op &op, const RedCtx &rc, int tid,
+                                            int nth, const G &g, const BigScratch &sc,
+                                            const RowAhead<LV> &held) {
+    using T = typename LV::val_t;
+    const int i = held.row;
+    if (op.kind == OP_GS) {
+        const T *f = vec_of(L, op.fsel);
+        T *u = vec_of(L, op.usel);
+        const bool big = L.fine && op.bb1 > op.bb0;
+        if (big) prefetch_big_tasks(L, op, f, u, tid, nth, (int)blockIdx.x, (int)gridDim.x);
+        if (i >= 0) {
+            const int b = op.i0 + tid;
+            const int r0 = L.fine ? L.bptr[b] : i, r1 = L.fine ? L.bptr[b + 1] : i + 1;
+            const T fi = f[i], di = L.dinv[i], acc = row_dot_held(L, held, 1, u);
+            if (!(big && r1 - r0 > kBigBlockRows)) {  // (those: in level order, below)
+                u[i] = (fi - acc) * di;
+                if (!op.backward)
+                    for (int k = r0 + 1; k < r1; k++) gs_row(L, k, f, u);
+                else
+                    for (int k = r1 - 2; k >= r0; k--) gs_row(L, k, f, u);
+            }
+        }
+        if (big) op_gs_big_blocks(L, op, f, u, tid, nth, (int)blockIdx.x, (int)gridDim.x, sc);
+    } else if (op.kind == OP_RESID) {
+        const T *f = vec_of(L, op.fsel), *u = vec_of(L, op.usel);
+        if (i >= 0) pick(L.q, op.step)[i] = f[i] - row_dot_held(L, held, 0, u);
+    } else {
+        const T *p = pick(L.p, op.step), *r = op.step == 0 ? L.rhs : L.r;
+        T v[2] = {0, 0};
+        if (i >= 0) {
+            const T pr = p[i], ri = r[i], acc = row_dot_held(L, held, 0, p);
+            pick(L.q, op.step)[i] = acc;
+            v[0] = pr * acc;
+            v[1] = ri * pr;
+        }
+        double *out[2] = {&L.sc[SC_PQ0 + op.step], &L.sc[SC_RP0 + op.step]};
+        reduce_store<2, RM, T>(v, out, rc, op.red_pb, g);
+    }
+}
+
 template <class LV, int RM, class G, class Next>
 __device__ __forceinline__ void run_op_on(const LV &L, const Next &next, const Op &op,
                                           const RedCtx &rc, int tid, int nth, const G &g,

@@ -151,6 +151,8 @@ __global__ void __launch_bounds__(cycle_threads<T>(), 1) k_cycle(CycleArgs<T> a)
         sc.wwarps = a.big_wwarps;
         sc.wslice = a.big_wslice;
     }
+    RowAhead<GL> held;
+    op_ahead(gtab[sop[a.k0 & 1].level], sop[a.k0 & 1], gtid, gnth, held);
     for (int k = a.k0; k < a.k1; k++) {
         const Op &op = sop[k & 1];
         // the next descriptor into the other buffer (last read by op k-1), issued before op k
@@ -158,10 +160,16 @@ __global__ void __launch_bounds__(cycle_threads<T>(), 1) k_cycle(CycleArgs<T> a)
         if (threadIdx.x < kOpWords && k + 1 < a.k1)
             ((int *)&sop[(k + 1) & 1])[threadIdx.x] = ((const int *)(a.prog + k + 1))[threadIdx.x];
         if (op.fin_pb >= 0) finalize(a, gtab, op);
-        if (op.kind != OP_NOP) run_op<GL, RM_PARTIAL>(gtab, op, rc, gtid, gnth, sc);
+        if (op_has_ahead(gtab[op.level], op, gnth))
+            run_op_held<GL, RM_PARTIAL>(gtab[op.level], op, rc, gtid, gnth, BlockGroup{}, sc, held);
+        else if (op.kind != OP_NOP)
+            run_op<GL, RM_PARTIAL>(gtab, op, rc, gtid, gnth, sc);
         // the end of the launch orders its last op before whatever follows on the stream
         const bool last = k + 1 == a.k1;
-        if (!last && !grid_barrier(a.bar, a.err, target, abort_flag, a.bar_limit_ns)) break;
+        const Op &nx = sop[(k + 1) & 1];
+        if (!last && !grid_barrier(a.bar, a.err, target, abort_flag, a.bar_limit_ns,
+                                   [&] { op_ahead(gtab[nx.level], nx, gtid, gnth, held); }))
+            break;
         if (a.ts && blockIdx.x == 0 && threadIdx.x == 0) a.ts[k] = global_ns();
     }
 }
