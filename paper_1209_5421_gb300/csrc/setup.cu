@@ -343,7 +343,7 @@ __global__ void k_children(int n, const int *__restrict__ parent, const int *__r
 }
 
 // ---------------------------------------------------------------------------------------
-// exact coarsest solve: dense A (pi order) -> Cholesky A = L L^t -> A^{-1} = L^{-t} L^{-1}.
+// exact coarsest solve: dense A (pi order) -> A = L D L^t -> A^{-1} = L^{-t} D^{-1} L^{-1}.
 // One CTA; n <= kMaxCoarsest. Bit 8 of err: not positive definite.
 __global__ void k_dense_from_sell(int n, const int *__restrict__ sl, const int *__restrict__ col,
                                   const double *__restrict__ val, double *__restrict__ a) {

@@ -188,7 +188,7 @@ __device__ __forceinline__ void rap_row(int P, const int *__restrict__ bptr,
 
 
 // ---------------------------------------------------------------------------------------
-// exact coarsest solve, one CTA: dense A -> Cholesky A = L L^t -> A^{-1} = L^{-t} L^{-1}.
+// exact coarsest solve, one CTA: dense A -> A = L D L^t -> A^{-1} = L^{-t} D^{-1} L^{-1}.
 // The factor and the inverse factor live in shared memory (smat, 2 n^2 doubles) when ga is
 // null -- the dense matrix then arrives in ainv --, else in the global scratch ga, gw. Bit 8
 // of err: not positive definite. ainv32 receives the inverse as float high parts, then low
@@ -200,46 +200,48 @@ __device__ __forceinline__ void chol_inverse_block(int n, double *ga, double *gw
     const bool in_smem = (ga == nullptr);
     double *a = in_smem ? smat : ga;
     double *w = in_smem ? smat + (size_t)n * n : gw;
-    __shared__ int bad;
+    __shared__ int bad;                  // first pivot that is not positive (n: none)
+    __shared__ double rd[kMaxCoarsest];  // reciprocal pivots
     const int t = threadIdx.x, T = blockDim.x;
-    if (t == 0) bad = 0;
-    if (in_smem)
-        for (int e = t; e < n * n; e += T) a[e] = ainv[e];  // the dense matrix arrives in ainv
-    __syncthreads();
     const int lane = t & 31, warp = t >> 5, nwarp = T >> 5;
-    for (int j = 0; j < n; j++) {
-        if (t == 0) {
-            double d = a[(size_t)j * n + j];
-            if (!(d > 0.0) || !isfinite(d)) bad = 1;
-            a[(size_t)j * n + j] = sqrt(fabs(d));
-        }
-        __syncthreads();
-        if (bad) break;
-        double djj = a[(size_t)j * n + j];
-        for (int i = j + 1 + t; i < n; i += T) a[(size_t)i * n + j] /= djj;
-        __syncthreads();
-        // trailing update of the lower triangle, a warp per row (each entry once per j)
+    for (int e = t; e < n * n; e += T) {
+        if (in_smem) a[e] = ainv[e];  // the dense matrix arrives in ainv
+        w[e] = e % (n + 1) == 0 ? 1.0 : 0.0;
+    }
+    auto pivot = [&](int j) {  // one thread
+        const double d = a[(size_t)j * n + j];
+        if ((!(d > 0.0) || !isfinite(d)) && bad == n) bad = j;
+        rd[j] = 1.0 / d;
+    };
+    if (t == 0) bad = n;
+    __syncthreads();
+    if (t == 0) pivot(0);
+    __syncthreads();
+    // A = L D L^t without storing L: step j takes l_ij = a_ij / d_j times row j off the rows below
+    // it, of A's lower triangle and of W (= I at the start, L^{-1} at the end); a warp per row.
+    // The first warp's row is the next pivot's: its reciprocal is taken while the others
+    // still work, so a step has one barrier, no square root and no division by others. Bound
+    // by the FP64 pipe (19 cycles per warp instruction) and the 64 steps: 260 -> 118 us for 64
+    // rows (Cholesky's three barriers, a square root and a division per column, then the
+    // inverse factor one column per thread: 43k dependent FP64 operations on two warps).
+    // (step j writes at most j + 1 into `bad`, so every thread leaves the loop at the same step)
+    for (int j = 0; j < n && j < bad; j++) {
+        const double r = rd[j];
         for (int i = j + 1 + warp; i < n; i += nwarp) {
-            const double lij = a[(size_t)i * n + j];
+            const double lij = a[(size_t)i * n + j] * r;
             for (int k = j + 1 + lane; k <= i; k += 32) a[(size_t)i * n + k] -= lij * a[(size_t)k * n + j];
+            if (i == j + 1 && lane == 0) pivot(i);
+            for (int c = lane; c <= j; c += 32) w[(size_t)i * n + c] -= lij * w[(size_t)j * n + c];
         }
         __syncthreads();
     }
-    if (bad) {
+    if (bad < n) {
         if (t == 0) atomicOr(err, 8);
         return;
     }
-    // W = L^{-1} (lower), one column per thread
-    for (int c = t; c < n; c += T) {
-        for (int i = 0; i < c; i++) w[(size_t)i * n + c] = 0.0;
-        for (int i = c; i < n; i++) {
-            double s = (i == c) ? 1.0 : 0.0;
-            for (int k = c; k < i; k++) s -= a[(size_t)i * n + k] * w[(size_t)k * n + c];
-            w[(size_t)i * n + c] = s / a[(size_t)i * n + i];
-        }
-    }
+    // A^{-1} = W^t D^{-1} W: D^{-1} W over A's triangle, then entry (i, j), i >= j, and its mirror
+    for (int e = t; e < n * n; e += T) a[e] = w[e] * rd[e / n];
     __syncthreads();
-    // A^{-1} = W^t W: entry (i, j), i >= j, and its mirror (the same sum: products commute)
     const int tri = n * (n + 1) / 2;
     for (int q = t; q < tri; q += T) {
         int i = (int)((sqrtf(8.0f * (float)q + 1.0f) - 1.0f) * 0.5f);  // q = i (i+1) / 2 + j
@@ -247,7 +249,7 @@ __device__ __forceinline__ void chol_inverse_block(int n, double *ga, double *gw
         while ((i + 1) * (i + 2) / 2 <= q) i++;
         const int j = q - i * (i + 1) / 2;
         double s = 0.0;
-        for (int k = i; k < n; k++) s += w[(size_t)k * n + i] * w[(size_t)k * n + j];
+        for (int k = i; k < n; k++) s += a[(size_t)k * n + i] * w[(size_t)k * n + j];
         const float hi = (float)s;  // FP32 cycle: high and low parts, s ~ hi + lo
         const float lo = (float)(s - (double)hi);
         for (int m = 0; m < (i == j ? 1 : 2); m++) {
