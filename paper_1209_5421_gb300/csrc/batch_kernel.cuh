@@ -13,6 +13,8 @@ namespace amg {
 template <class T>
 using BLev = LevelDev<T, int>;
 
+// levels of a system: the finest and at most 15 auxiliary ones (depth 14 to 0)
+constexpr int kBatchLevels = 16;
 constexpr int kBatchChunk = 64;  // directions orthogonalised against per pass
 constexpr int kBatchResume = 1000;  // status: the directions are full, the host adds more
 constexpr int kMaxTeam = 8;    // CTAs of one team at most
@@ -87,7 +89,7 @@ template <int NV>
 __device__ __forceinline__ void team_sum(const double (&v)[NV], double (&r)[NV]) {
     __shared__ double bc[4];
     double s[NV];
-    block_sum<NV, double>(v, s, BlockGroup{});
+    block_sum<NV, double>(v, s, SmallGroup{});
     if (bt_team.K == 1) {
         if (threadIdx.x == 0)
 #pragma unroll
@@ -258,14 +260,14 @@ __device__ __forceinline__ void bc_post(const BatchCycle<T, BIG> &c, int l, int 
         first_colour(c, l, op.f0, op.f1);
     }
     if (i > 0) {
-        op_multidot<BLev<T>, RM_TEAM>(L, op, rc, tid, nth, BlockGroup{});
+        op_multidot<BLev<T>, RM_TEAM>(L, op, rc, tid, nth, SmallGroup{});
         team_sync();
-        op_orth(L, op, tid, nth, BlockGroup{});
+        op_orth(L, op, tid, nth, SmallGroup{});
         team_sync();
     }
-    op_spmv_dot<BLev<T>, RM_TEAM>(L, op, rc, tid, nth, BlockGroup{});
+    op_spmv_dot<BLev<T>, RM_TEAM>(L, op, rc, tid, nth, SmallGroup{});
     team_sync();
-    op_update<BLev<T>, RM_TEAM>(L, op, rc, tid, nth, BlockGroup{});
+    op_update<BLev<T>, RM_TEAM>(L, op, rc, tid, nth, SmallGroup{});
     team_sync();
 }
 
@@ -485,7 +487,7 @@ k_batch(const BatchProb<T> *__restrict__ probs, const int4 *__restrict__ slots, 
         double *team_part, unsigned int *team_cnt, unsigned long long bar_limit_ns,
         int bar_extra, int *resume) {
     __shared__ BatchProb<T> sp;
-    __shared__ BLev<T> stab[kMaxLevels];
+    __shared__ BLev<T> stab[kBatchLevels];
     __shared__ int q;
     for (;;) {
         if (threadIdx.x == 0) q = atomicAdd(next, 1);

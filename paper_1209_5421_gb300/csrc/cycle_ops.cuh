@@ -150,8 +150,15 @@ __device__ __forceinline__ typename LV::val_t *vec_of(const LV &L, int sel) {
 // ---------------------------------------------------------------------------------------
 // the threads of one CTA that run an op together, and the barrier they meet at
 struct BlockGroup {  // every thread of the CTA; barrier 0
+    static constexpr bool small = false;
     __device__ __forceinline__ void sync() const { __syncthreads(); }
     __device__ __forceinline__ int nwarps() const { return (blockDim.x + 31) >> 5; }
+};
+// the same with sums that need little shared memory (the batch kernel: with 1024 threads its
+// 16 KB of static shared memory were just below a step of the L1 / shared split, and 128 bytes
+// more cost the 256-system batch 12%)
+struct SmallGroup : BlockGroup {
+    static constexpr bool small = true;
 };
 
 // ---------------------------------------------------------------------------------------
@@ -163,9 +170,32 @@ enum : int { RM_LASTBLOCK = 0, RM_BLOCK = 1, RM_PARTIAL = 2, RM_TEAM = 3 };
 // per-warp sums) and only the sum over CTAs is FP64; FP64 partials go through shared memory
 // and one warp sums them (32 values per lane in fixed order, then a 5-level shuffle tree),
 // about one FP64 add per partial instead of five for a shuffle tree over every warp.
+template <int N>
 __device__ __forceinline__ double *red_scratch() {
-    __shared__ double s[1024];  // >= blockDim.x (1024 at most)
+    __shared__ double s[N];
     return s;
+}
+
+// Sums of P values (a power of two) over a warp, all at once: each exchange halves the values a
+// lane carries, so P values take P - 1 + 5 - log2 P additions instead of 5 P. Value v ends in
+// lanes [32 v / P, 32 (v + 1) / P).
+template <int P>
+__device__ __forceinline__ double warp_sums(double (&k)[P]) {
+    constexpr int LP = P == 8 ? 3 : P == 4 ? 2 : P == 2 ? 1 : 0;
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int l = 0; l < LP; l++) {  // lanes with bit 4 - l set keep the upper half
+        const int o = 16 >> l, h = P >> (l + 1);
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < h; i++) {
+            const double give = up ? k[i] : k[i + h], keep = up ? k[i + h] : k[i];
+            k[i] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+#pragma unroll
+    for (int o = 16 >> LP; o > 0; o >>= 1) k[0] += __shfl_xor_sync(0xffffffffu, k[0], o);
+    return k[0];
 }
 
 __device__ __forceinline__ double warp_sum(double y) {
@@ -179,9 +209,9 @@ __device__ __forceinline__ double warp_sum(double y) {
 // between two ops, and no op reduces twice).
 template <int NV, class A, class G>
 __device__ __forceinline__ void block_sum(const A (&v)[NV], double (&r)[NV], const G &g) {
-    double *s = red_scratch();
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nw = g.nwarps();
     if constexpr (sizeof(A) == 4) {
+        double *s = red_scratch<128>();  // (the size the small FP64 sums use: one array)
         // FP32 cycle: a warp tree, then one warp combines the per-warp sums, all in FP32
         float *sf = reinterpret_cast<float *>(s);
 #pragma unroll
@@ -200,17 +230,51 @@ __device__ __forceinline__ void block_sum(const A (&v)[NV], double (&r)[NV], con
                 for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
                 r[k] = (double)x;
             }
+    } else if constexpr (G::small) {
+        // every warp sums its own partials, one warp the warps'
+        constexpr int P = NV > 2 ? 4 : NV;
+        static_assert(NV <= 4, "scratch of four values");
+        double *s = red_scratch<128>();
+        double k[P];
+#pragma unroll
+        for (int i = 0; i < P; i++) k[i] = i < NV ? (double)v[i < NV ? i : 0] : 0.0;
+        double y = warp_sums<P>(k);
+        if ((lane & (32 / P - 1)) == 0) s[32 * (lane / (32 / P)) + w] = y;
+        g.sync();
+        if (w == 0) {
+#pragma unroll
+            for (int i = 0; i < P; i++) k[i] = lane < nw ? s[32 * i + lane] : 0.0;
+            y = warp_sums<P>(k);
+#pragma unroll
+            for (int i = 0; i < NV; i++) r[i] = i == 0 ? y : __shfl_sync(0xffffffffu, y, 32 / P * i);
+        }
     } else {
+        double *s = red_scratch<1024>();  // >= blockDim.x
+        // A warp's FP64 instruction takes 64 cycles, of four warps (one per scheduler) together 76:
+        // four warps share a value's partials, and one adds the four sums of every value. 256
+        // threads, one value: 13 dependent additions -> 8; 1024: 37 -> 14.
+        __shared__ double part[4 * NV];
+        const int nq = nw < 4 ? nw : 4;
 #pragma unroll
         for (int k = 0; k < NV; k++) {
             if (k > 0) g.sync();
             s[threadIdx.x] = (double)v[k];
             g.sync();
-            if (w == 0) {
+            if (w < nq) {
                 double y = 0.0;
-                for (int j = lane; j < 32 * nw; j += 32) y += s[j];
-                r[k] = warp_sum(y);
+                for (int j = 32 * w + lane; j < 32 * nw; j += 32 * nq) y += s[j];
+                y = warp_sum(y);
+                if (lane == 0) part[4 * k + w] = y;
             }
+        }
+        g.sync();
+        if (w == 0) {
+            static_assert(NV <= 8, "one lane per partial sum");
+            double y = (lane < 4 * NV && (lane & 3) < nq) ? part[lane] : 0.0;
+            y += __shfl_down_sync(0xffffffffu, y, 2);
+            y += __shfl_down_sync(0xffffffffu, y, 1);
+#pragma unroll
+            for (int k = 0; k < NV; k++) r[k] = k == 0 ? y : __shfl_sync(0xffffffffu, y, 4 * k);
         }
     }
 }
@@ -1086,7 +1150,13 @@ __device__ void op_multidot(const LV &L, const Op &op, const RedCtx &rc, int tid
     double *out[kMaxKcycle];
 #pragma unroll
     for (int j = 0; j < kMaxKcycle; j++) out[j] = j < i ? &L.sc[SC_ZQ0 + j] : nullptr;
-    reduce_store<kMaxKcycle, RM, T>(v, out, rc, op.red_pb, g);
+    if (i == 1) {  // the usual two steps: one value (every further one costs its own tree)
+        const T v1[1] = {v[0]};
+        double *out1[1] = {out[0]};
+        reduce_store<1, RM, T>(v1, out1, rc, op.red_pb, g);
+    } else {
+        reduce_store<kMaxKcycle, RM, T>(v, out, rc, op.red_pb, g);
+    }
 }
 
 // a / b for an Alg. 1 coefficient: in FP64 for the FP64 cycle, in FP32 for the FP32 cycle

@@ -74,29 +74,28 @@ __global__ void __launch_bounds__(kRedThreads) k_op(const GLev<T> *__restrict__ 
 // ---------------------------------------------------------------------------------------
 // persistent cycle kernel
 // sum the per-CTA partials of the previous op (every CTA, identical order) into sc; one
-// warp does it, in FP64 for the FP64 cycle and in FP32 for the FP32 cycle (whose per-CTA
+// warp per value, in FP64 for the FP64 cycle and in FP32 for the FP32 cycle (whose per-CTA
 // partials are FP32 sums)
 template <class T, class TAB>
 __device__ __forceinline__ void finalize(const CycleArgs<T> &a, const TAB *tab, const Op &op) {
-    if (threadIdx.x < 32) {
+    const int k = (int)threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (k < op.fin_n) {  // a warp per value
         const int G = gridDim.x;
         double *sc = tab[op.fin_level].sc;
-        for (int k = 0; k < op.fin_n; k++) {
-            const double *part = a.partials + ((size_t)op.fin_pb * 4 + k) * G;
-            double y;
-            if constexpr (sizeof(T) == 4) {
-                float x = 0.f;
-                for (int b = threadIdx.x; b < G; b += 32) x += (float)__ldcg(&part[b]);
+        const double *part = a.partials + ((size_t)op.fin_pb * 4 + k) * G;
+        double y;
+        if constexpr (sizeof(T) == 4) {
+            float x = 0.f;
+            for (int b = lane; b < G; b += 32) x += (float)__ldcg(&part[b]);
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-                y = (double)x;
-            } else {
-                y = 0.0;
-                for (int b = threadIdx.x; b < G; b += 32) y += __ldcg(&part[b]);
-                y = warp_sum(y);
-            }
-            if (threadIdx.x == 0 && op.fin_dst[k] >= 0) sc[op.fin_dst[k]] = y;
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
+            y = (double)x;
+        } else {
+            y = 0.0;
+            for (int b = lane; b < G; b += 32) y += __ldcg(&part[b]);
+            y = warp_sum(y);
         }
+        if (lane == 0 && op.fin_dst[k] >= 0) sc[op.fin_dst[k]] = y;
     }
     __syncthreads();
 }
@@ -237,31 +236,86 @@ __global__ void __launch_bounds__(kRedThreads) k_true_residual(GLev<double> L,
 }
 
 // outer scalars: osc[OS_BB] = (b,b), osc[OS_RR] = (r,r), osc[OS_STOP] = breakdown flag,
-// osc[OS_RP] = (r, p_i), osc[OS_TT] = (t, t), osc[OS_ZQ + j] = (z, A p_j); (p_j, A p_j) in opq
-enum : int { OS_BB = 0, OS_RR = 1, OS_STOP = 2, OS_RP = 4, OS_TT = 5, OS_ZQ = 8 };
+// osc[OS_RP] = (r, p_i), osc[OS_TT] = (t, t), osc[OS_ERR] = the cycle's error flag (copied here by
+// an iteration's last kernel: one read back per iteration), osc[OS_ZQ + j] = (z, A p_j);
+// (p_j, A p_j) in opq
+enum : int { OS_BB = 0, OS_RR = 1, OS_STOP = 2, OS_RP = 4, OS_TT = 5, OS_ERR = 7, OS_ZQ = 8 };
 
 // Dots of w with the basis vectors V[0..m), kDotChunk vectors per sweep over the rows: each
 // thread keeps one grid-stride partial sum per vector (in row order), each block reduces them
 // vector by vector, and the last block to finish sums the block partials in block order.
 constexpr int kDotChunk = 8;
 
-__device__ __forceinline__ void mdot_chunk(int n, const double *__restrict__ w,
-                                           double *const *__restrict__ V, int c0, int mc,
-                                           double *partials) {
-    const double *vp[kDotChunk];
+// partial sums of a[0..M) over the block into partials[(c0 + i) gridDim.x + block], i < M
+template <int M>
+__device__ __forceinline__ void mdot_block_sum(double (&a)[M], int c0, double *partials) {
+    constexpr int P = M > 4 ? 8 : M > 2 ? 4 : M;
+    __shared__ double part[8][kRedThreads / 32];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    double k[P];
 #pragma unroll
-    for (int i = 0; i < kDotChunk; i++) vp[i] = i < mc ? V[c0 + i] : nullptr;
-    double a[kDotChunk] = {}, r[kDotChunk];
+    for (int i = 0; i < P; i++) k[i] = i < M ? a[i < M ? i : 0] : 0.0;
+    const double y = warp_sums<P>(k);
+    const int v = lane / (32 / P);  // the value this lane ends with
+    if ((lane & (32 / P - 1)) == 0 && v < M) part[v][w] = y;
+    __syncthreads();
+    if (w < M) {  // a warp per value
+        double y = lane < kRedThreads / 32 ? part[w][lane] : 0.0;
+#pragma unroll
+        for (int o = kRedThreads / 64; o > 0; o >>= 1) y += __shfl_down_sync(0xffffffffu, y, o);
+        if (lane == 0) partials[(size_t)(c0 + w) * gridDim.x + blockIdx.x] = y;
+    }
+    __syncthreads();  // `part` is reused by the next chunk
+}
+
+// dots of w with V[c0 .. c0 + M). M is exact: an FP64 instruction that is predicated off takes
+// its 64 cycles all the same, and these kernels are bound by the FP64 pipe (2.0M rows, one
+// vector: 35 us with eight predicated products per row, 10 with one; eight vectors: 37)
+template <int M>
+__device__ __forceinline__ void mdot_exact(int n, const double *__restrict__ w,
+                                           double *const *__restrict__ V, int c0, double *partials) {
+    const double *vp[M];
+    double a[M];
+#pragma unroll
+    for (int i = 0; i < M; i++) {
+        vp[i] = V[c0 + i];
+        a[i] = 0.0;
+    }
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
         const double wk = w[k];
 #pragma unroll
-        for (int i = 0; i < kDotChunk; i++)
-            if (i < mc) a[i] += wk * vp[i][k];
+        for (int i = 0; i < M; i++) a[i] += wk * vp[i][k];
     }
-    block_sum<kDotChunk, double>(a, r, BlockGroup{});
-    if (threadIdx.x == 0)
-        for (int i = 0; i < mc; i++) partials[(size_t)(c0 + i) * gridDim.x + blockIdx.x] = r[i];
-    __syncthreads();  // the reduction scratch is reused by the next chunk
+    mdot_block_sum<M>(a, c0, partials);
+}
+__device__ __forceinline__ void mdot_chunk(int n, const double *__restrict__ w,
+                                           double *const *__restrict__ V, int c0, int mc,
+                                           double *partials) {
+    switch (mc) {
+        case 1: mdot_exact<1>(n, w, V, c0, partials); break;
+        case 2: mdot_exact<2>(n, w, V, c0, partials); break;
+        case 3: mdot_exact<3>(n, w, V, c0, partials); break;
+        case 4: mdot_exact<4>(n, w, V, c0, partials); break;
+        case 5: mdot_exact<5>(n, w, V, c0, partials); break;
+        case 6: mdot_exact<6>(n, w, V, c0, partials); break;
+        case 7: mdot_exact<7>(n, w, V, c0, partials); break;
+        default: mdot_exact<8>(n, w, V, c0, partials); break;
+    }
+}
+
+// x - sum_{i < m} c[i] V[i][k], in order; four vectors' loads at a time
+__device__ __forceinline__ double minus_combination(double x, int k, double *const *__restrict__ V, int m,
+                                                    const double *__restrict__ c) {
+    int i = 0;
+    for (; i + 4 <= m; i += 4) {
+        const double v0 = V[i][k], v1 = V[i + 1][k], v2 = V[i + 2][k], v3 = V[i + 3][k];
+        x -= c[i] * v0;
+        x -= c[i + 1] * v1;
+        x -= c[i + 2] * v2;
+        x -= c[i + 3] * v3;
+    }
+    for (; i < m; i++) x -= c[i] * V[i][k];
+    return x;
 }
 
 __device__ __forceinline__ void mdot_finish(int m, double *out, const RedCtx &rc) {
@@ -290,8 +344,7 @@ __device__ __forceinline__ void mdot_finish(int m, double *out, const RedCtx &rc
 // (z, q_j) for all j < it: each block loops over j; the last block reduces every j
 __global__ void __launch_bounds__(kRedThreads, 4)
     k_outer_multidot(int n, const double *__restrict__ z, double *const *__restrict__ Q,
-                     const int *__restrict__ it_ptr, double *osc, RedCtx rc) {
-    const int it = *it_ptr;
+                     int it, double *osc, RedCtx rc) {
     for (int c0 = 0; c0 < it; c0 += kDotChunk)
         mdot_chunk(n, z, Q, c0, min(kDotChunk, it - c0), rc.partials);
     mdot_finish(it, osc + OS_ZQ, rc);
@@ -303,9 +356,8 @@ __global__ void __launch_bounds__(kRedThreads, 4)
 constexpr int kOrthCoef = 256;
 
 __global__ void k_outer_orth(int n, const double *__restrict__ z, double *const *__restrict__ P,
-                             const int *__restrict__ it_ptr, const double *__restrict__ osc,
+                             int it, const double *__restrict__ osc,
                              const double *__restrict__ opq) {
-    const int it = *it_ptr;
     __shared__ double cf[kOrthCoef];
     for (int j = threadIdx.x; j < it && j < kOrthCoef; j += blockDim.x)
         cf[j] = -osc[OS_ZQ + j] / opq[j];
@@ -313,7 +365,15 @@ __global__ void k_outer_orth(int n, const double *__restrict__ z, double *const 
     double *p = P[it];
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         double acc = z[i];
-        for (int j = 0; j < it; j++)
+        int j = 0;
+        for (; j + 4 <= it && j + 4 <= kOrthCoef; j += 4) {  // four vectors' loads at a time
+            const double v0 = P[j][i], v1 = P[j + 1][i], v2 = P[j + 2][i], v3 = P[j + 3][i];
+            acc += cf[j] * v0;
+            acc += cf[j + 1] * v1;
+            acc += cf[j + 2] * v2;
+            acc += cf[j + 3] * v3;
+        }
+        for (; j < it; j++)
             acc += (j < kOrthCoef ? cf[j] : -osc[OS_ZQ + j] / opq[j]) * P[j][i];
         p[i] = acc;
     }
@@ -323,11 +383,10 @@ __global__ void k_outer_orth(int n, const double *__restrict__ z, double *const 
 __global__ void __launch_bounds__(kRedThreads) k_outer_spmv_dot(GLev<double> L,
                                                                 double *const *__restrict__ P,
                                                                 double *const *__restrict__ Q,
-                                                                const int *__restrict__ it_ptr,
+                                                                int it,
                                                                 const double *__restrict__ r,
                                                                 double *osc, double *opq,
                                                                 RedCtx rc) {
-    const int it = *it_ptr;
     const double *p = P[it];
     double *q = Q[it];
     double v[2] = {0.0, 0.0};
@@ -346,11 +405,10 @@ __global__ void __launch_bounds__(kRedThreads) k_outer_spmv_dot(GLev<double> L,
 // alpha = (r, p) / (p, Ap); x += alpha p; r -= alpha q; (r, r)
 __global__ void __launch_bounds__(kRedThreads) k_outer_update(int n, double *const *__restrict__ P,
                                                               double *const *__restrict__ Q,
-                                                              int *it_ptr, double *__restrict__ x,
+                                                              int it, double *__restrict__ x,
                                                               double *__restrict__ r, double *osc,
                                                               const double *__restrict__ opq,
-                                                              RedCtx rc) {
-    const int it = *it_ptr;
+                                                              const int *err, RedCtx rc) {
     const double pq = opq[it];
     const bool bad = !(pq > 0.0) || !isfinite(pq);
     __shared__ double alpha_s;  // one FP64 division per block, not per thread
@@ -368,13 +426,11 @@ __global__ void __launch_bounds__(kRedThreads) k_outer_update(int n, double *con
     }
     double *out[1] = {&osc[OS_RR]};
     reduce_store<1, RM_LASTBLOCK, double>(v, out, rc, 0, BlockGroup{});
-    if (blockIdx.x == 0 && threadIdx.x == 0 && bad) osc[OS_STOP] = 1.0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        if (bad) osc[OS_STOP] = 1.0;
+        osc[OS_ERR] = (double)*err;
+    }
 }
-
-__global__ void k_bump(int *it_ptr) {
-    if (threadIdx.x == 0 && blockIdx.x == 0) *it_ptr += 1;
-}
-
 
 // ---------------------------------------------------------------------------------------
 // FGMRES kernels (FP64, pi order); V and Z are arrays of vector pointers
@@ -404,9 +460,7 @@ __global__ void __launch_bounds__(kRedThreads, 4) k_orth_mdot(int n, double *__r
                                                            const double *__restrict__ c,
                                                            double *out, RedCtx rc) {
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        double x = w[k];
-        for (int i = 0; i < m; i++) x -= c[i] * V[i][k];
-        w[k] = x;
+        w[k] = minus_combination(w[k], k, V, m, c);
     }
     for (int c0 = 0; c0 < m; c0 += kDotChunk)
         mdot_chunk(n, w, V, c0, min(kDotChunk, m - c0), rc.partials);
@@ -417,16 +471,17 @@ __global__ void __launch_bounds__(kRedThreads, 4) k_orth_mdot(int n, double *__r
 __global__ void __launch_bounds__(kRedThreads) k_orth_sub(int n, double *__restrict__ w,
                                                           double *const *__restrict__ V, int m,
                                                           const double *__restrict__ c,
-                                                          double *nrm2, RedCtx rc) {
+                                                          double *nrm2, const int *err,
+                                                          double *err_out, RedCtx rc) {
     double a[1] = {0.0};
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-        double x = w[k];
-        for (int i = 0; i < m; i++) x -= c[i] * V[i][k];
+        const double x = minus_combination(w[k], k, V, m, c);
         w[k] = x;
         a[0] += x * x;
     }
     double *o[1] = {nrm2};
     reduce_store<1, RM_LASTBLOCK, double>(a, o, rc, 0, BlockGroup{});
+    if (blockIdx.x == 0 && threadIdx.x == 0) *err_out = (double)*err;
 }
 
 // v = w * s
@@ -1786,7 +1841,6 @@ int solve(amg_hierarchy *h, const double *b_nat, double tol, double *x_nat, int 
     AMG_CUDA(cudaMemcpyAsync(h->ro, h->bo, sizeof(double) * n, cudaMemcpyDeviceToDevice, s));
     AMG_CUDA(cudaMemsetAsync(h->xo, 0, sizeof(double) * n, s));
     AMG_CUDA(cudaMemsetAsync(h->osc, 0, sizeof(double) * 8, s));
-    AMG_CUDA(cudaMemsetAsync(h->oit, 0, sizeof(int), s));
     k_norm2<<<red_grid(n), kRedThreads, 0, s>>>(n, h->bo, h->osc + OS_BB, rc);
     AMG_LAUNCH_CHECK();
     AMG_CUDA(cudaMemcpyAsync(h->h_pinned, h->osc, sizeof(double) * 8, cudaMemcpyDeviceToHost, s));
@@ -1808,29 +1862,28 @@ int solve(amg_hierarchy *h, const double *b_nat, double tol, double *x_nat, int 
             apply_preconditioner(h);  // zo = B^[ro]
             Profiler::Rec rec{};
             if (prof) rec = h->prof->begin(K_OUTER_MULTIDOT, 0, 8.0 * nd * (1 + it), s);
-            k_outer_multidot<<<red_grid(n), kRedThreads, 0, s>>>(n, h->zo, h->dQ, h->oit, h->osc, rc);
+            k_outer_multidot<<<red_grid(n), kRedThreads, 0, s>>>(n, h->zo, h->dQ, it, h->osc, rc);
             AMG_LAUNCH_CHECK();
             if (prof) h->prof->end(rec, s);
             if (prof) rec = h->prof->begin(K_OUTER_ORTH, 0, 8.0 * nd * (2 + it), s);
-            k_outer_orth<<<nblocks_for(n, 256), 256, 0, s>>>(n, h->zo, h->dP, h->oit, h->osc, opq);
+            k_outer_orth<<<nblocks_for(n, 256), 256, 0, s>>>(n, h->zo, h->dP, it, h->osc, opq);
             AMG_LAUNCH_CHECK();
             if (prof) h->prof->end(rec, s);
             if (prof) rec = h->prof->begin(K_OUTER_SPMV_DOT, 0, 12.0 * nnz + 24.0 * nd, s);
-            k_outer_spmv_dot<<<red_grid(n), kRedThreads, 0, s>>>(Lf, h->dP, h->dQ, h->oit, h->ro,
+            k_outer_spmv_dot<<<red_grid(n), kRedThreads, 0, s>>>(Lf, h->dP, h->dQ, it, h->ro,
                                                                  h->osc, opq, rc);
             AMG_LAUNCH_CHECK();
             if (prof) h->prof->end(rec, s);
             if (prof) rec = h->prof->begin(K_OUTER_UPDATE, 0, 48.0 * nd, s);
-            k_outer_update<<<red_grid(n), kRedThreads, 0, s>>>(n, h->dP, h->dQ, h->oit, h->xo,
-                                                               h->ro, h->osc, opq, rc);
+            k_outer_update<<<red_grid(n), kRedThreads, 0, s>>>(n, h->dP, h->dQ, it, h->xo,
+                                                               h->ro, h->osc, opq,
+                                                               h->err_flag, rc);
             AMG_LAUNCH_CHECK();
             if (prof) h->prof->end(rec, s);
-            k_bump<<<1, 32, 0, s>>>(h->oit);
-            AMG_LAUNCH_CHECK();
             AMG_CUDA(cudaMemcpyAsync(h->h_pinned, h->osc, sizeof(double) * 8,
                                      cudaMemcpyDeviceToHost, s));
             AMG_CUDA(cudaStreamSynchronize(s));
-            if (h->nlev > 1) check_device_error(h);
+            if (h->nlev > 1) raise_device_error(h, (int)h->h_pinned[OS_ERR]);
             if (prof) {
                 h->prof->harvest();
                 if (h->nlev > 1) {
@@ -1959,22 +2012,18 @@ static int solve_fgmres(amg_hierarchy *h, const double *b_nat, double tol, doubl
             AMG_LAUNCH_CHECK();
             if (prof) h->prof->end(rec, s);
             if (prof) rec = h->prof->begin(K_FGMRES_ORTH, 0, 8.0 * nd * (j + 3), s);
-            k_orth_sub<<<red_grid(n), kRedThreads, 0, s>>>(n, w, dV, j + 1, dh2, dh + j + 1, rc);
+            k_orth_sub<<<red_grid(n), kRedThreads, 0, s>>>(n, w, dV, j + 1, dh2, dh + j + 1, h->err_flag,
+                                                          h->osc + OS_ERR, rc);
             AMG_LAUNCH_CHECK();
             if (prof) h->prof->end(rec, s);
-            {  // h1, the norm, h2 and the cycle's error flag: one round trip
-                int err = 0;
-                AMG_CUDA(cudaMemcpyAsync(h->h_pinned, dh, sizeof(double) * (j + 2),
+            {  // the cycle's error flag, h1 and the norm, h2: one read back of [OS_ERR, dh2 + j + 1)
+                const double *hp = h->h_pinned;
+                AMG_CUDA(cudaMemcpyAsync(h->h_pinned, h->osc + OS_ERR, sizeof(double) * (1 + m + 2 + j + 1),
                                          cudaMemcpyDeviceToHost, s));
-                AMG_CUDA(cudaMemcpyAsync(h->h_pinned + m + 2, dh2, sizeof(double) * (j + 1),
-                                         cudaMemcpyDeviceToHost, s));
-                if (h->nlev > 1)
-                    AMG_CUDA(cudaMemcpyAsync(&err, h->err_flag, sizeof(int), cudaMemcpyDeviceToHost, s));
                 AMG_CUDA(cudaStreamSynchronize(s));
-                raise_device_error(h, err);
-                for (int i = 0; i < j + 2; i++) hv[i] = h->h_pinned[i];
-                for (int i = 0; i <= j; i++)
-                    H[(size_t)i * m + j] = (0.0 + hv[i]) + h->h_pinned[m + 2 + i];
+                if (h->nlev > 1) raise_device_error(h, (int)hp[0]);
+                for (int i = 0; i < j + 2; i++) hv[i] = hp[1 + i];
+                for (int i = 0; i <= j; i++) H[(size_t)i * m + j] = (0.0 + hv[i]) + hp[1 + m + 2 + i];
             }
             if (prof) {
                 h->prof->harvest();
