@@ -34,8 +34,10 @@
 // The level above the coarsest: B^ there is linear (the coarsest solve is exact), so setup
 // forms M = B^ and A M as dense matrices once (k_dense_cycle, FP64), each CTA keeps 1/16 of
 // their rows, and one product with a residual gives p and A p of an Alg. 1 step; that replaces
-// about 13 dependent steps. Where the matrices do not fit, the level is swept like the others
-// and the coarsest solve is the dense product.
+// about 13 dependent steps. FP64 keeps M alone and multiplies by the sparse A after it (256
+// rows: a product with both is 4,900 cycles of the FP64 pipe, with M 2,450 and one more gather
+// 600: 9.7 -> 8.8 us per visit). Where the matrices do not fit, the level is swept like the
+// others and the coarsest solve is the dense product.
 #pragma once
 
 #include <cstddef>
@@ -96,6 +98,7 @@ struct ClLayout {
     int kc, nu_pre, nu_post;
     int nd, ch, stride;  // dense level: rows, rows per CTA (multiple of 4), row stride
     int mat, mat_lo;     // M then A M (or the inverse; FP32: high parts, low parts)
+    int aw, aval, acol;  // FP64: M alone, and A's rows: slots per row, values, columns
     int dhead, down;     // gather into the dense level: own rows (count; their pi-rows)
     int peers;           // neighbour CTAs: count, ranks
     int levels;          // lv[] (a copy in the image)
@@ -274,7 +277,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
     constexpr int NR = kClRanks;
     __shared__ __align__(8) unsigned long long mbs[5];   // neighbours x 2, all CTAs x 2, image
     __shared__ __align__(16) T red[2][NR * kClWarps][2]; // sums over the cluster: the warps'
-    __shared__ T coef_s[4];
+    __shared__ T coef_s[6];
     __shared__ T pqs[kClLevels + 1][kMaxKcycle];         // (p_i, A p_i) of every level; FP64:
                                                          //   its reciprocal (0: not positive)
     __shared__ int stops[kClLevels + 1][kMaxKcycle];     // Alg. 1 stopped at or before step i
@@ -759,9 +762,24 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
         {
             const int ch = y.ch, len = NR * ch;
             T *E = vec(y.E), *out = vec(y.out), *Rv = vec(y.Rv);
-            const int nsteps = y.dense ? y.kc : 1, parts = y.dense ? 2 : 1;
+            const int nsteps = y.dense ? y.kc : 1, parts = y.dense && !F64 ? 2 : 1;
             constexpr int LPR = 8;  // lanes per row
             constexpr int V = 16 / (int)sizeof(T);
+            // this CTA's rows of a product (in `out`: `parts` times ch values) to every CTA
+            auto gather_out = [&](int o0, int o1) {
+                __syncthreads();
+                const uint32_t mb = mb_a();
+                const int per = ch / V;
+                if (alive)
+#pragma unroll 1
+                    for (int k = tid; k < NR * parts * per; k += kClThreads) {
+                        const int piece = k >> 4, part = piece >= per, o = (piece - part * per) * V;
+                        const uint32_t to = dyn + (part ? o1 : o0) + (uint32_t)sizeof(T) * (rank * ch + o);
+                        cl_store16(cl_map(to, k & (NR - 1)), out + part * ch + o, cl_map(mb, k & (NR - 1)));
+                    }
+                arrive(mb, (int)sizeof(T) * parts * len);
+                wait_a();
+            };
 #pragma unroll 1
             for (int st = 0; st < nsteps; st++) {
                 const T *r = st == 0 ? vec(y.F) : Rv;
@@ -813,19 +831,21 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                     }
                     if (q == 0) out[row] = sum;
                 }
-                __syncthreads();
-                {  // this CTA's part of the product to every CTA
-                    const uint32_t mb = mb_a();
-                    const int per = ch / V, o0 = y.dense ? y.P[st] : y.E, o1 = y.Q[st];
-                    if (alive)
+                gather_out(y.dense ? y.P[st] : y.E, y.Q[st]);
+                if (F64 && y.dense) {  // w = A z: four lanes per row
+                    const T *z = vec(y.P[st]), *av = vec(y.aval);
+                    const unsigned short *ac = (const unsigned short *)at(y.acol);
+                    const int row = tid >> 2;
+                    if (32 * warp < 4 * ch) {
+                        T sum = 0;
+                        if (row < ch)
 #pragma unroll 1
-                        for (int k = tid; k < NR * parts * per; k += kClThreads) {
-                            const int piece = k >> 4, part = piece >= per, o = (piece - part * per) * V;
-                            const uint32_t to = dyn + (part ? o1 : o0) + (uint32_t)sizeof(T) * (rank * ch + o);
-                            cl_store16(cl_map(to, k & (NR - 1)), out + part * ch + o, cl_map(mb, k & (NR - 1)));
-                        }
-                    arrive(mb, (int)sizeof(T) * parts * len);
-                    wait_a();
+                            for (int k = tid & 3; k < y.aw; k += 4) sum += av[k * ch + row] * z[ac[k * ch + row]];
+                        sum += __shfl_xor_sync(0xffffffffu, sum, 1);
+                        sum += __shfl_xor_sync(0xffffffffu, sum, 2);
+                        if (row < ch && (tid & 3) == 0) out[row] = sum;
+                    }
+                    gather_out(y.Q[st], 0);
                 }
                 if (!y.dense) break;
                 // Alg. 1 step st, the same in every CTA: beta_j for j < st, then alpha
@@ -856,22 +876,22 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                             keep_pq(kClLevels, st, s0);
                         }
                         __syncthreads();  // every warp has read what changes now
-                    } else {  // warp k sums value k; one thread each for the coefficients
-                        if (warp < 2) {
-                            const T *u1 = warp == 0 ? qj : r;
+                    } else {  // two warps per value; one thread each for the coefficients
+                        if (warp < 4) {
+                            const T *u1 = warp < 2 ? qj : r;
                             T x = 0;
 #pragma unroll 4
-                            for (int k = lane; k < len; k += 32) x += p[k] * u1[k];
+                            for (int k = lane + 32 * (warp & 1); k < len; k += 64) x += p[k] * u1[k];
 #pragma unroll
                             for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
                             if (lane == 0) coef_s[1 + warp] = x;
                         }
                         __syncthreads();
                         if (tid == 0)
-                            coef_s[0] = j < st ? beta(kClLevels, j, coef_s[1])
-                                               : alpha(kClLevels, st, coef_s[1], coef_s[2]);
+                            coef_s[0] = j < st ? beta(kClLevels, j, coef_s[1] + coef_s[2])
+                                               : alpha(kClLevels, st, coef_s[1] + coef_s[2], coef_s[3] + coef_s[4]);
                         else if (tid == 32 && j == st)
-                            keep_pq(kClLevels, st, coef_s[1]);
+                            keep_pq(kClLevels, st, coef_s[1] + coef_s[2]);
                         __syncthreads();
                         c = coef_s[0];
                     }
@@ -1156,7 +1176,20 @@ __global__ void k_cl_image(const __grid_constant__ ClSrcs G, const __grid_consta
     unsigned char *im = image + (size_t)r * y.image_bytes;
     const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
     if (a == y.nsp) {
-        if (y.dense) return;
+        if (y.dense) {  // FP64: A's rows (columns are pi-rows)
+            if constexpr (sizeof(T) == 8) {
+                const ClSrc &S = G.lv[a];
+                for (int k = t0; k < y.ch * y.aw; k += nt) {
+                    const int row = k % y.ch, slot = k / y.ch, i = r * y.ch + row;
+                    if (i >= y.nd) continue;
+                    const int s0 = S.sl[i >> 5], width = (S.sl[(i >> 5) + 1] - s0) >> 5;
+                    const int o = s0 + 32 * slot + (i & 31), j = slot < width ? S.col[o] : -1;
+                    ((unsigned short *)(im + y.acol))[k] = (unsigned short)(j >= 0 ? j : i);
+                    ((double *)(im + y.aval))[k] = j >= 0 ? S.val64[o] : 0.0;
+                }
+            }
+            return;
+        }
         for (int k = t0; k < y.ch * y.nd; k += nt) {
             const int row = k / y.nd, j = k - row * y.nd, i = r * y.ch + row;
             if (i >= y.nd) continue;
@@ -1308,7 +1341,7 @@ k_dense_cycle(const __grid_constant__ ClSrc S, const __grid_constant__ ClLayout 
     for (int i = tid; i < n; i += nt) {
         T *row = (T *)(image + (size_t)(i / y.ch) * y.image_bytes + y.mat) + (size_t)(i % y.ch) * y.stride;
         row[unit] = (T)z[i];
-        row[(size_t)y.ch * y.stride + unit] = (T)dot(i, 0);
+        if constexpr (sizeof(T) == 4) row[(size_t)y.ch * y.stride + unit] = (T)dot(i, 0);
     }
 }
 

@@ -1190,7 +1190,12 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
         L.child = take(2 * (size_t)nch * L.Rn);
     }
     y.top = take(sizeof(int) * max_own[0]);
-    y.mat = take((size_t)(dense ? 2 : 1) * y.ch * y.stride * vb);
+    y.mat = take((size_t)(dense && vb == 4 ? 2 : 1) * y.ch * y.stride * vb);
+    if (dense && vb == 8) {
+        y.aw = widths[level0 + y.nsp];
+        y.aval = take((size_t)y.aw * y.ch * vb);
+        y.acol = take((size_t)y.aw * y.ch * 2);
+    }
     if (!dense && vb == 4) y.mat_lo = take((size_t)y.ch * y.stride * vb);
     y.image_bytes = (int)off;
     for (int a = 0; a < y.nsp; a++) {
