@@ -83,12 +83,13 @@ struct __align__(16) ClLev {
     int dinv, dst, over, head; //   1 / a_ii, destinations (and further ones), ClHead
     int lg, ns;        // log2 of the lanes per row; off-diagonal slots a lane takes (even)
     int R;             // stride of the matrix tables (largest strip's rows times lanes)
-    int xchild;        // 1: a child of an own next-level row may lie in another strip
+    int kind;          // 1: a child of an own next-level row may lie in another strip; 2: the
+                       //   finest level (block smoother)
     int pre, post, npre, npost;  // sweeps (ClOp) and their lengths
     int parent, child, nch, Rn;  // maps; children per row of the next level's rows, stride
     int rhs, r, e, nact;       // vectors: by own row, by window index; warps with rows in sums
     int p[kMaxKcycle], q[kMaxKcycle];
-    int level, ncol, w, pad;
+    int level, ncol, w, blk;   // blk: finest level, first own row of each own block
 };
 
 struct ClLayout {
@@ -388,7 +389,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
     __syncthreads();
     // ---- the level's constants ----------------------------------------------------------
     // (in registers: every wait and store makes the compiler read shared memory again)
-    uint4 lt0{}, lt1{}, lt2{};  // ClLev: own, col, val, diag | dinv, dst, over, head | lg, ns, R, xchild
+    uint4 lt0{}, lt1{}, lt2{};  // ClLev: own, col, val, diag | dinv, dst, over, head | lg, ns, R, kind
     uint4 h0{}, h1{};           // ClHead: nown, nwin, expect_all, fexp | fc0, fcn, fs0, fs1
     uint32_t lvb = cl_smem(lvs);  // its ClLev
     auto bind = [&](int l) {
@@ -463,6 +464,21 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
         dinv = cl_ld<T>(dyn + lt1.x + (int)sizeof(T) * m);
         load_dst(own, m, doff, kx);
     };
+    // Item `item` of [x0, x0 + cnt) of a sweep's colour: a row (times lanes), or on the finest level a
+    // block, whose rows are taken in ascending (backward: descending) order: the first row is
+    // read, `rest` more follow
+    int rest = 0;
+    auto load_item = [&](int x0, int item, int cnt, bool bwd, int blk, int zoff, unsigned kx) {
+        if (blk == 0) {
+            load_row(x0, item, cnt, zoff, zoff, kx);
+            return;
+        }
+        const bool on = item < cnt;
+        const uint32_t b = dyn + blk + 2 * (on ? x0 + item : 0);
+        const int s = cl_ld<unsigned short>(b), e = cl_ld<unsigned short>(b + 2);
+        rest = on ? e - s - 1 : 0;
+        load_row(bwd ? e - 1 : s, 0, on, zoff, zoff, kx);
+    };
     // off-diagonal part of the row's product with z, over its lanes
     auto gather = [&](int k) {
 #ifdef AMG_BOUNDS_CHECK
@@ -528,8 +544,9 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
     // Gauss-Seidel sweeps over n colours; the first one's rows are loaded already. The rows of
     // the step after the sweep (all own rows of the level; sent, if at all, to the vector at
     // next_off in the next exchange) are loaded before its last wait.
-    auto sweep = [&](int ops, int n, int foff, int zoff, int next_cnt, int next_off) {
+    auto sweep = [&](int ops, int n, bool bwd, int foff, int zoff, int next_cnt, int next_off) {
         const uint32_t z = dyn + zoff, f = dyn + foff;
+        const int blk = lt2.w == 2 ? CL_F(blk) : 0;
         uint4 op = cl_ld<uint4>(dyn + ops);  // a ClOp
 #pragma unroll 1
         for (int k = 0; k < n; k++) {
@@ -539,17 +556,26 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                 push(zoff, u);
                 cl_st_if(own, z + lb, u);
             };
+            auto rest_of_block = [&] {
+#pragma unroll 1
+                for (; rest > 0; rest--) {
+                    load_row(bwd ? mi - 1 : mi + 1, 0, 1, zoff, zoff, kn);
+                    relax();
+                }
+            };
             // (a warp without rows goes on at once)
             if (32 * warp < (int)op.y) relax();
+            if (blk) rest_of_block();
 #pragma unroll 1
             for (int c = kClThreads; c < (int)op.y; c += kClThreads) {  // strips of large levels
-                load_row(op.x, c + tid, op.y, zoff, zoff, kn);
+                load_item(op.x, c + tid, op.y, bwd, blk, zoff, kn);
                 if (c + 32 * warp < (int)op.y) relax();
+                if (blk) rest_of_block();
             }
             arrive_n(op.z);
             if (k + 1 < n) {
                 op = cl_ld<uint4>(dyn + ops + 16 * (k + 1));
-                load_row(op.x, tid, op.y, zoff, zoff, kn + 1);
+                load_item(op.x, tid, op.y, bwd, blk, zoff, kn + 1);
             } else {
                 load_row(0, tid, next_cnt, zoff, next_off, kn + 1);
             }
@@ -656,7 +682,8 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
         arrive_n((int)h0.w);
         const int npre = CL_F(npre);
         const uint4 op = cl_ld<uint4>(dyn + CL_F(pre));
-        load_row(npre ? op.x : 0, tid, npre ? op.y : h0.x << lt2.x, zoff, npre ? zoff : qoff, kn + 1);
+        if (lt2.w == 2) load_item(op.x, tid, op.y, false, CL_F(blk), zoff, kn + 1);
+        else load_row(npre ? op.x : 0, tid, npre ? op.y : h0.x << lt2.x, zoff, npre ? zoff : qoff, kn + 1);
         wait_n();
     };
     if (y.nsp > 0) {  // this strip's rows of the right-hand side, and their first colour
@@ -680,10 +707,11 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
             const int i = (int)(steps >> (4 * lv)) & 15;
             const int foff = i == 0 ? CL_F(rhs) : CL_F(r), zoff = p_off(i), toff = q_off(i);
             const int rows = (int)(h0.x << lt2.x), npre = CL_F(npre);
-            if (npre > 0) sweep(CL_F(pre), npre, foff, zoff, rows, toff);
+            if (npre > 0) sweep(CL_F(pre), npre, false, foff, zoff, rows, toff);
             const bool to_swept = lv + 1 < y.nsp;
             const int child = CL_F(child), nch = CL_F(nch), Rn = CL_F(Rn);
-            const bool xchild = lt2.w != 0;
+            const bool xchild = lt2.w == 1;
+            const uint32_t blk = lt2.w == 2 ? dyn + CL_F(blk) : 0, own0 = dyn + lt0.x;
             // t = f - A z into q_i (free until step i's product)
 #pragma unroll 1
             for (int c = 0;;) {
@@ -712,6 +740,13 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
             mark(lv, OP_RESID);
             const uint32_t t = dyn + toff;
             auto child_sum = [&](int m) {
+                if (blk) {  // the finest level: its block m's rows
+                    T acc = 0;
+                    const int e = cl_ld<unsigned short>(blk + 2 * m + 2);
+                    for (int k = cl_ld<unsigned short>(blk + 2 * m); k < e; k++)
+                        acc += cl_ld<T>(t + cl_ld<unsigned short>(own0 + 2 * k));
+                    return acc;
+                }
                 T w[2] = {T(0), T(0)};
 #pragma unroll
                 for (int h = 0; h < 2; h++) {
@@ -922,7 +957,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
             const uint32_t z = dyn + zoff;
             {  // z += P e on the window; the colour swept next is overwritten unread
                 const uint4 op = cl_ld<uint4>(dyn + post);
-                load_row(op.x, tid, op.y, zoff, zoff, kn);
+                load_item(op.x, tid, op.y, true, lt2.w == 2 ? CL_F(blk) : 0, zoff, kn + (lt2.w == 2));
                 const uint32_t en = dyn + (lv + 1 < y.nsp ? cl_ld<int>(lvb + (uint32_t)(sizeof(ClLev) + offsetof(ClLev, e)))
                                                           : y.E);
                 const uint32_t par = dyn + CL_F(parent);
@@ -933,10 +968,19 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                         const uint32_t zk = z + (uint32_t)sizeof(T) * k;
                         cl_st(zk, cl_ld<T>(zk) + cl_ld<T>(en + (uint32_t)sizeof(T) * cl_ld<unsigned short>(par + 2 * k)));
                     }
-                __syncthreads();
+                if (lt2.w == 2) {  // (blocks: the colour swept next is read too, so the neighbours
+                    arrive_n(0);   // must have added it everywhere before its rows come in)
+                    wait_n();
+                } else {
+                    __syncthreads();
+                }
                 mark(lv, OP_PROLONG);
             }
-            sweep(post, npost, foff, zoff, rows, zoff);
+            sweep(post, npost, true, foff, zoff, rows, zoff);
+            if (lt2.w == 2) {  // B^_0 is all: z is the result
+                done = true;
+                break;
+            }
 #pragma unroll 1
             for (int j = 0; j < i; j++) {  // p_i = z + sum_j beta_j p_j, on the window
                 T zq = 0;
@@ -1029,7 +1073,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
         if (y.nsp > 0) {
             const int nown = (int)h0.x;  // (level 0 is bound)
             const unsigned short *own = (const unsigned short *)at(lvs[0].own);
-            const T *e = vec(lvs[0].e);
+            const T *e = vec(lt2.w == 2 ? p_off(0) : CL_F(e));
 #pragma unroll 1
             for (int m = tid; m < nown; m += kClThreads) a.e[((const int *)at(y.top))[m]] = *(const T *)((const unsigned char *)e + own[m]);
         } else {
@@ -1059,6 +1103,7 @@ struct ClSrc {
     const int4 *ch, *ch2;        // children of the next level's rows
     const double *val64;
     const float *val32;
+    const int *bptr;             // finest level: row ranges of its blocks (the next level's rows)
     int cr[kClColors + 1];
 };
 struct ClSrcs {
@@ -1076,6 +1121,11 @@ __host__ __device__ inline int cl_part(int len, int r) { return (int)((long long
 __device__ __forceinline__ int cl_owner(const ClSrc &S, int c, int i) {
     const int len = S.cr[c + 1] - S.cr[c];
     return (kClRanks * (i - S.cr[c] + 1) - 1) / len;
+}
+// the CTA that owns row i (colour c) of level a: the finest level's rows go with their block
+__device__ __forceinline__ int cl_row_owner(const ClSrcs &G, int a, int c, int i) {
+    const ClSrc &S = G.lv[a];
+    return S.bptr ? cl_owner(G.lv[a + 1], c, S.parent[i]) : cl_owner(S, c, i);
 }
 // Window tables: [level][rank][colour] (first, last + 1). The children of the next level's rows
 // that lie in another strip than the row's owner have tables of their own: cwin[0] with the
@@ -1103,12 +1153,12 @@ __global__ void k_cl_windows(const __grid_constant__ ClSrcs G, int2 *win, int2 *
     const ClSrc &S = G.lv[a], &N = G.lv[a + 1];
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i < S.n) {
-        const int c = cl_colour(S, i), r = cl_owner(S, c, i);
+        const int c = cl_colour(S, i), r = cl_row_owner(G, a, c, i);
         const int s0 = S.sl[i >> 5], width = (S.sl[(i >> 5) + 1] - s0) >> 5;
         for (int k = 1; k < width; k++) {
             const int j = S.col[s0 + 32 * k + (i & 31)];
             if (j < 0) continue;
-            const int cj = cl_colour(S, j), rj = cl_owner(S, cj, j);
+            const int cj = cl_colour(S, j), rj = cl_row_owner(G, a, cj, j);
             if (rj == r) continue;
             cl_extend(win + cl_win(a, r, cj), j);
             cl_extend(win + cl_win(a, rj, c), i);
@@ -1116,8 +1166,8 @@ __global__ void k_cl_windows(const __grid_constant__ ClSrcs G, int2 *win, int2 *
     }
     if (i < N.n) {
         const int ra = cl_owner(N, cl_colour(N, i), i);
-        int rb = -1;
-        for (int q = 0; q < (S.ch2 ? 8 : 4); q++) {
+        int rb = S.bptr ? ra : -1;  // (a block's rows go with it)
+        for (int q = 0; q < (S.bptr ? 0 : S.ch2 ? 8 : 4); q++) {
             const int j = cl_child(S, i, q);
             if (j < 0) continue;
             const int cj = cl_colour(S, j), rj = cl_owner(S, cj, j);
@@ -1278,6 +1328,12 @@ __global__ void k_cl_image(const __grid_constant__ ClSrcs G, const __grid_consta
             R = ntab[c].g0 + m - ntab[c].m0;
         } else {
             R = ((const unsigned short *)(im + y.down))[m];
+        }
+        if (S.bptr) {
+            const int i = S.bptr[R], c = cl_colour(S, i);
+            ((unsigned short *)(im + L.blk))[m] = (unsigned short)(tab[c].m0 + i - tab[c].g0);
+            if (m == nn - 1) ((unsigned short *)(im + L.blk))[nn] = (unsigned short)H.nown;
+            continue;
         }
         for (int q = 0; q < L.nch; q++) {
             const int j = cl_child(S, R, q);

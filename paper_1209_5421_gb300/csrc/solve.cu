@@ -997,13 +997,21 @@ struct ClPlan {
     int table_bytes = 0;
 };
 
+// strip r's rows of colour c (the finest level: of its blocks, hb = their first rows)
+int2 cl_own_rows(const ClSrc &S, const std::vector<int> &hb, int r, int c) {
+    const ClSrc &B = S.bptr ? (&S)[1] : S;  // the next level: its rows are the blocks
+    const int len = B.cr[c + 1] - B.cr[c];
+    const int a = B.cr[c] + cl_part(len, r), b = B.cr[c] + cl_part(len, r + 1);
+    return S.bptr ? make_int2(hb[a], hb[b]) : make_int2(a, b);
+}
+
 // Layout and tables for the swept levels G.lv[s0 ..] (hierarchy levels level0 ..) and the dense
 // level after them, or false if they do not fit `budget` bytes of shared memory. win: their
 // windows; xchild: [2][nlv], by the next level's kind (swept, dense); fo: owner of each row of
 // the dense level.
 template <class T>
 bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vector<int> &xchild, int nlv,
-                  const int *fo, const std::vector<int> &widths, int s0, int level0, bool dense, int nch,
+                  const int *fo, const std::vector<int> &hb, const std::vector<int> &widths, int s0, int level0, bool dense, int nch,
                   const amg_options &opt, long budget, ClPlan &P) {
     constexpr int vb = (int)sizeof(T), NR = kClRanks;
     ClLayout &y = P.y;
@@ -1021,10 +1029,7 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
     auto win_of = [&](int a, int r, int c) {
         return win[cl_win(s0 + a, r, c)];
     };
-    auto own_of = [](const ClSrc &S, int r, int c) {
-        const int len = S.cr[c + 1] - S.cr[c];
-        return make_int2(S.cr[c] + cl_part(len, r), S.cr[c] + cl_part(len, r + 1));
-    };
+    auto own_of = [&](const ClSrc &S, int r, int c) { return cl_own_rows(S, hb, r, c); };
     // the strips: windows, bytes exchanged, neighbours
     P.geo.assign((size_t)std::max(1, y.nsp) * NR * kClColors, ClColor{});
     auto geo = [&](int a, int r, int c) -> ClColor & { return P.geo[cl_win(a, r, c)]; };
@@ -1061,6 +1066,7 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
                 const int t = r << lg, full = t / kClThreads, rest = (t % kClThreads + 31) / 32;
                 return (full * 19.0 * kClWarps + (rest ? std::max(64, 19 * rest) : 0)) * instr + 70.0 * lg;
             };
+            if (S.bptr && lg > 0) continue;  // a block is one lane's
             const double cost = vb == 8 ? colours * fp64(rows, ns + lg + 2) + 2 * fp64(all, ns + lg + 3) : lg;
             if (L.lg >= 0 && cost >= best) continue;
             L.lg = lg;
@@ -1093,12 +1099,12 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
             }
             if (h.nwin * vb > 65535) return false;  // 16-bit byte offsets
             h.fc0 = geo(a, r, cf).m0;
-            h.fcn = geo(a, r, cf).cnt;
+            h.fcn = S.bptr ? 0 : geo(a, r, cf).cnt;
             c_first[a] = cf;
             h.fs0 = geo(a, r, cf).seg0;
-            h.fs1 = h.fs0 + geo(a, r, cf).seglen;
+            h.fs1 = h.fs0 + (S.bptr ? 0 : geo(a, r, cf).seglen);
             h.ls0 = geo(a, r, cl).seg0;
-            h.ls1 = h.ls0 + geo(a, r, cl).seglen;
+            h.ls1 = h.ls0 + (S.bptr ? 0 : geo(a, r, cl).seglen);
             max_own[a] = std::max(max_own[a], (size_t)h.nown);
             max_win[a] = std::max(max_win[a], (size_t)h.nwin);
         }
@@ -1133,7 +1139,7 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
     for (int i = 0; i < D.n && y.nsp > 0; i++) down[fo[i]].push_back((unsigned short)i);
     for (int r = 0; r < NR; r++) max_own[y.nsp] = std::max(max_own[y.nsp], down[r].size());
     for (int a = 0; a < y.nsp; a++)
-        for (int r = 0; r < NR; r++) head[a][r].fexp = expect[a][r][c_first[a]];
+        for (int r = 0; r < NR; r++) head[a][r].fexp = G.lv[s0 + a].bptr ? 0 : expect[a][r][c_first[a]];
     // the sweeps of every strip: before the restriction (the first colour is done by the step
     // before) and after the correction
     auto lists = [&](int a, int r, std::vector<ClOp> &pre, std::vector<ClOp> &post) {
@@ -1142,12 +1148,22 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
         pre.clear();
         post.clear();
         auto colour = [&](int c) {
+            if (S.bptr) {  // own blocks, numbered colour by colour
+                int b0 = 0;
+                const ClSrc &B = G.lv[s0 + a + 1];
+                auto blocks = [&](int k) {
+                    const int len = B.cr[k + 1] - B.cr[k];
+                    return cl_part(len, r + 1) - cl_part(len, r);
+                };
+                for (int k = 0; k < c; k++) b0 += blocks(k);
+                return ClOp{b0, blocks(c), expect[a][r][c], 0};
+            }
             const ClColor &C = geo(a, r, c);
             return ClOp{C.m0 << L.lg, C.cnt << L.lg, expect[a][r][c], 0};
         };
         for (int sw = 0; sw < y.nu_pre; sw++)
             for (int c = 0; c < S.ncol; c++)
-                if (S.cr[c + 1] > S.cr[c] && (sw > 0 || c > c_first[a])) pre.push_back(colour(c));
+                if (S.cr[c + 1] > S.cr[c] && (sw > 0 || c > c_first[a] || S.bptr)) pre.push_back(colour(c));
         for (int sw = 0; sw < y.nu_post; sw++)
             for (int c = S.ncol - 1; c >= 0; c--)
                 if (S.cr[c + 1] > S.cr[c]) post.push_back(colour(c));
@@ -1178,7 +1194,8 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
         L.R = (int)max_own[a] << L.lg;
         L.nact = std::min(kClWarps, (L.R + 31) / 32);
         L.Rn = (int)max_own[a + 1];
-        L.xchild = xchild[(a + 1 < y.nsp ? 0 : 1) * nlv + s0 + a];
+        const bool fine = G.lv[s0 + a].bptr != nullptr;
+        L.kind = fine ? 2 : xchild[(a + 1 < y.nsp ? 0 : 1) * nlv + s0 + a];
         L.over = take(sizeof(unsigned) * over[a]);
         L.val = take((size_t)L.ns * L.R * vb);
         L.col = take((size_t)kClSlots * L.R * 2);
@@ -1187,7 +1204,8 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
         L.own = take(2 * max_own[a]);
         L.dst = take(sizeof(uint4) * max_own[a]);
         L.parent = take(2 * max_win[a]);
-        L.child = take(2 * (size_t)nch * L.Rn);
+        if (fine) L.blk = take(2 * ((size_t)L.Rn + 1));
+        else L.child = take(2 * (size_t)nch * L.Rn);
     }
     y.top = take(sizeof(int) * max_own[0]);
     y.mat = take((size_t)(dense && vb == 4 ? 2 : 1) * y.ch * y.stride * vb);
@@ -1201,10 +1219,13 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
     for (int a = 0; a < y.nsp; a++) {
         ClLev &L = y.lv[a];
         const size_t b = max_win[a] * vb;
+        const bool fine = G.lv[s0 + a].bptr != nullptr;  // B^_0 alone: no Alg. 1
         L.rhs = take(max_own[a] * vb);
-        L.r = take(max_own[a] * vb);
-        L.e = take(b);
-        for (int k = 0; k < y.kc; k++) {
+        if (!fine) {
+            L.r = take(max_own[a] * vb);
+            L.e = take(b);
+        }
+        for (int k = 0; k < (fine ? 1 : y.kc); k++) {
             L.p[k] = take(b);
             L.q[k] = take(b);
         }
@@ -1279,6 +1300,7 @@ void build_cluster(amg_hierarchy *h, EngineBase *E, int optin) {
         S.ch2 = l + 1 < nlev ? h->lev[l + 1].children2 : nullptr;
         S.val64 = lv.A.val;
         S.val32 = lv.A.val32;
+        S.bptr = l == 0 ? lv.bptr : nullptr;
         S.ncol = ranges ? (int)lv.color_rows.size() - 1 : 1;
         if (ranges)
             for (int c = 0; c <= S.ncol; c++) S.cr[c] = lv.color_rows[c];
@@ -1289,11 +1311,17 @@ void build_cluster(amg_hierarchy *h, EngineBase *E, int optin) {
     // the dense level is the one above the coarsest (M, A M) or the coarsest (its inverse);
     // windows are found for every level that may be swept
     const int last = nlev - 2;  // the coarsest level that is swept or dense
-    if (last < 1) return;
+    if (last < 0) return;
     int first = last + 1;
     while (first - 1 >= 1 && sweepable(first - 1) && last + 1 - (first - 1) <= kClLevels) first--;
+    // the finest level too, a small quadtree's: then an application is one launch (blocks of one
+    // lane: not the octree's of about eight rows, nor big ones). 65^2 nodes, FP64: 211 -> 153 us
+    // per application, 34^2 nodes: a solve 901 -> 667 us
+    if (first == 1 && sweepable(0) && last + 1 <= kClLevels && h->dim == 2 && h->lev[0].nbig == 0 &&
+        (int)h->lev[0].color_blocks.size() == (int)h->lev[0].color_rows.size())
+        first = 0;
     if (first > last) return;
-    const int nch = h->lev[nlev - 1].children2 ? 8 : 4;
+    const int nch = h->dim == 3 ? 8 : 4;
     ClSrcs G;
     std::memset(&G, 0, sizeof G);
     G.nsp = last + 1 - first;
@@ -1302,16 +1330,19 @@ void build_cluster(amg_hierarchy *h, EngineBase *E, int optin) {
     const bool crr = (int)h->lev[nlev - 1].color_rows.size() - 1 <= kClColors &&
                      h->lev[nlev - 1].color_rows.size() > 1;
     G.lv[G.nsp] = source(nlev - 1, crr);
+    std::vector<int> hb;  // the finest level's blocks
+    if (first == 0) {
+        hb.resize(h->lev[1].n + 1);
+        AMG_CUDA(cudaMemcpyAsync(hb.data(), h->lev[0].bptr, sizeof(int) * hb.size(), cudaMemcpyDeviceToHost, s));
+        AMG_CUDA(cudaStreamSynchronize(s));
+    }
     const size_t words = (size_t)G.nsp * kClRanks * kClColors;
     std::vector<int2> win(3 * words);
     for (int a = 0; a < G.nsp; a++)
         for (int r = 0; r < kClRanks; r++)
             for (int c = 0; c < kClColors; c++) {
                 const size_t o = cl_win(a, r, c);
-                const ClSrc &S = G.lv[a];
-                const int len = c < S.ncol ? S.cr[c + 1] - S.cr[c] : 0;
-                win[o] = c < S.ncol ? make_int2(S.cr[c] + cl_part(len, r), S.cr[c] + cl_part(len, r + 1))
-                                    : make_int2(0, 0);
+                win[o] = c < G.lv[a].ncol ? cl_own_rows(G.lv[a], hb, r, c) : make_int2(0, 0);
                 win[words + o] = win[2 * words + o] = make_int2(INT32_MAX, 0);
             }
     const int nc = h->lev[nlev - 1].n, nfo = nc + (G.nsp > 1 ? h->lev[last].n : 0);
@@ -1337,15 +1368,15 @@ void build_cluster(amg_hierarchy *h, EngineBase *E, int optin) {
     // the finest start that fits; with the dense matrices if that start allows them
     ClSrcs GD = G;  // dense level = the last swept one
     GD.nsp = G.nsp - 1;
-    const bool can_dense = h->lev[last].n <= kClDenseMax;
+    const bool can_dense = last >= 1 && h->lev[last].n <= kClDenseMax;
     ClPlan P;
     bool ok = false;
     int s0 = 0;
     for (; s0 < G.nsp; s0++) {
-        ok = can_dense && cluster_plan<T>(GD, win, xchild, G.nsp, fo.data() + nc, widths, s0, first + s0, true,
+        ok = can_dense && cluster_plan<T>(GD, win, xchild, G.nsp, fo.data() + nc, hb, widths, s0, first + s0, true,
                                           nch, h->opt, budget, P);
         if (!ok)
-            ok = cluster_plan<T>(G, win, xchild, G.nsp, fo.data(), widths, s0, first + s0, false, nch, h->opt,
+            ok = cluster_plan<T>(G, win, xchild, G.nsp, fo.data(), hb, widths, s0, first + s0, false, nch, h->opt,
                                  budget, P);
         if (ok) break;
     }
@@ -1395,11 +1426,13 @@ void build_engine(amg_hierarchy *h) {
     const int tl = E->cl.tl;
     h->tail_level = tl;
     Builder b{h, &E->hprog, tl};
-    b.bhat(0, V_RHS, V_E);
+    if (tl == 0) b.emit(Builder::mk(OP_TAIL, 0));  // the whole application
+    else b.bhat(0, V_RHS, V_E);
     annotate_reductions(E->hprog);
     if (tl < h->nlev) {
         Builder bt{h, &E->htail, h->nlev + 1};  // the cluster's ops (traffic accounting only)
-        bt.btilde(tl);
+        if (tl == 0) bt.bhat(0, V_RHS, V_E);
+        else bt.btilde(tl);
     }
     for (const Op &op : E->htail) E->tail_bytes += op_bytes(h, op, sizeof(T));
     for (const Op &op : E->hprog)
@@ -1534,7 +1567,7 @@ void launch_cycle(amg_hierarchy *h, T *rhs0 = nullptr, T *e0 = nullptr) {
     a.big_smem = E->big_smem;
     a.big_wwarps = E->big_wwarps;
     a.big_wslice = E->big_wslice;
-    AMG_CUDA(cudaMemsetAsync(h->bar, 0, sizeof(unsigned long long), s));
+    if (E->cl.tl > 0) AMG_CUDA(cudaMemsetAsync(h->bar, 0, sizeof(unsigned long long), s));
     a.ts = prof ? E->ts + 1 : nullptr;
     Profiler::Rec rec{};
     if (prof) {
@@ -1549,8 +1582,8 @@ void launch_cycle(amg_hierarchy *h, T *rhs0 = nullptr, T *e0 = nullptr) {
         const Vecs<T> &v = vecs<T>(h->lev[E->cl.tl]);
         ca.y = E->cl;
         ca.image = E->cl_image;
-        ca.rhs = v.rhs;
-        ca.e = v.e;
+        ca.rhs = E->cl.tl == 0 && rhs0 ? rhs0 : v.rhs;
+        ca.e = E->cl.tl == 0 && e0 ? e0 : v.e;
         ca.err = h->err_flag;
         ca.limit_ns = a.bar_limit_ns;
         ca.extra = h->dbg_bar_extra;
