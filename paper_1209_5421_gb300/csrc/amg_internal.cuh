@@ -73,7 +73,7 @@ __host__ __device__ inline size_t big_smem_align(size_t b) { return (b + 15) & ~
 __host__ __device__ inline size_t big_smem_bytes(int m, int nl, int ns, int vb) {
     if (m > 65535 || ns > 65535) return 0;
     return big_smem_align((size_t)3 * m * vb) + big_smem_align((size_t)6 * m) +
-           big_smem_align((size_t)2 * (nl + 1)) + big_smem_align((size_t)2 * ns * vb) +
+           big_smem_align((size_t)2 * (nl + 1)) + big_smem_align((size_t)ns * vb) +
            big_smem_align((size_t)2 * ns);
 }
 

@@ -710,15 +710,16 @@ struct LaneGroup {
     __device__ __forceinline__ void sync() const { __syncwarp(); }
 };
 
-// Big block k swept in shared memory (buf, bytes) by group g. Its rows' couplings are staged
-// first, in one pass over the block with no dependence between rows: each off-diagonal
-// slot's coefficient, and either the current value of a coupled unknown outside the block
-// (this colour does not change it) or the index of one inside; with each row's f and
-// 1/a_ii. The block's unknowns then live in shared memory and the level-ordered sweep reads
-// nothing else: a group barrier between levels, no memory round trip. Every row's sum takes
-// its slots in row_dot's order, with row_dot's zero terms up to the end of its last batch:
-// the same operations, the same bits. Returns false (nothing done) when the block does not
-// fit.
+// Big block k swept in shared memory (buf, bytes) by group g. What a colour's time hangs on is the
+// chain of the block's levels (89 of them in the largest on a 1449 x 1449 graded mesh), so a
+// row's chain is kept to what it must wait for. Staging, one pass over the block with no
+// dependence between rows, sums f_i minus every term whose value is final (unknowns outside
+// the block, which this colour does not change, and those inside that the sweep reaches
+// later), and keeps the couplings to rows reached earlier: about half of a row's. The
+// level-ordered sweep then subtracts these from shared memory, a group barrier between
+// levels. The update is the sequential sweep's with the sum in another order. Mean finest colour of
+// a 513 x 513 graded mesh, FP64: 59 -> 44 us (with every coupling in the chain, summed in
+// row_dot's order, before). Returns false (nothing done) when the block does not fit.
 template <class LV, class G>
 __device__ bool big_block_smem(const LV &L, const int *lofs, const int *lp, const int4 *ent,
                                int k, const typename LV::val_t *f, typename LV::val_t *u,
@@ -735,57 +736,69 @@ __device__ bool big_block_smem(const LV &L, const int *lofs, const int *lp, cons
     if (need == 0 || need > bytes) return false;
     unsigned char *q = buf;
     T *su = (T *)q;  // the block's unknowns (local index = row - r0)
-    T *ef = su + m, *ed = ef + m;  // per entry: f, 1/a_ii
+    T *es = su + m, *ed = es + m;  // per entry: f minus the final terms, 1/a_ii
     q += big_smem_align((size_t)3 * m * sizeof(T));
-    // per entry: local row, first slot, slot count
+    // per entry: local row, first early coupling, their number
     unsigned short *erow = (unsigned short *)q, *eo = erow + m, *ew = eo + m;
     q += big_smem_align((size_t)6 * m);
     unsigned short *slp = (unsigned short *)q;  // level boundaries, relative to e0
     q += big_smem_align((size_t)2 * (nl + 1));
-    T *sa = (T *)q, *sx = sa + ns;  // per slot: coefficient, outside value
-    q += big_smem_align((size_t)2 * ns * sizeof(T));
-    unsigned short *si = (unsigned short *)q;  // per slot: inside index, 0xFFFF outside
+    T *sa = (T *)q;  // per early coupling: coefficient, local row
+    q += big_smem_align((size_t)ns * sizeof(T));
+    unsigned short *si = (unsigned short *)q;
     const int t = g.rank(), nt = g.size();
+    const bool bwd = lofs == S->lofs_b;
     for (int j = t; j <= nl; j += nt) slp[j] = (unsigned short)(lp[l0 + j] - e0);
     for (int i = t; i < m; i += nt) {
         const int4 e = ent[e0 + i];
         const int row = e.x;
+        T s = f[row];
+        int early = 0;
+        for (int kb = 1; kb < e.z; kb += kRowBatch) {
+            typename LV::idx_t c[kRowBatch];
+            T a[kRowBatch], x[kRowBatch];
+#pragma unroll
+            for (int j = 0; j < kRowBatch; j++) {
+                const int kk = kb + j;
+                c[j] = kk < e.z ? L.col[e.y + 32 * kk] : (typename LV::idx_t)-1;
+                a[j] = kk < e.z ? L.val[e.y + 32 * kk] : T(0);
+            }
+#pragma unroll
+            for (int j = 0; j < kRowBatch; j++)
+                x[j] = (col_ok(c[j]) && idx_ok((int)c[j], L.n)) ? u[c[j]] : T(0);
+#pragma unroll
+            for (int j = 0; j < kRowBatch; j++) {
+                const int ci = (int)c[j];
+                if (col_ok(c[j]) && ci >= r0 && ci < r0 + m && (bwd ? ci > row : ci < row)) {
+                    sa[e.w + early] = a[j];
+                    si[e.w + early] = (unsigned short)(ci - r0);
+                    early++;
+                } else if (col_ok(c[j])) {
+                    s -= a[j] * x[j];
+                }
+            }
+        }
         erow[i] = (unsigned short)(row - r0);
         eo[i] = (unsigned short)e.w;
-        ew[i] = (unsigned short)e.z;
-        ef[i] = f[row];
+        ew[i] = (unsigned short)early;
+        es[i] = s;
         ed[i] = L.dinv[row];
-        su[row - r0] = u[row];
-        for (int kk = 1; kk < e.z; kk++) {
-            const auto c = L.col[e.y + 32 * kk];
-            const int s = e.w + kk - 1;
-            sa[s] = L.val[e.y + 32 * kk];
-            unsigned short ix = 0xFFFF;
-            T xv = T(0);
-            if (col_ok(c) && idx_ok((int)c, L.n)) {
-                const int ci = (int)c;
-                if (ci >= r0 && ci < r0 + m) ix = (unsigned short)(ci - r0);
-                else xv = u[ci];
-            }
-            si[s] = ix;
-            sx[s] = xv;
-        }
     }
     g.sync();
     for (int j = 0; j < nl; j++) {
         const int p1 = slp[j + 1];
         for (int i = slp[j] + t; i < p1; i += nt) {
-            const int o = (int)eo[i] - 1, w = ew[i];
-            T acc = 0;
-            int kk = 1;
-            for (; kk < w; kk++) {
-                const unsigned short ix = si[o + kk];
-                const T xv = ix != 0xFFFF ? su[ix] : sx[o + kk];
-                acc += sa[o + kk] * xv;
+            const int o = eo[i], w = ew[i];
+            T acc = es[i];
+            const T d = ed[i];
+            int kk = 0;
+            for (; kk + 2 <= w; kk += 2) {
+                const T x0 = su[si[o + kk]], x1 = su[si[o + kk + 1]], a0 = sa[o + kk], a1 = sa[o + kk + 1];
+                acc -= a0 * x0;
+                acc -= a1 * x1;
             }
-            for (const int kend = 1 + (w + kRowBatch - 2) / kRowBatch * kRowBatch; kk < kend; kk++)
-                acc += T(0) * T(0);  // row_dot's zero terms to the end of its batch
-            su[erow[i]] = (ef[i] - acc) * ed[i];
+            if (kk < w) acc -= sa[o + kk] * su[si[o + kk]];
+            su[erow[i]] = acc * d;
         }
         g.sync();
     }
@@ -818,12 +831,23 @@ __device__ void big_block_global(const LV &L, const int *lofs, const int *lp, co
 template <class LV>
 __device__ void op_gs_big_blocks(const LV &L, const Op &op, const typename LV::val_t *f,
                                  typename LV::val_t *u, int tid, int nth, int crank,
-                                 int ccount, const BigScratch &sc) {
+                                 int ccount, const BigScratch &sc, bool apart = false) {
     const BigSched *S = L.big;
     const bool bwd = op.backward != 0;
     const int *lofs = bwd ? S->lofs_b : S->lofs_f;
     const int *lp = bwd ? S->lp_b : S->lp_f;
     const int4 *ent = bwd ? S->ent_b : S->ent_f;
+    const int nbigc = op.bb1 - op.bbc;
+    if (apart) {  // CTAs [0, nbigc) sweep one CTA-sized block each, the others the warp-sized ones
+        if (crank < nbigc) {
+            const int k = op.bbc + crank;
+            if (!big_block_smem(L, lofs, lp, ent, k, f, u, sc.p, sc.bytes, CtaGroup{}))
+                big_block_global(L, lofs, lp, ent, k, f, u, CtaGroup{});
+            return;
+        }
+        crank -= nbigc;
+        ccount -= nbigc;
+    }
     if (sc.p) {
         const int w = (int)threadIdx.x >> 5;
         if (sc.wwarps > 0 && w < sc.wwarps) {  // warps with a slice: warp-sized blocks
@@ -836,6 +860,7 @@ __device__ void op_gs_big_blocks(const LV &L, const Op &op, const typename LV::v
             for (int k = op.bb0 + w * ccount + crank; k < op.bbc; k += nw)
                 big_block_global(L, lofs, lp, ent, k, f, u, LaneGroup{});
         }
+        if (apart) return;
         __syncthreads();  // the slices are the CTA-sized blocks' buffer next
     } else {
         for (int k = op.bb0 + (tid >> 5); k < op.bbc; k += nth >> 5)  // warp-sized blocks
@@ -1264,6 +1289,21 @@ __device__ void op_update(const LV &L, const Op &op, const RedCtx &rc, int tid, 
 
 // run one op (everything except OP_TAIL / OP_NOP) on level view L by threads tid < nth of
 // group g; next() gives the view of the next coarser level (only its rhs and e are used)
+// A finest colour with big blocks has three kinds of work, each a chain of its own length: the
+// CTA-sized blocks, the warp-sized ones and the small ones (a thread each). Where there is room
+// they run side by side: CTAs [0, nbigc) take a CTA-sized block each and nothing else, in the
+// others warps [0, wwarps) take the warp-sized blocks and the rest the small ones. One after
+// another in every CTA they took 44 us per colour (513 x 513 graded mesh, FP64), side by side
+// 24 us. Returns whether the small blocks go by (tid, nth) as set here.
+__device__ __forceinline__ bool gs_apart(const Op &op, const BigScratch &sc, int &tid, int &nth) {
+    const int nbigc = op.bb1 - op.bbc, cta = (int)blockIdx.x - nbigc, ctas = (int)gridDim.x - nbigc;
+    const int w = ((int)threadIdx.x >> 5) - sc.wwarps, nw = ((int)blockDim.x >> 5) - sc.wwarps;
+    if (op.bb1 <= op.bb0 || !sc.p || sc.wwarps == 0 || 2 * nbigc > (int)gridDim.x) return false;
+    if (nw <= 0 || op.i1 - op.i0 > ctas * nw * 32) return false;
+    nth = ctas * nw * 32;
+    tid = cta < 0 || w < 0 ? nth : (w * ctas + cta) * 32 + ((int)threadIdx.x & 31);
+    return true;
+}
 // Does op_ahead read the op's rows? At most one per thread (more rows are better left to loads
 // that overlap each other: a loop reading one row ahead took 36 us instead of 17 for the
 // residual of 965k rows), on a quadtree's levels (an octree's rows are wider than the batch
@@ -1280,11 +1320,12 @@ __device__ __forceinline__ bool op_has_ahead(const LV &L, const Op &op, int nth)
 // this thread's row of the op, read before the barrier in front of it (the matrix and the
 // block bounds only, which no op changes)
 template <class LV>
-__device__ __forceinline__ void op_ahead(const LV &L, const Op &op, int tid, int nth,
+__device__ __forceinline__ void op_ahead(const LV &L, const Op &op, int tid, int nth, const BigScratch &sc,
                                          RowAhead<LV> &held) {
     held.row = -1;
     if (!op_has_ahead(L, op, nth)) return;
     if (op.kind == OP_GS) {
+        if (L.fine) gs_apart(op, sc, tid, nth);
         const int b = op.i0 + tid;
         if (b < op.i1) row_load(L, !L.fine ? b : op.backward ? L.bptr[b + 1] - 1 : L.bptr[b], 1, held);
     } else if (tid < L.n) {
@@ -1302,9 +1343,11 @@ __device__ __forceinline__ void run_op_held(const LV &L, const Op &op, const Red
         const T *f = vec_of(L, op.fsel);
         T *u = vec_of(L, op.usel);
         const bool big = L.fine && op.bb1 > op.bb0;
-        if (big) prefetch_big_tasks(L, op, f, u, tid, nth, (int)blockIdx.x, (int)gridDim.x);
+        int stid = tid, snth = nth;
+        const bool apart = big && gs_apart(op, sc, stid, snth);
+        if (big && !apart) prefetch_big_tasks(L, op, f, u, tid, nth, (int)blockIdx.x, (int)gridDim.x);
         if (i >= 0) {
-            const int b = op.i0 + tid;
+            const int b = op.i0 + stid;
             const int r0 = L.fine ? L.bptr[b] : i, r1 = L.fine ? L.bptr[b + 1] : i + 1;
             const T fi = f[i], di = L.dinv[i], acc = row_dot_held(L, held, 1, u);
             if (!(big && r1 - r0 > kBigBlockRows)) {  // (those: in level order, below)
@@ -1315,7 +1358,7 @@ __device__ __forceinline__ void run_op_held(const LV &L, const Op &op, const Red
                     for (int k = r1 - 2; k >= r0; k--) gs_row(L, k, f, u);
             }
         }
-        if (big) op_gs_big_blocks(L, op, f, u, tid, nth, (int)blockIdx.x, (int)gridDim.x, sc);
+        if (big) op_gs_big_blocks(L, op, f, u, tid, nth, (int)blockIdx.x, (int)gridDim.x, sc, apart);
     } else if (op.kind == OP_RESID) {
         const T *f = vec_of(L, op.fsel), *u = vec_of(L, op.usel);
         if (i >= 0) pick(L.q, op.step)[i] = f[i] - row_dot_held(L, held, 0, u);

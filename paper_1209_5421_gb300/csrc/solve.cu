@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(cycle_threads<T>(), 1) k_cycle(CycleArgs<T> a)
         sc.wslice = a.big_wslice;
     }
     RowAhead<GL> held;
-    op_ahead(gtab[sop[a.k0 & 1].level], sop[a.k0 & 1], gtid, gnth, held);
+    op_ahead(gtab[sop[a.k0 & 1].level], sop[a.k0 & 1], gtid, gnth, sc, held);
     for (int k = a.k0; k < a.k1; k++) {
         const Op &op = sop[k & 1];
         // the next descriptor into the other buffer (last read by op k-1), issued before op k
@@ -167,7 +167,7 @@ __global__ void __launch_bounds__(cycle_threads<T>(), 1) k_cycle(CycleArgs<T> a)
         const bool last = k + 1 == a.k1;
         const Op &nx = sop[(k + 1) & 1];
         if (!last && !grid_barrier(a.bar, a.err, target, abort_flag, a.bar_limit_ns,
-                                   [&] { op_ahead(gtab[nx.level], nx, gtid, gnth, held); }))
+                                   [&] { op_ahead(gtab[nx.level], nx, gtid, gnth, sc, held); }))
             break;
         if (a.ts && blockIdx.x == 0 && threadIdx.x == 0) a.ts[k] = global_ns();
     }
