@@ -188,7 +188,6 @@ struct amg_hierarchy {
     std::vector<double *> P, Q;        // directions p_j, A p_j
     double **dP = nullptr, **dQ = nullptr;
     double *osc = nullptr;             // outer scalars
-    int *oit = nullptr;                // device iteration counter
     double *h_pinned = nullptr;        // pinned host scalars (allocated on first use)
     // FGMRES state (FP64 basis)
     double *gm_V = nullptr, *gm_Z = nullptr, *gm_H = nullptr;

@@ -271,8 +271,8 @@ __device__ __forceinline__ void bc_post(const BatchCycle<T, BIG> &c, int l, int 
     team_sync();
 }
 
-// B^_0 over the whole hierarchy: the recursion of Alg. 2 / Alg. 1 as a state machine (the
-// same walk as the shared-memory tail of the single-system kernel, from level 0)
+// B^_0 over the whole hierarchy: the recursion of Alg. 2 / Alg. 1 as a state machine
+// (the host-built program of the single-system kernel in another form, from level 0)
 template <class T, bool BIG>
 __device__ void batch_cycle(const BatchCycle<T, BIG> &c) {
     if (c.nlev == 1) {  // the only level is the coarsest: exact solve

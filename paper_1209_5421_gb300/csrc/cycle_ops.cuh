@@ -51,7 +51,7 @@ struct Op {
     // finest level, grid-wide executors: big blocks (aggregates of more than kBigBlockRows
     // unknowns) [bb0, bb1) of L.big->ids, swept by warps ([bb0, bbc)) and whole CTAs ([bbc,
     // bb1)) for GS (this colour's), summed by CTAs for RESTRICT (all); 0, 0, 0 = none (every
-    // block is one thread's, as in the batch and tail executors)
+    // block is one thread's)
     int bb0, bbc, bb1;
 };
 

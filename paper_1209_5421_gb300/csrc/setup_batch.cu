@@ -1242,7 +1242,7 @@ void build_batch(const std::vector<amg_hierarchy *> &hs, const amg_csr &A, const
         galerkin_multi(st, tmp, ps, l, reads);
     }
 
-    // ---- coarsest levels: dense Cholesky and explicit inverse, one CTA per system
+    // ---- coarsest levels: dense L D L^t and explicit inverse, one CTA per system
     {
         Multi<DDense> mz, md;
         std::vector<DChol> ch(P);
@@ -1333,7 +1333,6 @@ void build_batch(const std::vector<amg_hierarchy *> &hs, const amg_csr &A, const
         h->to = aget<double>(h, n);
         h->bo = aget<double>(h, n);
         h->osc = aget<double>(h, outer_scalar_count(maxit));
-        h->oit = aget<int>(h, 1);
         h->dP = aget<double *>(h, maxit);
         h->dQ = aget<double *>(h, maxit);
         for (int l = 0; l < h->nlev; l++) {

@@ -189,12 +189,6 @@ __global__ void k_scatter(int n, const int *__restrict__ idx, const double *__re
     if (p < n) dst[idx[p]] = src[p];
 }
 
-// 16-bit copy of column indices (padding -1 -> 0xFFFF)
-__global__ void k_col16(int n, const int *__restrict__ col, unsigned short *__restrict__ c16) {
-    int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) c16[i] = col[i] >= 0 ? (unsigned short)col[i] : (unsigned short)0xFFFF;
-}
-
 // 1 / a_ii of every row (slot 0 of the sliced ELL holds the diagonal)
 template <class T>
 __global__ void k_inv_diag(int n, const int *__restrict__ sl, const double *__restrict__ val,
@@ -506,7 +500,7 @@ thread_local int64_t g_launches = 0;
 enum : int { K_CYCLE = OP_NKINDS, K_OUTER_MULTIDOT, K_OUTER_ORTH, K_OUTER_SPMV_DOT, K_OUTER_UPDATE,
              K_TRUE_RESIDUAL, K_FGMRES_SPMV, K_FGMRES_MDOT, K_FGMRES_ORTH, K_NUM };
 constexpr int K_IN_CYCLE = 100;  // + op kind: an op timed inside the persistent kernel
-constexpr int K_IN_TAIL = 200;   // + op kind: an op timed inside the shared-memory tail
+constexpr int K_IN_TAIL = 200;   // + op kind: an op timed inside the cluster (CTA 0's clock)
 
 const char *kernel_name(int kind) {
     static const char *names[K_NUM] = {"zero", "gs_colour", "resid_restrict", "prolong_correct",
@@ -1717,7 +1711,6 @@ void allocate_solve_workspace(amg_hierarchy *h) {
     h->lev[0].v64.rhs = h->ro;
     h->lev[0].v64.e = h->zo;
     h->osc = halloc<double>(h, outer_scalar_count(h->opt.max_iters));
-    h->oit = halloc<int>(h, 1);
     h->dP = halloc<double *>(h, h->opt.max_iters);
     h->dQ = halloc<double *>(h, h->opt.max_iters);
     ensure_pinned(h);
