@@ -59,13 +59,19 @@ struct Op {
 enum : int { V_RHS = 0, V_E, V_R, V_P0 };  // V_P0 + i = p_i
 
 // view of one level; I = column index type;
-// B = 1 compiles the lane-parallel block smoother of finest levels with multi-row blocks
-// (a separate kernel instance, so that the code of the others stays as it is)
+// B: what the kernel instance compiles besides the plain rows, each in instances of its own, so
+// that the registers of the others stay free: kCoop the lane-parallel block smoother of finest
+// levels with multi-row blocks, kBig the sweeps of a graded finest level's big blocks
+// (compiled into every FP32 cycle these made 416 bytes of spill loads a thread instead of 124: a
+// solve of 1,046,529 unknowns 22.7 ms instead of 21.4, the octree of 129^3 nodes 27.7 instead
+// of 25.9)
+constexpr int kCoop = 1, kBig = 2;
 template <class T, class I, int B = 0>
 struct LevelDev {
     using val_t = T;
     using idx_t = I;
-    static constexpr int coop = B;
+    static constexpr int coop = B & kCoop;
+    static constexpr bool bigs = (B & kBig) != 0;
     int n;
     int fine;                       // 1 on the finest level (block smoother, bptr)
     int bg;                         // finest level: lanes that share a block (kBlockLanes), or
@@ -1325,7 +1331,7 @@ __device__ __forceinline__ void op_ahead(const LV &L, const Op &op, int tid, int
     held.row = -1;
     if (!op_has_ahead(L, op, nth)) return;
     if (op.kind == OP_GS) {
-        if (L.fine) gs_apart(op, sc, tid, nth);
+        if (LV::bigs && L.fine) gs_apart(op, sc, tid, nth);
         const int b = op.i0 + tid;
         if (b < op.i1) row_load(L, !L.fine ? b : op.backward ? L.bptr[b + 1] - 1 : L.bptr[b], 1, held);
     } else if (tid < L.n) {
@@ -1342,7 +1348,7 @@ __device__ __forceinline__ void run_op_held(const LV &L, const Op &op, const Red
     if (op.kind == OP_GS) {
         const T *f = vec_of(L, op.fsel);
         T *u = vec_of(L, op.usel);
-        const bool big = L.fine && op.bb1 > op.bb0;
+        const bool big = LV::bigs && L.fine && op.bb1 > op.bb0;
         int stid = tid, snth = nth;
         const bool apart = big && gs_apart(op, sc, stid, snth);
         if (big && !apart) prefetch_big_tasks(L, op, f, u, tid, nth, (int)blockIdx.x, (int)gridDim.x);
@@ -1383,13 +1389,13 @@ __device__ __forceinline__ void run_op_on(const LV &L, const Next &next, const O
     switch (op.kind) {
         case OP_ZERO: op_zero(L, vec_of(L, op.usel), tid, nth); break;
         case OP_GS:
-            op_gs<LV, true>(L, op, vec_of(L, op.fsel), vec_of(L, op.usel), tid, nth, -1, -1, sc);
+            op_gs<LV, LV::bigs>(L, op, vec_of(L, op.fsel), vec_of(L, op.usel), tid, nth, -1, -1, sc);
             break;
         case OP_GS_FIRST: op_gs_first(L, op, vec_of(L, op.fsel), vec_of(L, op.usel), tid, nth); break;
         case OP_RESTRICT: {
             const auto &N = next();
             op_restrict(L, vec_of(L, op.fsel), vec_of(L, op.usel), N.rhs, tid, nth,
-                        op.fuse ? N.p[0] : nullptr, N.dinv, op.f0, op.f1, op.bb1 > op.bb0);
+                        op.fuse ? N.p[0] : nullptr, N.dinv, op.f0, op.f1, LV::bigs && op.bb1 > op.bb0);
             break;
         }
         case OP_RESID:

@@ -22,7 +22,7 @@
 namespace amg {
 
 template <class T>
-using GLev = LevelDev<T, int>;                 // level in HBM
+using GLev = LevelDev<T, int, kBig>;           // level in HBM
 
 // persistent kernel CTA size (one CTA per SM): the FP64 cycle runs with fewer threads and
 // twice the registers each, as its ops at the 64-register cap of 1024 threads spill
@@ -100,8 +100,7 @@ __device__ __forceinline__ void finalize(const CycleArgs<T> &a, const TAB *tab, 
     __syncthreads();
 }
 
-// ops [k0, k1) of an application's program. B = 1: finest-level blocks of several rows take
-// the lane-parallel block smoother
+// ops [k0, k1) of an application's program. B: kCoop, kBig (LevelDev)
 extern __shared__ __align__(16) unsigned char amg_smem[];
 
 template <class T, int B>
@@ -142,7 +141,7 @@ __global__ void __launch_bounds__(cycle_threads<T>(), 1) k_cycle(CycleArgs<T> a)
     const int gnth = gridDim.x * blockDim.x;
     const RedCtx rc{a.partials, nullptr};
     BigScratch sc;
-    if (a.big_smem) {
+    if ((B & kBig) && a.big_smem) {
         unsigned dyn;
         asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
         sc.p = amg_smem;
@@ -656,7 +655,7 @@ struct EngineBase {
     int nops = 0;
     int grid = 0;
     size_t smem = 0;   // of the cycle kernel (big blocks)
-    int coop = 0;  // the cycle kernel instance with the lane-parallel block smoother
+    int form = 0;  // the cycle kernel's instance (kCoop, kBig)
     int big_smem = 0;  // the CTAs sweep the big blocks in their shared memory
     int big_wwarps = 0;  // warps of a CTA with a slice for the warp-sized blocks
     unsigned big_wslice = 0;
@@ -977,7 +976,12 @@ EngineBase *&engine_slot(amg_hierarchy *h) {
 
 template <class T>
 void *cycle_kernel(int B) {
-    return B ? (void *)k_cycle<T, 1> : (void *)k_cycle<T, 0>;
+    switch (B) {
+        case 0: return (void *)k_cycle<T, 0>;
+        case kCoop: return (void *)k_cycle<T, kCoop>;
+        case kBig: return (void *)k_cycle<T, kBig>;
+        default: return (void *)k_cycle<T, kCoop | kBig>;
+    }
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1415,7 +1419,7 @@ void build_engine(amg_hierarchy *h) {
     int dev = h->device, optin = 0, nsm = 0;
     AMG_CUDA(cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
     AMG_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
-    E->coop = coop_blocks(h->lev[0]) ? 1 : 0;
+    E->form = (coop_blocks(h->lev[0]) ? kCoop : 0) | (h->lev[0].nbig > 0 ? kBig : 0);
     build_cluster<T>(h, E, optin);
     const int tl = E->cl.tl;
     h->tail_level = tl;
@@ -1440,7 +1444,7 @@ void build_engine(amg_hierarchy *h) {
     // largest one that fits on the device; the warp-sized ones get a slice each on as many
     // warps per CTA as the most of them in one colour need (a block that does not fit takes
     // the global-memory sweep; the forward and backward schedules each count).
-    void *kern = cycle_kernel<T>(E->coop);
+    void *kern = cycle_kernel<T>(E->form);
     cudaFuncAttributes fa;
     AMG_CUDA(cudaFuncGetAttributes(&fa, kern));
     const size_t static_smem = fa.sharedSizeBytes;
@@ -1610,7 +1614,7 @@ void launch_cycle(amg_hierarchy *h, T *rhs0 = nullptr, T *e0 = nullptr) {
         a.bar_base = bars * (unsigned long long)E->grid;
         bars += (unsigned long long)(a.k1 - a.k0 - 1);
         void *args[] = {&a};
-        AMG_CUDA(cudaLaunchCooperativeKernel(cycle_kernel<T>(E->coop), dim3(E->grid),
+        AMG_CUDA(cudaLaunchCooperativeKernel(cycle_kernel<T>(E->form), dim3(E->grid),
                                              dim3(cycle_threads<T>()), args, E->smem, s));
         AMG_LAUNCH_CHECK();
     }
