@@ -306,6 +306,10 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
     }
     cl_sync_all();  // every CTA's mbarriers are ready
     bool alive = cl_mb_try(mb0 + 32, 0) || cl_wait_slow(mb0 + 32, 0, gave_up, a.err, kBarrierLimitNs);
+    // launched before the end of the kernel before it (its writes can be seen from here on);
+    // nothing above depends on that one, and the one after this waits in the same way
+    asm volatile("griddepcontrol.launch_dependents;");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!__syncthreads_and(alive)) {  // no image: the others give up at their first exchange
         cl_sync_all();
         return;
