@@ -29,6 +29,12 @@
 // colour are not coupled, and the steps that fill a whole window (from zero, prolongation)
 // leave out the colour that is exchanged next. One that still computes step k-1 can only be
 // at rows it does not send here, which read nothing of this CTA's (symmetric windows).
+// A token comes from the CTA's last warp and vouches for that warp alone; rows vouch for the warps
+// that sent them. So a step that writes window entries which other CTAs own, and which a
+// neighbour may send in the exchange after this one, has a CTA barrier before its arrival: the
+// zeroed windows at the entry and before a level's first colour, the correction added on the
+// finest level. (The checking build, -DAMG_BOUNDS_CHECK, keeps some warps of every step waiting
+// for a few microseconds, another set each step, so that a missing one shows in the results.)
 // Sums over the cluster and gathers to all CTAs count on two mbarriers of their own.
 //
 // The level above the coarsest: B^ there is linear (the coarsest solve is exact), so setup
@@ -539,8 +545,15 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                          cl_map(mb0 + par, (int)(d >> 16)));
         }
     };
+    // checking build: this warp is late now and then (chosen by CTA, warp and exchange)
+    auto perhaps_late = [&] {
+#ifdef AMG_BOUNDS_CHECK
+        if ((5 * rank + 3 * warp + 7 * (int)(kn + ka)) % 11 < 4) __nanosleep(4000);
+#endif
+    };
     // z = 0 on the window, except the colour whose values come next
     auto zero_window = [&](uint32_t z) {  // of the level bound
+        perhaps_late();
 #pragma unroll 1
         for (unsigned k = tid; k < h0.y; k += kClThreads)
             if (k < h1.z || k >= h1.w) cl_st(z + (uint32_t)sizeof(T) * k, T(0));
@@ -554,6 +567,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
         uint4 op = cl_ld<uint4>(dyn + ops);  // a ClOp
 #pragma unroll 1
         for (int k = 0; k < n; k++) {
+            perhaps_late();
             auto relax = [&] {
                 const T fi = cl_ld<T>(f + (uint32_t)sizeof(T) * mi);
                 const T u = (fi - row_dot()) * dinv;
@@ -700,6 +714,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
             vec(roff)[m] = x;
             first_colour(m, zoff, x);
         }
+        __syncthreads();  // every warp's zeros, before the neighbours may send what they leave out
         first_exchange(zoff, q_off(0));
         mark(0, OP_GS_FIRST);
     }
@@ -821,6 +836,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
             };
 #pragma unroll 1
             for (int st = 0; st < nsteps; st++) {
+                perhaps_late();
                 const T *r = st == 0 ? vec(y.F) : Rv;
                 const int q = tid & (LPR - 1);
 #pragma unroll 1
@@ -966,17 +982,17 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                                                           : y.E);
                 const uint32_t par = dyn + CL_F(parent);
                 const uint2 ls = cl_ld<uint2>(dyn + lt1.w + 32);
+                perhaps_late();
 #pragma unroll 1
                 for (unsigned k = tid; k < (unsigned)nwin; k += kClThreads)
                     if (k < ls.x || k >= ls.y) {
                         const uint32_t zk = z + (uint32_t)sizeof(T) * k;
                         cl_st(zk, cl_ld<T>(zk) + cl_ld<T>(en + (uint32_t)sizeof(T) * cl_ld<unsigned short>(par + 2 * k)));
                     }
+                __syncthreads();
                 if (lt2.w == 2) {  // (blocks: the colour swept next is read too, so the neighbours
                     arrive_n(0);   // must have added it everywhere before its rows come in)
                     wait_n();
-                } else {
-                    __syncthreads();
                 }
                 mark(lv, OP_PROLONG);
             }
@@ -996,6 +1012,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                 }
                 const T c = cluster_sum(zq, T(0), nact, nothing, [&](T x, T) { return beta(lv, j, x); }, no_pq);
                 mark(lv, OP_MULTIDOT);
+                perhaps_late();
 #pragma unroll 1
                 for (int k = tid; k < nwin; k += kClThreads) {
                     const uint32_t o = (uint32_t)sizeof(T) * k;
@@ -1032,6 +1049,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                                      [&](T x, T y2) { return alpha(lv, i, x, y2); },
                                      [&](T x) { keep_pq(lv, i, x); });
             mark(lv, OP_SPMV_DOT);
+            perhaps_late();
             // e (+)= alpha p, r = r - alpha q; the next step's first colour
 #pragma unroll 1
             for (int m = tid; m < (int)h0.x;) {
