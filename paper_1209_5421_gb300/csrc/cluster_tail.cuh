@@ -35,7 +35,10 @@
 // zeroed windows at the entry and before a level's first colour, the correction added on the
 // finest level. (The checking build, -DAMG_BOUNDS_CHECK, keeps some warps of every step waiting
 // for a few microseconds, another set each step, so that a missing one shows in the results.)
-// Sums over the cluster and gathers to all CTAs count on two mbarriers of their own.
+// Sums over the cluster and gathers to all CTAs count on two mbarriers of their own, by the same
+// rule: every CTA sends something in each (its sums, its rows of a product, and in the gather into
+// the dense level a token, as it may own no row there), so none is more than one behind. A CTA
+// without rows on any level has no neighbours and is held to the others by these alone.
 //
 // The level above the coarsest: B^ there is linear (the coarsest solve is exact), so setup
 // forms M = B^ and A M as dense matrices once (k_dense_cycle, FP64), each CTA keeps 1/16 of
@@ -622,6 +625,10 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                 cl_store(cl_map(part + (uint32_t)sizeof(T) * (2 * (rank * nact + warp) + (lane >> 4)), lane & (NR - 1)),
                          k, cl_map(mb, lane & (NR - 1)));
         }
+        perhaps_late();
+#ifdef AMG_BOUNDS_CHECK
+        if (npeer == 0) __nanosleep(100000);  // held back by nothing but the sums and gathers
+#endif
         arrive(mb, NR * nact * 2 * (int)sizeof(T));
         before_wait();
         wait_a();
@@ -808,7 +815,9 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                 for (int k = tid; k < NR * nown; k += kClThreads)
                     cl_store(cl_map(to + (uint32_t)sizeof(T) * pi[k >> 4], k & (NR - 1)), stage[k >> 4],
                              cl_map(mb, k & (NR - 1)));
-            arrive(mb, (int)sizeof(T) * y.nd);
+            cl_store_if(alive && warp == kClWarps - 1 && lane < NR, cl_map(cl_smem(&token), lane & (NR - 1)), 0.f,
+                        cl_map(mb, lane & (NR - 1)));
+            arrive(mb, (int)sizeof(T) * y.nd + 4 * NR);
             wait_a();
             mark(lv, OP_RESTRICT);
         }
