@@ -267,6 +267,15 @@ __device__ __noinline__ bool cl_wait_slow(uint32_t mb, unsigned parity, volatile
     }
 }
 
+// A CTA of which a wait ran out, once every CTA has stopped sending: what was under way to its
+// shared memory lands before it leaves. Its image is counted (again with a limit). The stores of
+// an exchange that never completes are not; one takes about 400 cycles, so 100 us are ample.
+__device__ __noinline__ void cl_drain(uint32_t image_mb) {
+    const unsigned long long t0 = global_ns();
+    while (!cl_mb_try(image_mb, 0) && global_ns() - t0 < kBarrierLimitNs) {}
+    while (global_ns() - t0 < 100000) {}
+}
+
 // At these sizes a step is a few dozen instructions per thread, each about 4-5 cycles after the
 // one before, so what counts is the number of instructions between the end of one wait and
 // the stores that end the next. A row's constants (its columns' addresses, values, 1 / a_ii,
@@ -321,6 +330,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (!__syncthreads_and(alive)) {  // no image: the others give up at their first exchange
         cl_sync_all();
+        cl_drain(mb0 + 32);
         return;
     }
     // after an error of an earlier launch of this application the steps run without exchanges
@@ -1120,6 +1130,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                 a.tprof[16 * kMaxLevels + 16 * y.tl + k] += prof_s[1][k];
             }
     cl_sync_all();  // no CTA leaves while a neighbour may still write into it
+    if (*gave_up) cl_drain(mb0 + 32);
     if (a.ts && rank == 0 && tid == 0) *a.ts = global_ns();
 }
 
