@@ -447,6 +447,14 @@ int amg_debug_barrier_fault(amg_hierarchy *h, int64_t limit_ns, int32_t extra);
 int amg_debug_batch_barrier_fault(amg_batch *bt, int64_t limit_ns, int32_t extra);
 
 /*
+ * First level that h's cycle (in its precision, cycle_prec) runs in the thread-block cluster:
+ * 0 the whole cycle, the number of levels none of it, -1 not decided yet (the FP32 cycle, and
+ * every cycle of a batch's hierarchies, is laid out by the first call that runs it).
+ * Tests ask which path they took. Errors: AMG_ERR_INVALID_ARG for NULL arguments.
+ */
+int amg_debug_cluster_level(const amg_hierarchy *h, int32_t *level);
+
+/*
  * Allocation fault: with k > 0 the k-th device allocation the library makes from now on (any
  * thread, any call) fails as if the device were out of memory, so the call making it returns
  * AMG_ERR_OOM after releasing what it had allocated; later allocations succeed again. k = 0

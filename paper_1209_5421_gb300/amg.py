@@ -122,6 +122,8 @@ def lib():
         L.amg_debug_barrier_fault.restype = C.c_int
         L.amg_debug_batch_barrier_fault.argtypes = [P, C.c_int64, C.c_int32]
         L.amg_debug_batch_barrier_fault.restype = C.c_int
+        L.amg_debug_cluster_level.argtypes = [P, C.POINTER(C.c_int32)]
+        L.amg_debug_cluster_level.restype = C.c_int
         L.amg_debug_fail_allocation.argtypes = [C.c_int64]
         L.amg_debug_fail_allocation.restype = C.c_int
         L.amg_debug_pool_bytes_in_use.argtypes = [C.c_int32, C.POINTER(C.c_int64)]
@@ -391,6 +393,13 @@ class Hierarchy:
         """Host-set barrier fault of the cycle kernel for the following solves (0, 0: off)."""
         _check(lib().amg_debug_barrier_fault(self.h, int(limit_ns), int(extra)),
                "amg_debug_barrier_fault")
+
+    def debug_cluster_level(self) -> int:
+        """First level the cycle runs in the cluster (0: all of it, nlev: none, -1: not yet
+        decided)."""
+        v = C.c_int32()
+        _check(lib().amg_debug_cluster_level(self.h, C.byref(v)), "amg_debug_cluster_level")
+        return v.value
 
     def profile(self, enable: bool | int = True):
         """0/False: off; 1/True: per-kernel and per-op timing, tail ops one by one; 2: the

@@ -204,7 +204,6 @@ struct amg_hierarchy {
     std::vector<int *> cell_nat, color_nat;
     // per-level device tables (solve.cu)
     void *lev_tab64 = nullptr, *lev_tab32 = nullptr;
-    int tail_level = -1;
     bool fp32_ready = false;
     amg::BatchWs bws;                  // batched solves (allocated on first use)
     // diagnostics: per-op CUDA-event profiling and launch counts (solve.cu)
@@ -335,6 +334,7 @@ inline void bind_stream(amg_hierarchy *h, void *user_stream) {
 void build_hierarchy(amg_hierarchy *h, const amg_csr &A, const double *x, const double *y,
                      const double *z);
 void free_engines(amg_hierarchy *h);
+int first_cluster_level(const amg_hierarchy *h);  // -1: engine not built
 void profiler_enable(amg_hierarchy *h, int mode);
 void profiler_free(amg_hierarchy *h);
 int profiler_read(const amg_hierarchy *h, int cap, int32_t *kind, int32_t *level,

@@ -694,6 +694,12 @@ int amg_debug_batch_barrier_fault(amg_batch *bt, int64_t limit_ns, int32_t extra
     return AMG_OK;
 }
 
+int amg_debug_cluster_level(const amg_hierarchy *h, int32_t *level) {
+    if (!h || !level) return fail(AMG_ERR_INVALID_ARG, "NULL argument");
+    *level = amg::first_cluster_level(h);
+    return AMG_OK;
+}
+
 int amg_debug_fail_allocation(int64_t k) {
     if (k < 0) return fail(AMG_ERR_INVALID_ARG, "k must be >= 0");
     amg::g_fail_alloc_countdown.store(k);

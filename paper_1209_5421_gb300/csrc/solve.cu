@@ -1351,9 +1351,12 @@ void build_cluster(amg_hierarchy *h, EngineBase *E, int optin) {
     if (last < 0) return;
     int first = last + 1;
     while (first - 1 >= 1 && sweepable(first - 1) && last + 1 - (first - 1) <= kClLevels) first--;
-    // the finest level too, a small quadtree's: then an application is one launch (blocks of one
-    // lane: not the octree's of about eight rows, nor big ones). 65^2 nodes, FP64: 211 -> 153 us
-    // per application, 34^2 nodes: a solve 901 -> 667 us
+    // the finest level too, a small quadtree's: then an application is one launch (a block is one
+    // lane's: not big ones, nor an octree's). 65^2 nodes, FP64: 211 -> 153 us per application, 34^2
+    // nodes: a solve 901 -> 667 us. Blocks of 6 to 16 rows too, although the grid has a lane per
+    // row for them (kCoop): per application, FP64 (FP32), 90^2 nodes over 32^2 cells 185 (145) us
+    // with the finest level on the grid, 145 (106) here; 45^2 over 16^2: 153 (125), 115 (90);
+    // 100^2 over 32^2: 202 (149), 159 (109)
     if (first == 1 && sweepable(0) && last + 1 <= kClLevels && h->dim == 2 && h->lev[0].nbig == 0 &&
         (int)h->lev[0].color_blocks.size() == (int)h->lev[0].color_rows.size())
         first = 0;
@@ -1461,7 +1464,6 @@ void build_engine(amg_hierarchy *h) {
     E->form = (coop_blocks(h->lev[0]) ? kCoop : 0) | (h->lev[0].nbig > 0 ? kBig : 0);
     build_cluster<T>(h, E, optin);
     const int tl = E->cl.tl;
-    h->tail_level = tl;
     Builder b{h, &E->hprog, tl};
     if (tl == 0) b.emit(Builder::mk(OP_TAIL, 0));  // the whole application
     else b.bhat(0, V_RHS, V_E);
@@ -1807,6 +1809,11 @@ size_t level_table_image(amg_hierarchy *h, bool fp32, std::vector<unsigned char>
     std::vector<GLev<double>> tab;
     table_image<double>(h, tab);
     return put(tab);
+}
+
+int first_cluster_level(const amg_hierarchy *h) {
+    const EngineBase *E = h->opt.cycle_prec == AMG_FP32 ? h->eng32 : h->eng64;
+    return E ? E->cl.tl : -1;
 }
 
 void free_engines(amg_hierarchy *h) {
