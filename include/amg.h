@@ -463,6 +463,13 @@ int amg_debug_cluster_level(const amg_hierarchy *h, int32_t *level);
 int amg_debug_fail_allocation(int64_t k);
 
 /*
+ * With on != 0, cycles laid out from now on (any thread) find no room on the device for the
+ * thread-block cluster of the coarse levels, as on a part of a GPU without 16 SMs in one GPC:
+ * every level then runs on the grid. 0 ends it. Cycles laid out before keep their form.
+ */
+int amg_debug_no_cluster(int32_t on);
+
+/*
  * Index checks: in a library built with -DAMG_BOUNDS_CHECK (`python -m
  * paper_1209_5421_gb300.build --bounds-check`), every gather of the cycle's and the batch
  * kernel's ops checks its index against the vector's length; an index outside it is skipped

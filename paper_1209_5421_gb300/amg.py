@@ -124,6 +124,8 @@ def lib():
         L.amg_debug_batch_barrier_fault.restype = C.c_int
         L.amg_debug_cluster_level.argtypes = [P, C.POINTER(C.c_int32)]
         L.amg_debug_cluster_level.restype = C.c_int
+        L.amg_debug_no_cluster.argtypes = [C.c_int32]
+        L.amg_debug_no_cluster.restype = C.c_int
         L.amg_debug_fail_allocation.argtypes = [C.c_int64]
         L.amg_debug_fail_allocation.restype = C.c_int
         L.amg_debug_pool_bytes_in_use.argtypes = [C.c_int32, C.POINTER(C.c_int64)]
@@ -137,6 +139,11 @@ def lib():
 def debug_fail_allocation(k: int):
     """Make the k-th device allocation of the library from now on fail (0: disarm)."""
     _check(lib().amg_debug_fail_allocation(int(k)), "amg_debug_fail_allocation")
+
+
+def debug_no_cluster(on: bool):
+    """Cycles laid out from now on find no room for the cluster on the device (False: ends it)."""
+    _check(lib().amg_debug_no_cluster(int(on)), "amg_debug_no_cluster")
 
 
 def bounds_flags() -> int:

@@ -252,6 +252,7 @@ inline int nblocks_for(int64_t n, int threads) {
 // (amg_debug_fail_allocation) makes the k-th one from then on fail as if the device had no
 // memory left: it throws the library's out-of-memory error without calling CUDA.
 bool fail_this_allocation();  // capi.cu: counts down the armed fault
+bool fault_no_cluster();      // capi.cu: host-set (amg_debug_no_cluster)
 inline void device_alloc(void **p, size_t bytes, cudaStream_t s) {
     if (fail_this_allocation())
         throw Error{AMG_ERR_OOM, "device allocation failed (host-set fault)"};

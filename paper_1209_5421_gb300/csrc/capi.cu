@@ -29,6 +29,8 @@ int set_last_error(int status, const char *what) { return fail(status, what); }
 
 // host-set allocation fault: 0 = off, k > 0 = the k-th device allocation from now fails
 static std::atomic<int64_t> g_fail_alloc_countdown{0};
+static std::atomic<bool> g_no_cluster{false};
+bool fault_no_cluster() { return g_no_cluster.load(std::memory_order_relaxed); }
 bool fail_this_allocation() {
     int64_t k = g_fail_alloc_countdown.load(std::memory_order_relaxed);
     while (k > 0) {
@@ -703,6 +705,11 @@ int amg_debug_cluster_level(const amg_hierarchy *h, int32_t *level) {
 int amg_debug_fail_allocation(int64_t k) {
     if (k < 0) return fail(AMG_ERR_INVALID_ARG, "k must be >= 0");
     amg::g_fail_alloc_countdown.store(k);
+    return AMG_OK;
+}
+
+int amg_debug_no_cluster(int32_t on) {
+    amg::g_no_cluster.store(on != 0);
     return AMG_OK;
 }
 

@@ -1306,6 +1306,42 @@ void *cluster_kernel() {
     return (void *)k_cluster_tail<T>;
 }
 
+// Launch of the cluster with `smem` bytes per CTA; attr: two attributes of the caller's. Its image
+// may come in while the launch before it ends.
+cudaLaunchConfig_t cluster_config(size_t smem, cudaStream_t s, cudaLaunchAttribute *attr) {
+    cudaLaunchConfig_t cfg;
+    std::memset(&cfg, 0, sizeof cfg);
+    cfg.gridDim = dim3(kClRanks);
+    cfg.blockDim = dim3(kClThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = kClRanks;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
+    return cfg;
+}
+
+// Can the device (or the part of it this process has) hold a cluster of 16 CTAs, one per SM?
+// That takes 16 SMs of one GPC; without them every level runs on the grid.
+template <class T>
+bool cluster_fits(size_t smem, cudaStream_t s) {
+    if (fault_no_cluster()) return false;
+    cudaLaunchAttribute attr[2];
+    const cudaLaunchConfig_t cfg = cluster_config(smem, s, attr);
+    int clusters = 0;
+    if (cudaFuncSetAttribute(cluster_kernel<T>(), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess &&
+        cudaFuncSetAttribute(cluster_kernel<T>(), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+        cudaOccupancyMaxActiveClusters(&clusters, cluster_kernel<T>(), &cfg) == cudaSuccess)
+        return clusters > 0;
+    cudaGetLastError();
+    return false;
+}
+
 // Chooses the cluster's levels (the finest level from which everything fits) and builds their
 // image. E->cl.tl = nlev if there are none: every level runs on the grid.
 template <class T>
@@ -1317,9 +1353,7 @@ void build_cluster(amg_hierarchy *h, EngineBase *E, int optin) {
     cudaFuncAttributes fa;
     AMG_CUDA(cudaFuncGetAttributes(&fa, cluster_kernel<T>()));
     const long budget = (long)optin - (long)fa.sharedSizeBytes;
-    AMG_CUDA(cudaFuncSetAttribute(cluster_kernel<T>(), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)budget));
-    AMG_CUDA(cudaFuncSetAttribute(cluster_kernel<T>(), cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    if (!cluster_fits<T>((size_t)budget, s)) return;
     const std::vector<int> widths = slice_widths(h);
     auto sweepable = [&](int l) {
         const Level &lv = h->lev[l];
@@ -1627,20 +1661,7 @@ void launch_cycle(amg_hierarchy *h, T *rhs0 = nullptr, T *e0 = nullptr) {
         ca.limit_ns = a.bar_limit_ns;
         ca.extra = h->dbg_bar_extra;
         ca.tprof = (prof && h->prof->tail_ops) ? E->tprof : nullptr;
-        std::memset(&cfg, 0, sizeof cfg);
-        cfg.gridDim = dim3(kClRanks);
-        cfg.blockDim = dim3(kClThreads);
-        cfg.dynamicSmemBytes = (size_t)E->cl.bytes;
-        cfg.stream = s;
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = kClRanks;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        // its image may come in while the launch before it ends
-        attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[1].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 2;
+        cfg = cluster_config((size_t)E->cl.bytes, s, attr);
     }
     unsigned long long bars = 0;  // barriers of the launches so far
     for (int k = 0; k < E->nops;) {

@@ -4,6 +4,7 @@
   on the grid with the coarse levels in the cluster;
 * a quadtree with blocks of several rows (the lane-parallel block smoother) whose finest level
   is on the grid;
+* a device without room for the cluster (host-set): every level on the grid;
 * the bounded waits made to run out on either path (a host-set limit of 1 ms and a first wait
   for more than comes): AMG_ERR_TIMEOUT, then the same bits as before.
 
@@ -90,4 +91,32 @@ def test_timeout_on_either_path(amg, n, whole, prec):
     H.debug_barrier_fault(0, 0)
     x1, it1, _, st1 = H.solve(prob.b, 1e-8)
     assert st1 == amg.OK and it1 == it0 and np.array_equal(x1, x0)
+    H.close()
+
+
+@pytest.fixture
+def no_cluster(amg):
+    amg.debug_no_cluster(True)
+    yield
+    amg.debug_no_cluster(False)
+
+
+@pytest.mark.parametrize("prec", PRECS)
+@pytest.mark.parametrize("mesh,n", [
+    (_square, 34), (_square, 257), (lambda n: disk_poisson(n, jitter=0.2, seed=n), 51),
+    (lambda n: p1_poisson_3d(n, seed=n), 17)])
+def test_every_level_on_the_grid(amg, no_cluster, mesh, n, prec):
+    from oracle import oracle
+
+    prob = mesh(n)
+    O = oracle.Hierarchy.from_problem(prob)
+    H = _hierarchy(amg, prob, prec)
+    z, zo = H.apply_cycle(0, prob.b), O.bhat(0, prob.b)
+    assert H.debug_cluster_level() == H.nlev
+    rel = np.linalg.norm(z - zo) / np.linalg.norm(zo)
+    assert rel <= (1e-11 if prec == "fp64" else 1e-5), rel
+    x, it, _, st = H.solve(prob.b, 1e-8)
+    assert st == amg.OK
+    if prec == "fp64":  # the plain method: the oracle's iteration count within one
+        assert abs(it - O.solve(prob.b, 1e-8)[1]) <= 1
     H.close()
