@@ -276,6 +276,9 @@ __device__ __noinline__ void cl_drain(uint32_t image_mb) {
     while (global_ns() - t0 < 100000) {}
 }
 
+// a / b out of line, for the rare case (the kernel's code is larger than an SM's instruction cache)
+__device__ __noinline__ double cl_quotient(double a, double b) { return a / b; }
+
 // At these sizes a step is a few dozen instructions per thread, each about 4-5 cycles after the
 // one before, so what counts is the number of instructions between the end of one wait and
 // the stores that end the next. A row's constants (its columns' addresses, values, 1 / a_ii,
@@ -297,8 +300,8 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
     __shared__ __align__(8) unsigned long long mbs[5];   // neighbours x 2, all CTAs x 2, image
     __shared__ __align__(16) T red[2][NR * kClWarps][2]; // sums over the cluster: the warps'
     __shared__ T coef_s[6];
-    __shared__ T pqs[kClLevels + 1][kMaxKcycle];         // (p_i, A p_i) of every level; FP64:
-                                                         //   its reciprocal (0: not positive)
+    __shared__ T pqs[kClLevels + 1][kMaxKcycle];         // (p_i, A p_i) of every level
+    __shared__ T inv_s[F64 ? kClLevels + 1 : 1][kMaxKcycle][2];  // FP64: its reciprocal, two parts
     __shared__ int stops[kClLevels + 1][kMaxKcycle];     // Alg. 1 stopped at or before step i
     __shared__ int gave_up_s, token;
     volatile int *gave_up = &gave_up_s;
@@ -682,15 +685,31 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
         if (tid == 0) stops[lv][i] = stopped;
         return stopped ? T(0) : (T)ratio<T>((double)rp, (double)pq);
     };
+    // FP64: a division takes about 560 cycles, so 1 / pq is kept, off the path to the next step, as
+    // a sum of two doubles (error of about 2^-106): zq / pq is then a product and an FMA, rounded
+    // once but for 2^-53 of a rounding. Only where neither part leaves the normal range (pq of 2^-960
+    // to 2^960); elsewhere (0 here) a division. Every beta by a division, 257^2 nodes: 6.13 -> 6.22 ms
+    // per solve; in this form 6.16 (by 1 / pq alone, rounded twice and infinite for a subnormal
+    // pq, 6.13).
     auto keep_pq = [&](int lv, int i, T pq) {
-        T k = pq;
-        if constexpr (F64) k = positive(pq) ? T(1) / pq : T(0);  // off the path to the next step
-        if (tid == (F64 ? 32 : 0)) pqs[lv][i] = k;
+        if (tid != (F64 ? 32 : 0)) return;
+        pqs[lv][i] = pq;
+        if constexpr (F64) {
+            const unsigned long long e = (unsigned long long)__double_as_longlong(pq) >> 52;
+            const bool ok = e - (1023 - 960) <= 2 * 960;  // sign bit clear: positive
+            const T k = ok ? T(1) / pq : T(0);
+            inv_s[lv][i][0] = k;
+            inv_s[lv][i][1] = ok ? k * fma(-k, pq, T(1)) : T(0);
+        }
     };
     auto beta = [&](int lv, int j, T zq) {
-        const T k = pqs[lv][j];
-        if constexpr (F64) return -(zq * k);
-        else return k > T(0) ? -(T)ratio<T>((double)zq, (double)k) : T(0);
+        if constexpr (F64) {
+            const T k = inv_s[lv][j][0], k2 = inv_s[lv][j][1];
+            if (__double_as_longlong(k) != 0) return -fma(zq, k, zq * k2);
+        }
+        const T pq = pqs[lv][j];
+        if constexpr (F64) return positive(pq) ? -cl_quotient(zq, pq) : T(0);
+        else return positive(pq) ? -(T)ratio<T>((double)zq, (double)pq) : T(0);
     };
     auto nothing = [] {};
     auto no_pq = [](T) {};

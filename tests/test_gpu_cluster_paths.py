@@ -5,6 +5,7 @@
 * a quadtree with blocks of several rows (the lane-parallel block smoother) whose finest level
   is on the grid;
 * a device without room for the cluster (host-set): every level on the grid;
+* a right-hand side so small that (p, A p) of Alg. 1 is subnormal;
 * the bounded waits made to run out on either path (a host-set limit of 1 ms and a first wait
   for more than comes): AMG_ERR_TIMEOUT, then the same bits as before.
 
@@ -119,4 +120,20 @@ def test_every_level_on_the_grid(amg, no_cluster, mesh, n, prec):
     assert st == amg.OK
     if prec == "fp64":  # the plain method: the oracle's iteration count within one
         assert abs(it - O.solve(prob.b, 1e-8)[1]) <= 1
+    H.close()
+
+
+@pytest.mark.parametrize("n,opts", [(34, {}), (34, dict(kcycle_n=3)), (257, {}), (257, dict(kcycle_n=3))])
+def test_subnormal_energy(amg, n, opts):
+    # B^ is homogeneous, so B^[c f] / c is B^[f], with c chosen so that (p, A p) is about
+    # 2^-1030: a sum of n products, each rounded by at most 2^-1075, has a relative error of
+    # n 2^-45 (5e-10 at the cluster's 16,384 rows); a few such sums in turn: bar 1e-6
+    prob = _square(n)
+    H = _hierarchy(amg, prob, "fp64", **opts)
+    f = np.ones(prob.n)
+    z = H.apply_cycle(0, f)
+    c = 2.0 ** np.floor((-1030 - np.log2(f @ z)) / 2)
+    zc = H.apply_cycle(0, c * f) / c
+    assert np.isfinite(zc).all()
+    assert np.linalg.norm(zc - z) <= 1e-6 * np.linalg.norm(z)
     H.close()
