@@ -43,10 +43,15 @@
 // The level above the coarsest: B^ there is linear (the coarsest solve is exact), so setup
 // forms M = B^ and A M as dense matrices once (k_dense_cycle, FP64), each CTA keeps 1/16 of
 // their rows, and one product with a residual gives p and A p of an Alg. 1 step; that replaces
-// about 13 dependent steps. FP64 keeps M alone and multiplies by the sparse A after it (256
-// rows: a product with both is 4,900 cycles of the FP64 pipe, with M 2,450 and one more gather
-// 600: 9.7 -> 8.8 us per visit). Where the matrices do not fit, the level is swept like the
-// others and the coarsest solve is the dense product.
+// about 13 dependent steps. In FP32 M takes the coarsest inverse's place and is held like it, as a
+// sum of two floats with a compensated product, so p is rounded once; A M is one float with a plain
+// sum, as A itself is where a level is swept (its error, of the order of eps |A M| |r|, is below
+// the eps |A| |p| of a product with A, which also bounds A p - q for the rounded p). FP64
+// keeps M alone and multiplies by the sparse A after it (256 rows: a product with both is 4,900
+// cycles of the FP64 pipe, with M 2,450 and one more gather 600: 9.7 -> 8.8 us per visit). So does
+// FP32 where M's two parts fit but not A M beside them (512 rows); A's few rows per CTA are then read
+// through L1. Where M does not fit, the level is swept like the others and the coarsest solve is
+// the dense product.
 #pragma once
 
 #include <cstddef>
@@ -107,22 +112,23 @@ struct ClLayout {
     int dense;         // 1: M and A M of the level above the coarsest, 0: coarsest inverse
     int kc, nu_pre, nu_post;
     int nd, ch, stride;  // dense level: rows, rows per CTA (multiple of 4), row stride
-    int mat, mat_lo;     // M then A M (or the inverse; FP32: high parts, low parts)
-    int aw, aval, acol;  // FP64: M alone, and A's rows: slots per row, values, columns
+    int mat, mat_lo;     // M, FP32: then A M (or the inverse); FP32: M's (the inverse's) low parts
+    int aw, aval, acol;  // > 0: M alone, and A's rows: slots per row, values, columns (FP32: in the
+                         //   image beyond what is copied)
     int dhead, down;     // gather into the dense level: own rows (count; their pi-rows)
     int peers;           // neighbour CTAs: count, ranks
     int levels;          // lv[] (a copy in the image)
     int top;             // pi-rows of the top level's own rows
     int F, Rv, E, out, P[kMaxKcycle], Q[kMaxKcycle];  // dense level's vectors (every CTA: all)
     int stage;           // one value per own row of the dense level
-    int image_bytes, bytes;
+    int image_bytes, image_stride, bytes;  // copied; one CTA's; shared memory
     ClLev lv[kClLevels];
 };
 
 template <class T>
 struct ClArgs {
     ClLayout y;
-    const unsigned char *image;  // [kClRanks][image_bytes]
+    const unsigned char *image;  // [kClRanks][image_stride]
     const T *rhs;                // level tl, pi order
     T *e;
     int *err;
@@ -322,7 +328,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
         cl_mb_expect(mb0 + 32, y.image_bytes);
         asm volatile(
             "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dyn),
-            "l"(a.image + (size_t)rank * y.image_bytes), "r"(y.image_bytes), "r"(mb0 + 32)
+            "l"(a.image + (size_t)rank * y.image_stride), "r"(y.image_bytes), "r"(mb0 + 32)
             : "memory");
     }
     cl_sync_all();  // every CTA's mbarriers are ready
@@ -854,9 +860,67 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
         {
             const int ch = y.ch, len = NR * ch;
             T *E = vec(y.E), *out = vec(y.out), *Rv = vec(y.Rv);
-            const int nsteps = y.dense ? y.kc : 1, parts = y.dense && !F64 ? 2 : 1;
+            const int nsteps = y.dense ? y.kc : 1, parts = y.dense && y.aw == 0 ? 2 : 1;
             constexpr int LPR = 8;  // lanes per row
             constexpr int V = 16 / (int)sizeof(T);
+            // FP32: [z; w] = [M; A M] r, 16 lanes per row, 16-byte reads; M r as a compensated sum
+            // (Dot2 of Ogita, Rump and Oishi), four of them per lane. Bound by its 11 instructions
+            // per entry: 256 rows 3.5 us per visit with M in one float and a plain sum, 3.9 so;
+            // 512 rows 5.8, 8.7. The error of one application against FP64, over that of the
+            // coarsest inverse in two parts with this level swept (540 right-hand sides, squares,
+            // disks, cubes, graded): 1.01 in the mean with one float, 0.985 so
+            auto dense_product = [&](const T *r, T *out) {
+                if constexpr (!F64) {
+                    const float *hi = vec(y.mat), *lo = vec(y.mat_lo), *am = hi + (size_t)ch * y.stride;
+                    const int q = tid & 15;
+#pragma unroll 1
+                    for (int row = tid >> 4; row < ch; row += kClThreads / 16) {
+                        const size_t o = (size_t)row * y.stride;
+                        float s[4] = {0.f, 0.f, 0.f, 0.f}, e[4] = {0.f, 0.f, 0.f, 0.f}, w0 = 0.f, w1 = 0.f;
+                        auto add = [&](int k, float m, float l, float x) {
+                            const float ph = __fmul_rn(m, x);
+                            const float pe = fmaf(l, x, fmaf(m, x, -ph));
+                            float t2, e2;
+                            two_sum(s[k], ph, t2, e2);
+                            s[k] = t2;
+                            e[k] = __fadd_rn(e[k], __fadd_rn(e2, pe));
+                        };
+                        auto join = [&](float s1, float e1) {
+                            float t2, e2;
+                            two_sum(s[0], s1, t2, e2);
+                            s[0] = t2;
+                            e[0] = __fadd_rn(e[0], __fadd_rn(e1, e2));
+                        };
+#pragma unroll 2
+                        for (int j = 4 * q; j < len; j += 64) {
+                            const float4 xv = *(const float4 *)(r + j), hv = *(const float4 *)(hi + o + j),
+                                         lv4 = *(const float4 *)(lo + o + j);
+                            add(0, hv.x, lv4.x, xv.x);
+                            add(1, hv.y, lv4.y, xv.y);
+                            add(2, hv.z, lv4.z, xv.z);
+                            add(3, hv.w, lv4.w, xv.w);
+                            if (parts == 2) {
+                                const float4 av = *(const float4 *)(am + o + j);
+                                w0 += av.x * xv.x;
+                                w1 += av.y * xv.y;
+                                w0 += av.z * xv.z;
+                                w1 += av.w * xv.w;
+                            }
+                        }
+                        for (int k = 1; k < 4; k++) join(s[k], e[k]);
+                        w0 += w1;
+#pragma unroll
+                        for (int d = 8; d > 0; d >>= 1) {
+                            join(__shfl_xor_sync(0xffffffffu, s[0], d), __shfl_xor_sync(0xffffffffu, e[0], d));
+                            w0 += __shfl_xor_sync(0xffffffffu, w0, d);
+                        }
+                        if (q == 0) {
+                            out[row] = __fadd_rn(s[0], e[0]);
+                            if (parts == 2) out[ch + row] = w0;
+                        }
+                    }
+                }
+            };
             // this CTA's rows of a product (in `out`: `parts` times ch values) to every CTA
             auto gather_out = [&](int o0, int o1) {
                 __syncthreads();
@@ -877,29 +941,23 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                 perhaps_late();
                 const T *r = st == 0 ? vec(y.F) : Rv;
                 const int q = tid & (LPR - 1);
+                if constexpr (!F64)
+                    if (y.dense) dense_product(r, out);
 #pragma unroll 1
-                for (int row = tid / LPR; row < parts * ch; row += kClThreads / LPR) {
+                for (int row = tid / LPR; row < (!F64 && y.dense ? 0 : ch); row += kClThreads / LPR) {
                     const T *m = vec(y.mat) + (size_t)row * y.stride;
                     T sum = 0, err = 0;
-                    if (F64 || y.dense) {  // [z; w] = [M; A M] r (or A^{-1} r): 16-byte reads
+                    if constexpr (F64) {  // z = M r (or A^{-1} r): 16-byte reads
 #pragma unroll 8
                         for (int j = q * V; j < len; j += LPR * V) {
-                            if constexpr (!F64) {
-                                const float4 mv = *(const float4 *)(m + j), xv = *(const float4 *)(r + j);
-                                sum += mv.x * xv.x;
-                                err += mv.y * xv.y;
-                                sum += mv.z * xv.z;
-                                err += mv.w * xv.w;
-                            } else {
-                                const double2 mv = *(const double2 *)(m + j), xv = *(const double2 *)(r + j);
-                                sum += mv.x * xv.x;
-                                err += mv.y * xv.y;
-                            }
+                            const double2 mv = *(const double2 *)(m + j), xv = *(const double2 *)(r + j);
+                            sum += mv.x * xv.x;
+                            err += mv.y * xv.y;
                         }
                         sum += err;
 #pragma unroll
                         for (int o = LPR / 2; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-                    } else if constexpr (!F64) {  // A^{-1} r in FP32: op_coarse's compensated sum
+                    } else {  // A^{-1} r in FP32: op_coarse's compensated sum
                         const T *ml = vec(y.mat_lo) + (size_t)row * y.stride;
 #pragma unroll 1
                         for (int j = q; j < y.nd; j += LPR) {
@@ -925,14 +983,15 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                     if (q == 0) out[row] = sum;
                 }
                 gather_out(y.dense ? y.P[st] : y.E, y.Q[st]);
-                if (F64 && y.dense) {  // w = A z: four lanes per row
-                    const T *z = vec(y.P[st]), *av = vec(y.aval);
-                    const unsigned short *ac = (const unsigned short *)at(y.acol);
+                if (y.aw > 0) {  // w = A z: four lanes per row
+                    const unsigned char *A = F64 ? at(0) : a.image + (size_t)rank * y.image_stride;
+                    const T *z = vec(y.P[st]), *av = (const T *)(A + y.aval);
+                    const unsigned short *ac = (const unsigned short *)(A + y.acol);
                     const int row = tid >> 2;
                     if (32 * warp < 4 * ch) {
                         T sum = 0;
                         if (row < ch)
-#pragma unroll 1
+#pragma unroll (F64 ? 1 : 4)
                             for (int k = tid & 3; k < y.aw; k += 4) sum += av[k * ch + row] * z[ac[k * ch + row]];
                         sum += __shfl_xor_sync(0xffffffffu, sum, 1);
                         sum += __shfl_xor_sync(0xffffffffu, sum, 2);
@@ -1284,20 +1343,23 @@ __global__ void k_cl_image(const __grid_constant__ ClSrcs G, const __grid_consta
                            unsigned char *image, const ClColor *geo, int *over_n,
                            const double *Ainv, const float *Ainv2) {
     const int a = blockIdx.z, r = blockIdx.y;
-    unsigned char *im = image + (size_t)r * y.image_bytes;
+    unsigned char *im = image + (size_t)r * y.image_stride;
     const int t0 = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
     if (a == y.nsp) {
-        if (y.dense) {  // FP64: A's rows (columns are pi-rows)
-            if constexpr (sizeof(T) == 8) {
-                const ClSrc &S = G.lv[a];
-                for (int k = t0; k < y.ch * y.aw; k += nt) {
-                    const int row = k % y.ch, slot = k / y.ch, i = r * y.ch + row;
-                    if (i >= y.nd) continue;
-                    const int s0 = S.sl[i >> 5], width = (S.sl[(i >> 5) + 1] - s0) >> 5;
-                    const int o = s0 + 32 * slot + (i & 31), j = slot < width ? S.col[o] : -1;
-                    ((unsigned short *)(im + y.acol))[k] = (unsigned short)(j >= 0 ? j : i);
-                    ((double *)(im + y.aval))[k] = j >= 0 ? S.val64[o] : 0.0;
+        if (y.dense) {  // A's rows (columns are pi-rows)
+            const ClSrc &S = G.lv[a];
+            for (int k = t0; k < y.ch * y.aw; k += nt) {
+                const int row = k % y.ch, slot = k / y.ch, i = r * y.ch + row;
+                if (i >= y.nd) continue;
+                const int s0 = S.sl[i >> 5], width = (S.sl[(i >> 5) + 1] - s0) >> 5;
+                const int o = s0 + 32 * slot + (i & 31), j = slot < width ? S.col[o] : -1;
+                ((unsigned short *)(im + y.acol))[k] = (unsigned short)(j >= 0 ? j : i);
+                T v = T(0);
+                if (j >= 0) {
+                    if constexpr (sizeof(T) == 8) v = S.val64[o];
+                    else v = S.val32[o];
                 }
+                ((T *)(im + y.aval))[k] = v;
             }
             return;
         }
@@ -1456,9 +1518,14 @@ k_dense_cycle(const __grid_constant__ ClSrc S, const __grid_constant__ ClLayout 
     for (int sw = 0; sw < y.nu_post; sw++)
         for (int c = S.ncol - 1; c >= 0; c--) sweep(c);
     for (int i = tid; i < n; i += nt) {
-        T *row = (T *)(image + (size_t)(i / y.ch) * y.image_bytes + y.mat) + (size_t)(i % y.ch) * y.stride;
-        row[unit] = (T)z[i];
-        if constexpr (sizeof(T) == 4) row[(size_t)y.ch * y.stride + unit] = (T)dot(i, 0);
+        unsigned char *im = image + (size_t)(i / y.ch) * y.image_stride;
+        const size_t o = (size_t)(i % y.ch) * y.stride + unit;
+        const T hi = (T)z[i];
+        ((T *)(im + y.mat))[o] = hi;
+        if constexpr (sizeof(T) == 4) {
+            ((T *)(im + y.mat_lo))[o] = (T)(z[i] - (double)hi);
+            if (y.aw == 0) ((T *)(im + y.mat))[(size_t)y.ch * y.stride + o] = (T)dot(i, 0);
+        }
     }
 }
 

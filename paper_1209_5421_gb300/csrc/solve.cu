@@ -1045,10 +1045,10 @@ int2 cl_own_rows(const ClSrc &S, const std::vector<int> &hb, int r, int c) {
 // Layout and tables for the swept levels G.lv[s0 ..] (hierarchy levels level0 ..) and the dense
 // level after them, or false if they do not fit `budget` bytes of shared memory. win: their
 // windows; xchild: [2][nlv], by the next level's kind (swept, dense); fo: owner of each row of
-// the dense level.
+// the dense level; sparse: M alone and the sparse A after it.
 template <class T>
 bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vector<int> &xchild, int nlv,
-                  const int *fo, const std::vector<int> &hb, const std::vector<int> &widths, int s0, int level0, bool dense, int nch,
+                  const int *fo, const std::vector<int> &hb, const std::vector<int> &widths, int s0, int level0, bool dense, bool sparse, int nch,
                   const amg_options &opt, long budget, ClPlan &P) {
     constexpr int vb = (int)sizeof(T), NR = kClRanks;
     ClLayout &y = P.y;
@@ -1245,14 +1245,21 @@ bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vect
         else L.child = take(2 * (size_t)nch * L.Rn);
     }
     y.top = take(sizeof(int) * max_own[0]);
-    y.mat = take((size_t)(dense && vb == 4 ? 2 : 1) * y.ch * y.stride * vb);
-    if (dense && vb == 8) {
+    // dense level: FP32 M's high parts and A M (unless the product with A is sparse), M's low parts; FP64
+    // M. Without it, the coarsest inverse, in FP32 its two parts
+    const size_t rows_bytes = (size_t)y.ch * y.stride * vb;
+    y.mat = take((dense && !sparse ? 2 : 1) * rows_bytes);
+    if (vb == 4) y.mat_lo = take(rows_bytes);
+    size_t beyond = 0;
+    if (dense && sparse) {
         y.aw = widths[level0 + y.nsp];
-        y.aval = take((size_t)y.aw * y.ch * vb);
-        y.acol = take((size_t)y.aw * y.ch * 2);
+        const size_t val_bytes = align16((size_t)y.aw * y.ch * vb), col_bytes = align16((size_t)y.aw * y.ch * 2);
+        if (vb == 4) beyond = val_bytes + col_bytes;
+        y.aval = vb == 4 ? (int)off : take(val_bytes);
+        y.acol = vb == 4 ? (int)(off + val_bytes) : take(col_bytes);
     }
-    if (!dense && vb == 4) y.mat_lo = take((size_t)y.ch * y.stride * vb);
     y.image_bytes = (int)off;
+    y.image_stride = (int)(off + beyond);
     for (int a = 0; a < y.nsp; a++) {
         ClLev &L = y.lv[a];
         const size_t b = max_win[a] * vb;
@@ -1447,11 +1454,12 @@ void build_cluster(amg_hierarchy *h, EngineBase *E, int optin) {
     bool ok = false;
     int s0 = 0;
     for (; s0 < G.nsp; s0++) {
-        ok = can_dense && cluster_plan<T>(GD, win, xchild, G.nsp, fo.data() + nc, hb, widths, s0, first + s0, true,
-                                          nch, h->opt, budget, P);
+        for (int sparse = sizeof(T) == 8; !ok && can_dense && sparse < 2; sparse++)
+            ok = cluster_plan<T>(GD, win, xchild, G.nsp, fo.data() + nc, hb, widths, s0, first + s0, true, sparse != 0,
+                                 nch, h->opt, budget, P);
         if (!ok)
-            ok = cluster_plan<T>(G, win, xchild, G.nsp, fo.data(), hb, widths, s0, first + s0, false, nch, h->opt,
-                                 budget, P);
+            ok = cluster_plan<T>(G, win, xchild, G.nsp, fo.data(), hb, widths, s0, first + s0, false, false, nch,
+                                 h->opt, budget, P);
         if (ok) break;
     }
     if (!ok) return;
@@ -1461,9 +1469,9 @@ void build_cluster(amg_hierarchy *h, EngineBase *E, int optin) {
         for (int a = 0; a + s0 <= U.nsp; a++) U.lv[a] = U.lv[a + s0];
         U.nsp -= s0;
     }
-    E->cl_image = halloc<unsigned char>(h, (size_t)kClRanks * y.image_bytes);
-    AMG_CUDA(cudaMemsetAsync(E->cl_image, 0, (size_t)kClRanks * y.image_bytes, s));
-    AMG_CUDA(cudaMemcpy2DAsync(E->cl_image, y.image_bytes, P.tables.data(), P.table_bytes, P.table_bytes,
+    E->cl_image = halloc<unsigned char>(h, (size_t)kClRanks * y.image_stride);
+    AMG_CUDA(cudaMemsetAsync(E->cl_image, 0, (size_t)kClRanks * y.image_stride, s));
+    AMG_CUDA(cudaMemcpy2DAsync(E->cl_image, y.image_stride, P.tables.data(), P.table_bytes, P.table_bytes,
                                kClRanks, cudaMemcpyHostToDevice, s));
     const Level &C = h->lev[nlev - 1];
     ClColor *geo = tmp.get<ClColor>(P.geo.size());
