@@ -472,8 +472,10 @@ int amg_debug_no_cluster(int32_t on);
 /*
  * Index checks: in a library built with -DAMG_BOUNDS_CHECK (`python -m
  * paper_1209_5421_gb300.build --bounds-check`), every gather of the cycle's and the batch
- * kernel's ops checks its index against the vector's length; an index outside it is skipped
- * and sets a flag. *flags receives the flags set since the last call (0: none) and clears
+ * kernel's ops, and every store of the cluster's into another CTA, checks its index against
+ * the vector's length (a store's against the shared memory); an index outside it is skipped and
+ * sets a flag. That build also makes warps of the cluster's kernel late now and then, so that
+ * a missing wait shows. *flags receives the flags set since the last call (0: none) and clears
  * them. Errors: AMG_ERR_UNSUPPORTED in a library built without the checks (the default).
  */
 int amg_debug_bounds_flags(int32_t *flags);

@@ -403,6 +403,11 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
     unsigned long long steps = 0;  // Alg. 1 step of every swept level, 4 bits each
     // the destinations as addresses: (place, mbarrier) of two, mapped once
     for (int l = 0; l < y.nsp; l++) {
+        int last = 0;  // (index checks: the level's last window vector)
+#ifdef AMG_BOUNDS_CHECK
+        last = lvs[l].e;
+        for (int k = 0; k < kMaxKcycle; k++) last = max(last, max(lvs[l].p[k], lvs[l].q[k]));
+#endif
         uint4 *d = (uint4 *)at(lvs[l].dst);
         const int nown = ((const ClHead *)at(lvs[l].head))->nown;
 #pragma unroll 1
@@ -410,6 +415,10 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
             uint4 q = d[m];
             auto place = [&](unsigned &p, unsigned &b) {
                 if (p >> 31 || p == kClNone) return;  // further ones: stays as it is
+                if (!idx_ok((int)(p >> 16), NR) || !idx_ok(last + (int)(p & 0xFFFFu), y.bytes)) {
+                    p = kClNone;
+                    return;
+                }
                 b = cl_map(mb0, (int)(p >> 16));
                 p = cl_map(dyn, (int)(p >> 16)) + (p & 0xFFFFu);
             };
@@ -473,6 +482,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
         mi = m;
         own = has && (o & ((1 << lt2.x) - 1)) == 0;
         lb = cl_ld<unsigned short>(dyn + lt0.x + 2 * m);
+        if (has && !idx_ok((int)lb, (int)sizeof(T) * (int)h0.y)) lb = 0;
         const uint4 c = cl_ld<uint4>(dyn + lt0.y + 16 * o);
         dg = cl_ld<T>(dyn + lt0.w + (int)sizeof(T) * m);
         if constexpr (!F64) {
@@ -563,7 +573,8 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
             const unsigned *list = (const unsigned *)at(lt1.z) + (more & 0x7FFFFFFFu);
 #pragma unroll 1
             for (unsigned d = *list; d != kClNone; d = *++list)
-                cl_store(cl_map(dyn + off + (d & 0xFFFFu), (int)(d >> 16)), u,
+                if (idx_ok((int)(d >> 16), NR) && idx_ok(off + (int)(d & 0xFFFFu), y.bytes))
+                    cl_store(cl_map(dyn + off + (d & 0xFFFFu), (int)(d >> 16)), u,
                          cl_map(mb0 + par, (int)(d >> 16)));
         }
     };
@@ -848,8 +859,9 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
             if (alive)
 #pragma unroll 1
                 for (int k = tid; k < NR * nown; k += kClThreads)
-                    cl_store(cl_map(to + (uint32_t)sizeof(T) * pi[k >> 4], k & (NR - 1)), stage[k >> 4],
-                             cl_map(mb, k & (NR - 1)));
+                    if (idx_ok((int)pi[k >> 4], y.nd))
+                        cl_store(cl_map(to + (uint32_t)sizeof(T) * pi[k >> 4], k & (NR - 1)), stage[k >> 4],
+                                 cl_map(mb, k & (NR - 1)));
             cl_store_if(alive && warp == kClWarps - 1 && lane < NR, cl_map(cl_smem(&token), lane & (NR - 1)), 0.f,
                         cl_map(mb, lane & (NR - 1)));
             arrive(mb, (int)sizeof(T) * y.nd + 4 * NR);
@@ -992,7 +1004,10 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                         T sum = 0;
                         if (row < ch)
 #pragma unroll (F64 ? 1 : 4)
-                            for (int k = tid & 3; k < y.aw; k += 4) sum += av[k * ch + row] * z[ac[k * ch + row]];
+                            for (int k = tid & 3; k < y.aw; k += 4) {
+                                const int j = ac[k * ch + row];
+                                if (idx_ok(j, y.nd)) sum += av[k * ch + row] * z[j];
+                            }
                         sum += __shfl_xor_sync(0xffffffffu, sum, 1);
                         sum += __shfl_xor_sync(0xffffffffu, sum, 2);
                         if (row < ch && (tid & 3) == 0) out[row] = sum;
@@ -1079,12 +1094,14 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                                                           : y.E);
                 const uint32_t par = dyn + CL_F(parent);
                 const uint2 ls = cl_ld<uint2>(dyn + lt1.w + 32);
+                const int nen = lv + 1 < y.nsp ? ((const ClHead *)at(lvs[lv + 1].head))->nwin : y.nd;  // (index checks)
                 perhaps_late();
 #pragma unroll 1
                 for (unsigned k = tid; k < (unsigned)nwin; k += kClThreads)
                     if (k < ls.x || k >= ls.y) {
                         const uint32_t zk = z + (uint32_t)sizeof(T) * k;
-                        cl_st(zk, cl_ld<T>(zk) + cl_ld<T>(en + (uint32_t)sizeof(T) * cl_ld<unsigned short>(par + 2 * k)));
+                        const unsigned pk = cl_ld<unsigned short>(par + 2 * k);
+                        if (idx_ok((int)pk, nen)) cl_st(zk, cl_ld<T>(zk) + cl_ld<T>(en + (uint32_t)sizeof(T) * pk));
                     }
                 __syncthreads();
                 if (lt2.w == 2) {  // (blocks: the colour swept next is read too, so the neighbours
