@@ -354,7 +354,7 @@ size_t outer_scalar_count(int max_iters);
 // algorithmic bytes of one application of B^_0 (Alg. 2 over every level, values of
 // value_bytes bytes; the per-op counts of the cycle's roofline)
 double cycle_application_bytes(amg_hierarchy *h, int value_bytes);
-// host image of h's device level table in the cycle precision fp32 (LevelDev<T, int>[nlev]):
+// host image of h's device level table in the cycle precision fp32 (LevelDev<T>[nlev]):
 // what the level table holds once the level arrays exist; returns its size in bytes
 size_t level_table_image(amg_hierarchy *h, bool fp32, std::vector<unsigned char> &out);
 // the finest level's big blocks and their level-ordered sweep schedules (setup.cu)

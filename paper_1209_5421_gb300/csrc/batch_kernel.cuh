@@ -11,7 +11,7 @@
 namespace amg {
 
 template <class T>
-using BLev = LevelDev<T, int>;
+using BLev = LevelDev<T>;
 
 // levels of a system: the finest and at most 15 auxiliary ones (depth 14 to 0)
 constexpr int kBatchLevels = 16;

@@ -58,18 +58,16 @@ struct Op {
 
 enum : int { V_RHS = 0, V_E, V_R, V_P0 };  // V_P0 + i = p_i
 
-// view of one level; I = column index type;
-// B: what the kernel instance compiles besides the plain rows, each in instances of its own, so
+// view of one level. B: what the kernel instance compiles besides the plain rows, each in instances of its own, so
 // that the registers of the others stay free: kCoop the lane-parallel block smoother of finest
 // levels with multi-row blocks, kBig the sweeps of a graded finest level's big blocks
 // (compiled into every FP32 cycle these made 416 bytes of spill loads a thread instead of 124: a
 // solve of 1,046,529 unknowns 22.7 ms instead of 21.4, the octree of 129^3 nodes 27.7 instead
 // of 25.9)
 constexpr int kCoop = 1, kBig = 2;
-template <class T, class I, int B = 0>
+template <class T, int B = 0>
 struct LevelDev {
     using val_t = T;
-    using idx_t = I;
     static constexpr int coop = B & kCoop;
     static constexpr bool bigs = (B & kBig) != 0;
     int n;
@@ -78,7 +76,7 @@ struct LevelDev {
                                     // 0: one thread per block
     int w;                          // > 0: every slice has width w (sl not read)
     const int *sl;
-    const I *col;
+    const int *col;
     const T *val;
     const T *dinv;                  // 1 / a_ii (smoother)
     const int *bptr;
@@ -96,8 +94,8 @@ struct LevelDev {
 };
 
 // first slot and slot count of row i
-template <class T, class I, int B>
-__device__ __forceinline__ void row_span(const LevelDev<T, I, B> &L, int i, int &base,
+template <class T, int B>
+__device__ __forceinline__ void row_span(const LevelDev<T, B> &L, int i, int &base,
                                          int &width) {
     const int s = i >> 5;
     if (L.w > 0) {
@@ -169,7 +167,7 @@ struct SmallGroup : BlockGroup {
 
 // ---------------------------------------------------------------------------------------
 // reductions: fixed-order trees, no floating-point atomics (bitwise reproducible)
-enum : int { RM_LASTBLOCK = 0, RM_BLOCK = 1, RM_PARTIAL = 2, RM_TEAM = 3 };
+enum : int { RM_LASTBLOCK = 0, RM_PARTIAL = 1, RM_TEAM = 2 };
 
 // GB300 executes FP64 arithmetic at a small fraction of its FP32 rate, so reductions keep
 // FP64 work low: in the FP32 cycle a block sums in FP32 (a warp tree, then one warp over the
@@ -317,9 +315,9 @@ static __device__ __noinline__ void team_reduce_store(const double *r, int nv,
 }
 
 // RM_LASTBLOCK: per-block partial; the last block to finish sums them in block order.
-// RM_BLOCK (one CTA): the block sum. RM_PARTIAL (persistent kernel): per-block partials
-// into buffer pb; the next op sums them. RM_TEAM: LASTBLOCK over the rc.size CTAs of a team
-// (team_reduce_store; a team of one is RM_BLOCK; the group must be the whole CTA). Final
+// RM_PARTIAL (persistent kernel): per-block partials into buffer pb; the next op sums them.
+// RM_TEAM: LASTBLOCK over the rc.size CTAs of a team (team_reduce_store; a team of one stores
+// its block sum; the group must be the whole CTA). Final
 // values are stored by thread 0 into out[k]; they are visible to the team after its next
 // barrier.
 template <int NV, int RM, class A, class G>
@@ -327,7 +325,7 @@ __device__ __forceinline__ void reduce_store(const A (&v)[NV], double *const (&o
                                              const RedCtx &rc, int pb, const G &g) {
     double r[NV];
     block_sum<NV, A>(v, r, g);
-    if (RM == RM_BLOCK || (RM == RM_TEAM && rc.size == 1)) {  // visible after the next barrier
+    if (RM == RM_TEAM && rc.size == 1) {  // visible after the next barrier
         if (threadIdx.x == 0)
 #pragma unroll
             for (int k = 0; k < NV; k++)
@@ -441,14 +439,13 @@ __device__ __forceinline__ typename LV::val_t row_dot(const LV &L, int base, int
                                                       const typename LV::val_t *x,
                                                       typename LV::val_t acc = 0) {
     using T = typename LV::val_t;
-    using I = typename LV::idx_t;
     for (int kb = k0; kb < width; kb += kRowBatch) {
-        I c[kRowBatch];
+        int c[kRowBatch];
         T a[kRowBatch];
 #pragma unroll
         for (int j = 0; j < kRowBatch; j++) {
             const int k = kb + j;
-            c[j] = k < width ? L.col[base + 32 * k] : (I)-1;
+            c[j] = k < width ? L.col[base + 32 * k] : -1;
             a[j] = k < width ? L.val[base + 32 * k] : T(0);
         }
         T xv[kRowBatch];
@@ -469,19 +466,18 @@ template <class LV>
 struct RowAhead {
     int row = -1;                  // the row held, -1: none
     int base = 0, width = 0;
-    typename LV::idx_t c[kRowBatch];
+    int c[kRowBatch];
     typename LV::val_t a[kRowBatch];
 };
 template <class LV>
 __device__ __forceinline__ void row_load(const LV &L, int i, int k0, RowAhead<LV> &p) {
     using T = typename LV::val_t;
-    using I = typename LV::idx_t;
     p.row = i;
     row_span(L, i, p.base, p.width);
 #pragma unroll
     for (int j = 0; j < kRowBatch; j++) {
         const int k = k0 + j;
-        p.c[j] = k < p.width ? L.col[p.base + 32 * k] : (I)-1;
+        p.c[j] = k < p.width ? L.col[p.base + 32 * k] : -1;
         p.a[j] = k < p.width ? L.val[p.base + 32 * k] : T(0);
     }
 }
@@ -553,7 +549,6 @@ template <class LV>
 __device__ void op_gs_blocks_coop(const LV &L, const Op &op, const typename LV::val_t *f,
                                   typename LV::val_t *u, int tid, int nth, bool skip_big) {
     using T = typename LV::val_t;
-    using I = typename LV::idx_t;
     constexpr int G = kBlockLanes;
     const int q = tid & (G - 1);
     const unsigned gmask = 0xFFFFu << ((threadIdx.x & 31) & 16);  // this group's 16 lanes
@@ -585,12 +580,12 @@ __device__ void op_gs_blocks_coop(const LV &L, const Op &op, const typename LV::
             int rb, width;
             row_span(L, i, rb, width);
             for (int kb = 1; kb < width; kb += kRowBatch) {
-                I c[kRowBatch];
+                int c[kRowBatch];
                 T a[kRowBatch];
 #pragma unroll
                 for (int j = 0; j < kRowBatch; j++) {
                     const int kk = kb + j;
-                    c[j] = kk < width ? L.col[rb + 32 * kk] : (I)-1;
+                    c[j] = kk < width ? L.col[rb + 32 * kk] : -1;
                     a[j] = kk < width ? L.val[rb + 32 * kk] : T(0);
                 }
                 T xv[kRowBatch];
@@ -661,7 +656,7 @@ __device__ void prefetch_big_block(const LV &L, const int *lofs, const int *lp, 
     const int e0 = lp[lofs[k]], e1 = lp[lofs[k + 1]];
     prefetch_l2(ent + e0, sizeof(int4) * (size_t)(e1 - e0));
     const int s0 = L.sl[r0 >> 5], s1 = L.sl[((r1 - 1) >> 5) + 1];
-    prefetch_l2(L.col + s0, sizeof(typename LV::idx_t) * (size_t)(s1 - s0));
+    prefetch_l2(L.col + s0, sizeof(int) * (size_t)(s1 - s0));
     prefetch_l2(L.val + s0, sizeof(T) * (size_t)(s1 - s0));
     prefetch_l2(f + r0, sizeof(T) * (size_t)(r1 - r0));
     prefetch_l2(L.dinv + r0, sizeof(T) * (size_t)(r1 - r0));
@@ -761,12 +756,12 @@ __device__ bool big_block_smem(const LV &L, const int *lofs, const int *lp, cons
         T s = f[row];
         int early = 0;
         for (int kb = 1; kb < e.z; kb += kRowBatch) {
-            typename LV::idx_t c[kRowBatch];
+            int c[kRowBatch];
             T a[kRowBatch], x[kRowBatch];
 #pragma unroll
             for (int j = 0; j < kRowBatch; j++) {
                 const int kk = kb + j;
-                c[j] = kk < e.z ? L.col[e.y + 32 * kk] : (typename LV::idx_t)-1;
+                c[j] = kk < e.z ? L.col[e.y + 32 * kk] : -1;
                 a[j] = kk < e.z ? L.val[e.y + 32 * kk] : T(0);
             }
 #pragma unroll
@@ -1289,7 +1284,7 @@ __device__ void op_update(const LV &L, const Op &op, const RedCtx &rc, int tid, 
         double *out[1] = {&L.sc[SC_RR0 + i]};
         reduce_store<1, RM, T>(v, out, rc, op.red_pb, g);
     }
-    if ((RM == RM_BLOCK || (RM == RM_TEAM ? rc.rank == 0 : blockIdx.x == 0)) && threadIdx.x == 0)
+    if ((RM == RM_TEAM ? rc.rank == 0 : blockIdx.x == 0) && threadIdx.x == 0)
         L.sc[SC_STOP0 + i] = stopped ? 1.0 : 0.0;
 }
 

@@ -22,7 +22,7 @@
 namespace amg {
 
 template <class T>
-using GLev = LevelDev<T, int, kBig>;           // level in HBM
+using GLev = LevelDev<T, kBig>;           // level in HBM
 
 // persistent kernel CTA size (one CTA per SM): the FP64 cycle runs with fewer threads and
 // twice the registers each, as its ops at the 64-register cap of 1024 threads spill
@@ -105,7 +105,7 @@ extern __shared__ __align__(16) unsigned char amg_smem[];
 
 template <class T, int B>
 __global__ void __launch_bounds__(cycle_threads<T>(), 1) k_cycle(CycleArgs<T> a) {
-    using GL = LevelDev<T, int, B>;  // the same layout as GLev<T>
+    using GL = LevelDev<T, B>;  // the same layout as GLev<T>
     __shared__ GL gtab[kMaxLevels];
     __shared__ unsigned long long target;
     __shared__ int abort_flag;
@@ -1765,7 +1765,7 @@ void prepare_cycle(amg_hierarchy *h) {
     h->fp32_ready = true;
 }
 
-// device level table of the cycle precision (LevelDev<T, int>[nlev])
+// device level table of the cycle precision (LevelDev<T>[nlev])
 const void *level_table(const amg_hierarchy *h, bool fp32) {
     return fp32 ? h->lev_tab32 : h->lev_tab64;
 }
