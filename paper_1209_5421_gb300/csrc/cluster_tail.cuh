@@ -356,18 +356,15 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
     const uint32_t peer_tok = cl_map(cl_smem(&token), peer), peer_mb = cl_map(mb0, peer);
     long long tp0 = 0;
     const bool mark_on = a.tprof && rank == 0 && tid == 0;
-    // profiling: cycles and count per (level, kind), summed here and added up at the end
-    __shared__ unsigned prof_s[2][16 * (kClLevels + 2)];
-    if (mark_on) {
-        for (int k = 0; k < 2 * 16 * (kClLevels + 2); k++) (&prof_s[0][0])[k] = 0;
-        tp0 = clock64();
-    }
+    // profiling: cycles and count per (level, kind); in global memory, as 1.3 KB of shared memory can
+    // cost a level its place (97^2 nodes, kcycle_n = 4, FP64: 644 -> 1,079 us per application)
+    if (mark_on) tp0 = clock64();
     auto mark = [&](int slot_level, int kind) {
         if (!mark_on) return;
         const long long t1 = clock64();
-        const int slot = 16 * slot_level + kind;
-        prof_s[0][slot] += (unsigned)(t1 - tp0);
-        prof_s[1][slot] += 1;
+        const int slot = 16 * (y.tl + slot_level) + kind;
+        atomicAdd(&a.tprof[slot], (unsigned long long)(t1 - tp0));
+        atomicAdd(&a.tprof[16 * kMaxLevels + slot], 1ull);
         tp0 = t1;
     };
     // this CTA's arrivals at mbarrier mb, which counts its warps and `bytes` of stores (the last
@@ -862,8 +859,9 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
                     if (idx_ok((int)pi[k >> 4], y.nd))
                         cl_store(cl_map(to + (uint32_t)sizeof(T) * pi[k >> 4], k & (NR - 1)), stage[k >> 4],
                                  cl_map(mb, k & (NR - 1)));
-            cl_store_if(alive && warp == kClWarps - 1 && lane < NR, cl_map(cl_smem(&token), lane & (NR - 1)), 0.f,
-                        cl_map(mb, lane & (NR - 1)));
+            if (warp == kClWarps - 1)
+                cl_store_if(alive && lane < NR, cl_map(cl_smem(&token), lane & (NR - 1)), 0.f,
+                            cl_map(mb, lane & (NR - 1)));
             arrive(mb, (int)sizeof(T) * y.nd + 4 * NR);
             wait_a();
             mark(lv, OP_RESTRICT);
@@ -872,7 +870,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
         {
             const int ch = y.ch, len = NR * ch;
             T *E = vec(y.E), *out = vec(y.out), *Rv = vec(y.Rv);
-            const int nsteps = y.dense ? y.kc : 1, parts = y.dense && y.aw == 0 ? 2 : 1;
+            const int nsteps = y.dense ? y.kc : 1, parts = !F64 && y.dense && y.aw == 0 ? 2 : 1;
             constexpr int LPR = 8;  // lanes per row
             constexpr int V = 16 / (int)sizeof(T);
             // FP32: [z; w] = [M; A M] r, 16 lanes per row, 16-byte reads; M r as a compensated sum
@@ -1218,12 +1216,6 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
             for (int k = rank * y.ch + tid; k < min(y.nd, (rank + 1) * y.ch); k += kClThreads) a.e[k] = E[k];
         }
     }
-    if (mark_on)
-        for (int k = 0; k < 16 * (y.nsp + 1); k++)
-            if (prof_s[1][k]) {
-                a.tprof[16 * y.tl + k] += prof_s[0][k];
-                a.tprof[16 * kMaxLevels + 16 * y.tl + k] += prof_s[1][k];
-            }
     cl_sync_all();  // no CTA leaves while a neighbour may still write into it
     if (*gave_up) cl_drain(mb0 + 32);
     if (a.ts && rank == 0 && tid == 0) *a.ts = global_ns();
