@@ -782,7 +782,7 @@ def run_ours(args, world, rank, local):
     kernels = None
     if not args.no_profile:
         h = amg.Hierarchy(*A, **opts)
-        h.profile(2)  # per kernel and per grid op; the shared-memory tail timed as a whole
+        h.profile(2)  # per kernel and per grid op; the cluster's launches timed as wholes
         flush.fill_(0.0)
         torch.cuda.synchronize()
         h.solve(b, args.tol, x=x)

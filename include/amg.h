@@ -406,9 +406,10 @@ int amg_launch_counts(const amg_hierarchy *h, int64_t *setup_launches, int64_t *
  * (kernel kind, level) together with its algorithmic bytes: the bytes of every array it must
  * read or write once at its width (4-byte indices, value width of the cycle precision; no
  * padding). Inside the persistent cycle kernel every op is timed from in-kernel timestamps
- * (each op's time includes the grid barrier that ends it); with enable = 1 the ops of the
- * shared-memory tail are also timed one by one (SM clock cycles, which adds work to the tail),
- * with enable = 2 the tail is timed as a whole. Enabling or disabling resets the totals.
+ * (each op's time includes the grid barrier that ends it); with enable = 1 the steps inside the
+ * cluster that runs the coarse levels are also timed one by one (SM clock cycles, which adds
+ * work to them), with enable = 2 each of its launches is timed as a whole. Enabling or
+ * disabling resets the totals.
  * Measure throughput with profiling off. Errors: AMG_ERR_INVALID_ARG for another value.
  */
 int amg_profile_enable(amg_hierarchy *h, int enable);
@@ -430,10 +431,10 @@ const char *amg_kernel_name(int kind);
  * ------------------------------------------------------------------------------------- */
 
 /*
- * Barrier fault of h's cycle kernel for the following solves (until reset with 0, 0): every
- * grid barrier of the persistent kernel gives up after limit_ns nanoseconds (0 = the default
- * 2 s), and the first barrier of each launch waits for `extra` arrivals more than the grid
- * makes, so that it runs out (0 = none). The solve then returns AMG_ERR_TIMEOUT and leaves h
+ * Barrier fault of h's cycle for the following solves (until reset with 0, 0): every grid
+ * barrier of the persistent kernel and every exchange of the cluster's gives up after limit_ns
+ * nanoseconds (0 = the default 2 s), and the first of each launch waits for `extra` arrivals
+ * (in the cluster: bytes) more than come, so that it runs out (0 = none). The solve then returns AMG_ERR_TIMEOUT and leaves h
  * ready for the next solve. Errors: AMG_ERR_INVALID_ARG for NULL or negative arguments.
  */
 int amg_debug_barrier_fault(amg_hierarchy *h, int64_t limit_ns, int32_t extra);

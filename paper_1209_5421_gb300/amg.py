@@ -397,7 +397,7 @@ class Hierarchy:
         return int(s[0]), int(v[0])
 
     def debug_barrier_fault(self, limit_ns: int = 0, extra: int = 0):
-        """Host-set barrier fault of the cycle kernel for the following solves (0, 0: off)."""
+        """Host-set fault of the cycle's waits for the following solves (0, 0: off)."""
         _check(lib().amg_debug_barrier_fault(self.h, int(limit_ns), int(extra)),
                "amg_debug_barrier_fault")
 
@@ -409,8 +409,8 @@ class Hierarchy:
         return v.value
 
     def profile(self, enable: bool | int = True):
-        """0/False: off; 1/True: per-kernel and per-op timing, tail ops one by one; 2: the
-        same with the shared-memory tail timed as a whole (no per-op work added to it)."""
+        """0/False: off; 1/True: per-kernel and per-op timing, the cluster's steps one by
+        one; 2: the same with each launch of the cluster timed as a whole (no work added to it)."""
         _check(lib().amg_profile_enable(self.h, int(enable)), "amg_profile_enable")
 
     def profile_read(self) -> list[dict]:

@@ -171,9 +171,11 @@ enum : int { RM_LASTBLOCK = 0, RM_PARTIAL = 1, RM_TEAM = 2 };
 
 // GB300 executes FP64 arithmetic at a small fraction of its FP32 rate, so reductions keep
 // FP64 work low: in the FP32 cycle a block sums in FP32 (a warp tree, then one warp over the
-// per-warp sums) and only the sum over CTAs is FP64; FP64 partials go through shared memory
-// and one warp sums them (32 values per lane in fixed order, then a 5-level shuffle tree),
-// about one FP64 add per partial instead of five for a shuffle tree over every warp.
+// per-warp sums), and the sum over CTAs is FP32 too in the persistent kernel (finalize), FP64
+// elsewhere (a few values). FP64 partials go through shared memory and four warps, one per
+// scheduler, share a value's (8 partials per lane in fixed order for 1,024 threads, then a
+// 5-level shuffle tree); one adds the four sums. Where shared memory is scarce (SmallGroup) every
+// warp sums its own partials, all values at once (warp_sums).
 template <int N>
 __device__ __forceinline__ double *red_scratch() {
     __shared__ double s[N];
@@ -386,7 +388,8 @@ __device__ __forceinline__ int ld_volatile_int(const int *p) {
 // loads until the counter reaches (k+1) * gridDim.x for its k-th barrier (the load that sees
 // the last arrival orders every later access after the other CTAs' writes; the CTA's other
 // threads follow through the closing __syncthreads). The counter is zeroed before every
-// launch. Returns false if the kernel must stop.
+// application; a launch starts from the arrivals of those before it. Returns false if the
+// kernel must stop.
 __device__ __forceinline__ unsigned long long ld_acquire_u64(const unsigned long long *p) {
     unsigned long long v;
     asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
@@ -1288,8 +1291,6 @@ __device__ void op_update(const LV &L, const Op &op, const RedCtx &rc, int tid, 
         L.sc[SC_STOP0 + i] = stopped ? 1.0 : 0.0;
 }
 
-// run one op (everything except OP_TAIL / OP_NOP) on level view L by threads tid < nth of
-// group g; next() gives the view of the next coarser level (only its rhs and e are used)
 // A finest colour with big blocks has three kinds of work, each a chain of its own length: the
 // CTA-sized blocks, the warp-sized ones and the small ones (a thread each). Where there is room
 // they run side by side: CTAs [0, nbigc) take a CTA-sized block each and nothing else, in the
@@ -1377,6 +1378,8 @@ __device__ __forceinline__ void run_op_held(const LV &L, const Op &op, const Red
     }
 }
 
+// run one op (everything except OP_TAIL / OP_NOP) on level view L by threads tid < nth of
+// group g; next() gives the view of the next coarser level (only its rhs and e are used)
 template <class LV, int RM, class G, class Next>
 __device__ __forceinline__ void run_op_on(const LV &L, const Next &next, const Op &op,
                                           const RedCtx &rc, int tid, int nth, const G &g,

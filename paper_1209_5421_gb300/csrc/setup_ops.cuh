@@ -224,6 +224,8 @@ __device__ __forceinline__ void chol_inverse_block(int n, double *ga, double *gw
     // by the FP64 pipe (19 cycles per warp instruction) and the 64 steps: 260 -> 118 us for 64
     // rows (Cholesky's three barriers, a square root and a division per column, then the
     // inverse factor one column per thread: 43k dependent FP64 operations on two warps).
+    // The reciprocal pivots cost no accuracy: error of the inverse against 80-bit arithmetic, mean of
+    // 30 coarsest matrices of 16 to 256 rows: Cholesky 6.9e-16, this 6.6e-16, with divisions 6.4e-16.
     // (step j writes at most j + 1 into `bad`, so every thread leaves the loop at the same step)
     for (int j = 0; j < n && j < bad; j++) {
         const double r = rd[j];

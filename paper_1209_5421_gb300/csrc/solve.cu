@@ -4,12 +4,13 @@
 // finest level, flexible CG with full A-orthogonalisation).
 //
 // Execution. One application of the preconditioner B^_fine is a fixed program of ops (see
-// cycle_ops.cuh) over device-resident data; every scalar stays on the device. It runs as ONE
-// persistent cooperative kernel (one CTA per SM): the CTAs execute each op row-parallel and
-// meet at a bounded grid barrier before the next. The coarse levels (pure latency) run in the
-// shared memory of a thread-block cluster (cluster_tail.cuh), a launch of its own between
-// launches of the persistent kernel. The outer Krylov update is four small kernels per
-// iteration; the host reads one residual per iteration.
+// cycle_ops.cuh) over device-resident data; every scalar stays on the device. It runs as a
+// sequence of two kinds of launches. The fine levels' ops between two visits of the coarse levels
+// are one launch of a persistent cooperative kernel (one CTA per SM): the CTAs execute each op
+// row-parallel and meet at a bounded grid barrier before the next. The coarse levels (pure
+// latency) run in the shared memory of a thread-block cluster (cluster_tail.cuh), a launch per
+// visit; of a small quadtree all levels do, and an application is that one launch. The outer
+// Krylov update is four small kernels per iteration; the host reads one residual per iteration.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -36,7 +37,7 @@ constexpr int cycle_threads() { return sizeof(T) == 8 ? kPThreads64 : kPThreads;
 constexpr int kSplitRestrictRows = 524288;
 
 
-constexpr int kTprofCount = 16 * kMaxLevels;  // tail profile slots: 16 op kinds per level
+constexpr int kTprofCount = 16 * kMaxLevels;  // cluster's profile slots: 16 op kinds per level
 
 template <class T>
 struct CycleArgs {
@@ -574,7 +575,7 @@ struct Profiler {
         cudaEvent_t a, b;
     };
     bool on = false;
-    bool tail_ops = false;  // also time every op inside the shared-memory tail
+    bool tail_ops = false;  // also time every step inside the cluster
     std::vector<Rec> pending;
     struct Acc {
         int64_t launches = 0;
@@ -735,8 +736,8 @@ bool is_reduction(const Op &op) {
 }
 
 // Walks Alg. 2 / Alg. 1 from a level and appends the ops to a program. The recursion stops
-// at `stop_level`, where one OP_TAIL stands for B~ of that level (persistent program), or
-// continues to the coarsest level (tail program, standalone execution).
+// at `stop_level`, where one OP_TAIL stands for B~ of that level (the cycle's program), or
+// continues to the coarsest level (traffic accounting, standalone execution).
 struct Builder {
     amg_hierarchy *h;
     std::vector<Op> *out;
@@ -1048,8 +1049,8 @@ int2 cl_own_rows(const ClSrc &S, const std::vector<int> &hb, int r, int c) {
 // the dense level; sparse: M alone and the sparse A after it.
 template <class T>
 bool cluster_plan(const ClSrcs &G, const std::vector<int2> &win, const std::vector<int> &xchild, int nlv,
-                  const int *fo, const std::vector<int> &hb, const std::vector<int> &widths, int s0, int level0, bool dense, bool sparse, int nch,
-                  const amg_options &opt, long budget, ClPlan &P) {
+                  const int *fo, const std::vector<int> &hb, const std::vector<int> &widths, int s0, int level0,
+                  bool dense, bool sparse, int nch, const amg_options &opt, long budget, ClPlan &P) {
     constexpr int vb = (int)sizeof(T), NR = kClRanks;
     ClLayout &y = P.y;
     std::memset(&y, 0, sizeof y);
@@ -1709,7 +1710,7 @@ void harvest_cycle_timestamps(amg_hierarchy *h) {
                        : (op.kind == OP_NOP) ? 0.0 : op_bytes(h, op, sizeof(T));
         h->prof->add(K_IN_CYCLE + op.kind, op.level, ms, bytes);
     }
-    // inside the tail: SM cycles per op kind and level, reported at the nominal clock
+    // inside the cluster: SM cycles per op kind and level, reported at the nominal clock
     std::vector<unsigned long long> tp(2 * kTprofCount);
     AMG_CUDA(cudaMemcpy(tp.data(), E->tprof, sizeof(unsigned long long) * tp.size(),
                         cudaMemcpyDeviceToHost));
@@ -1885,14 +1886,14 @@ static GLev<double> fine_view(amg_hierarchy *h) {
     return L;
 }
 
-// the cycle kernel's error flag, read by the caller
+// the error flag of the cycle's kernels, read by the caller
 static void raise_device_error(amg_hierarchy *h, int err) {
     if (err & kErrTimeout) {
-        // the kernel left its op loop: clear the flag and the barrier state for the next launch
+        // the kernels ended early: clear the flag and the barrier state for the next launch
         AMG_CUDA(cudaMemsetAsync(h->err_flag, 0, sizeof(int), h->stream));
         AMG_CUDA(cudaMemsetAsync(h->bar, 0, sizeof(unsigned long long), h->stream));
         AMG_CUDA(cudaStreamSynchronize(h->stream));
-        throw Error{AMG_ERR_TIMEOUT, "a grid barrier of the cycle kernel timed out"};
+        throw Error{AMG_ERR_TIMEOUT, "a wait inside the cycle (grid barrier or cluster exchange) timed out"};
     }
 }
 
