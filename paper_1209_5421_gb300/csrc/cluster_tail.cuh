@@ -45,13 +45,13 @@
 // their rows, and one product with a residual gives p and A p of an Alg. 1 step; that replaces
 // about 13 dependent steps. In FP32 M takes the coarsest inverse's place and is held like it, as a
 // sum of two floats with a compensated product, so p is rounded once; A M is one float with a plain
-// sum, as A itself is where a level is swept (its error, of the order of eps |A M| |r|, is below
-// the eps |A| |p| of a product with A, which also bounds A p - q for the rounded p). FP64
-// keeps M alone and multiplies by the sparse A after it (256 rows: a product with both is 4,900
-// cycles of the FP64 pipe, with M 2,450 and one more gather 600: 9.7 -> 8.8 us per visit). So does
-// FP32 where M's two parts fit but not A M beside them (512 rows); A's few rows per CTA are then read
-// through L1. Where M does not fit, the level is swept like the others and the coarsest solve is
-// the dense product.
+// sum, as A itself is where a level is swept: its error against 64 bits is 5e-8 to 1e-7, of a
+// product of A with the rounded p 1.3e-7 to 1.6e-6 (squares, disks, graded, cubes; random and smooth
+// r), as |A M| |r| is 0.03 to 0.7 of |A| |p|. FP64 keeps M alone and multiplies by the sparse A
+// after it (256 rows: a product with both is 4,900 cycles of the FP64 pipe, with M 2,450 and one
+// more gather 600: 9.7 -> 8.8 us per visit, 9.1 with beta rounded once). So does FP32 where M's two
+// parts fit but not A M beside them (512 rows); A's few rows per CTA are then read through L1. Where
+// M does not fit, the level is swept like the others and the coarsest solve is the dense product.
 #pragma once
 
 #include <cstddef>
@@ -294,7 +294,7 @@ __device__ __noinline__ double cl_quotient(double a, double b) { return a / b; }
 // colour, exchange included: 0.59-0.80 us with each step's code in line and no read ahead,
 // 1.1-1.5 us as an interpreter of ops with all bodies in one loop, 0.40 us in this form
 // (FP64: 0.91-0.98 -> 0.63-0.75 us). All levels from 16,384 rows down, 2 Alg. 1 steps each,
-// 1.05M unknowns, FP32: 118 us per visit (8 per application); on one CTA the levels from
+// 1.05M unknowns, FP32: 127 us per visit (8 per application); on one CTA the levels from
 // 4,096 rows down took 139-150 us (16 per application) and the level above 3.0 us per step.
 extern __shared__ __align__(16) unsigned char cl_dyn[];
 
@@ -703,7 +703,7 @@ k_cluster_tail(const __grid_constant__ ClArgs<T> a) {
     // a sum of two doubles (error of about 2^-106): zq / pq is then a product and an FMA, rounded
     // once but for 2^-53 of a rounding. Only where neither part leaves the normal range (pq of 2^-960
     // to 2^960); elsewhere (0 here) a division. Every beta by a division, 257^2 nodes: 6.13 -> 6.22 ms
-    // per solve; in this form 6.16 (by 1 / pq alone, rounded twice and infinite for a subnormal
+    // per solve; in this form 6.19 (by 1 / pq alone, rounded twice and infinite for a subnormal
     // pq, 6.13).
     auto keep_pq = [&](int lv, int i, T pq) {
         if (tid != (F64 ? 32 : 0)) return;
