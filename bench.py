@@ -145,8 +145,8 @@ def kernel_source_hash():
 
 
 def recorded_traffic(workload, prec):
-    """DRAM bytes per launch of the cycle kernel (or of the batch kernel: one launch is a
-    whole batch solve) from the committed ncu summary, if it was taken on the current kernel
+    """DRAM bytes per application of the cycle (all its launches; or of the batch kernel: one
+    launch is a whole batch solve) from the committed ncu summary, if it was taken on the current kernel
     sources (else None)."""
     p = os.path.join(ROOT, "profiles", "cycle_traffic.json")
     try:
