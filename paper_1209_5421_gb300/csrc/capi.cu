@@ -685,7 +685,9 @@ int amg_debug_barrier_fault(amg_hierarchy *h, int64_t limit_ns, int32_t extra) {
     if (!h) return fail(AMG_ERR_INVALID_ARG, "NULL hierarchy");
     if (limit_ns < 0 || extra < 0) return fail(AMG_ERR_INVALID_ARG, "negative limit or arrivals");
     h->dbg_bar_limit_ns = limit_ns;
-    h->dbg_bar_extra = extra;
+    // (in the cluster these are bytes an mbarrier expects, whose count ends at 2^20 - 1 with the
+    // up to 232,448 of an exchange; any number that never comes is the same fault)
+    h->dbg_bar_extra = std::min(extra, 65536);
     return AMG_OK;
 }
 
